@@ -252,7 +252,8 @@ int slimwise_moe_decode_shared_ex(const void *hidden, const float *router_w,
  * output y (before gating), adds to the caller's fp64 [E, 4] device buffer:
  *   stats[e][0] += 1,  stats[e][1] += g,  stats[e][2] += ||y||_2,
  *   stats[e][3] += g * ||y||_2
- * Tokens are taken in order for each expert.  The buffer is caller-owned and
+ * Each expert's tokens are summed in fp64 in one fixed order (the same for
+ * every run).  The buffer is caller-owned and
  * accumulates across calls (zero it before the first batch).  Other
  * arguments as slimwise_moe_decode_full; stats must be 8-byte aligned.
  */
