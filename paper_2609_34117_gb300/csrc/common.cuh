@@ -53,6 +53,14 @@ __host__ __device__ inline int token_chunk_for(int B, int k, int m_ret) {
   if (c < kTokBox) c = kTokBox;
   return c < most ? c : most;
 }
+// Tokens per entry of an expert with n tokens: as few entries as chunks of at
+// most `chunk` tokens need, their sizes even in units of 16 (257 tokens in
+// chunks of 256 are 144 + 113, not 256 + 1), since every entry streams the
+// expert's weights and takes time with its padded token count.
+__host__ __device__ inline int entry_tokens(int n, int chunk) {
+  const int parts = (n + chunk - 1) / chunk;
+  return parts > 1 ? round16((n + parts - 1) / parts) : chunk;
+}
 // Index m of the token box (kTokBox * (m + 1) rows) that covers n16 16-row groups.
 __host__ __device__ inline int token_box_for(int n16) { return n16 - 1; }
 constexpr int kMinTokChunk = 16;     // smallest token_chunk_for(): bounds the entry count

@@ -31,6 +31,8 @@ namespace slimwise {
 // B = 512: 2 us slower); four per CTA was slower at every size.
 inline int group_tokens_per_cta(int B) { return B <= 64 ? 1 : 2; }
 constexpr int kGroupThreads = 512;
+// Batches from here on take the tiled kernels below.
+constexpr int kGroupTiledMin = 768;
 
 // Exclusive scan of vals[0..n) (n <= kMaxExperts) into outp[0..n], by one
 // warp; returns the total.  Each lane scans a contiguous run.
@@ -47,12 +49,75 @@ __device__ int warp_exclusive_scan(const int *vals, int *outp, int n, int lane) 
   }
   int run = incl - local;
   for (int i = lo; i < hi; ++i) {
+    const int v = vals[i];  // outp may be vals
     outp[i] = run;
-    run += vals[i];
+    run += v;
   }
   const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
   if (lane == 0) outp[n] = total;
   return total;
+}
+
+// Sigmoid gate of the shared expert for token t, by one warp: lane l
+// accumulates elements 128c + 4l + q (c, q ascending) with fused
+// multiply-adds, then an xor butterfly over the lanes.
+__device__ __forceinline__ void shared_gate_token(const __nv_bfloat16 *__restrict__ hidden,
+                                                  const float *__restrict__ w_sg, const Dims &d,
+                                                  const Ws &ws, int t, int lane) {
+  const __nv_bfloat16 *xr = hidden + (size_t)t * d.H;
+  float p = 0.0f;
+  for (int c = 0; c < d.H / 128; ++c) {
+    const int h = 128 * c + 4 * lane;
+    const uint2 xv = *reinterpret_cast<const uint2 *>(xr + h);
+    const float4 wv = *reinterpret_cast<const float4 *>(w_sg + h);
+    p = fmaf(__uint_as_float(xv.x << 16), wv.x, p);
+    p = fmaf(__uint_as_float(xv.x & 0xFFFF0000u), wv.y, p);
+    p = fmaf(__uint_as_float(xv.y << 16), wv.z, p);
+    p = fmaf(__uint_as_float(xv.y & 0xFFFF0000u), wv.w, p);
+  }
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) p = p + __shfl_xor_sync(0xFFFFFFFFu, p, off);
+  if (lane == 0) ws.shared_gate[t] = 1.0f / (1.0f + expf(-p));
+}
+
+// The batch-wide results and the FFN work list, each expert written by one of
+// the grid's gstride threads.  cnt[e] selections, offs/flag_scan/entry_base
+// the exclusive scans (with totals at [E]) of the counts, of the union flags
+// and of the work-entry counts.  Entries [0, S) are the shared expert's
+// (expert -1, token order); the routed ones follow.
+__device__ __forceinline__ void publish_groups(const Dims &d, const Ws &ws, const int *cnt,
+                                               const int *offs, const int *flag_scan,
+                                               const int *entry_base, int gtid, int gstride) {
+  const int E = d.E, B = d.B;
+  const int U = flag_scan[E];
+  const int n_entries = entry_base[E];
+  const int n_se = d.S;
+  for (int e = gtid; e < E; e += gstride) {
+    const int n_e = cnt[e];
+    ws.counts[e] = n_e;
+    ws.offsets[e] = offs[e];
+    if (n_e > 0) ws.union_ids[flag_scan[e]] = e;
+    if (e >= U) ws.union_ids[e] = -1;
+    const int per = entry_tokens(n_e, d.tok_chunk);
+    for (int c = 0; c < entry_base[e + 1] - entry_base[e]; ++c) {
+      const int base = c * per;
+      ws.entries[n_se + entry_base[e] + c] = make_int4(e, offs[e] + base, min(per, n_e - base), 0);
+    }
+  }
+  for (int sidx = gtid; sidx < n_se; sidx += gstride)
+    ws.entries[sidx] = make_int4(-1, sidx * d.tok_chunk, min(d.tok_chunk, B - sidx * d.tok_chunk), 0);
+  for (int i = gtid; i < n_se + n_entries; i += gstride) ws.entry_done[i] = 0;
+  if (gtid == 0) {
+    const int t1_items = gate_up_tiles(d);
+    const int t2_items = down_tiles(d);
+    const int t1s_items = d.Is / kGateRows;
+    ws.offsets[E] = offs[E];
+    ws.ctrl[kCtrlUnionSize] = U;
+    ws.ctrl[kCtrlNumEntries] = n_se + n_entries;
+    ws.ctrl[kCtrlItems1] = n_entries * t1_items;
+    ws.ctrl[kCtrlTotalItems] = n_se * (t1s_items + t2_items) + n_entries * (t1_items + t2_items);
+    ws.ctrl[kCtrlWorkCounter] = 0;
+  }
 }
 
 template <int kGroupTokens>
@@ -197,59 +262,11 @@ __global__ void __launch_bounds__(kGroupThreads)
       }
     }
   }
-  // shared-expert gate of this CTA's tokens: warp w takes token t0 + w; lane
-  // l accumulates elements 128c + 4l + q (c, q ascending) with fused
-  // multiply-adds, then an xor butterfly over the lanes
-  if (d.Is > 0 && warp < nt) {
-    const __nv_bfloat16 *xr = hidden + (size_t)(t0 + warp) * H;
-    float p = 0.0f;
-    for (int c = 0; c < H / 128; ++c) {
-      const int h = 128 * c + 4 * lane;
-      const uint2 xv = *reinterpret_cast<const uint2 *>(xr + h);
-      const float4 wv = *reinterpret_cast<const float4 *>(w_sg + h);
-      p = fmaf(__uint_as_float(xv.x << 16), wv.x, p);
-      p = fmaf(__uint_as_float(xv.x & 0xFFFF0000u), wv.y, p);
-      p = fmaf(__uint_as_float(xv.y << 16), wv.z, p);
-      p = fmaf(__uint_as_float(xv.y & 0xFFFF0000u), wv.w, p);
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) p = p + __shfl_xor_sync(0xFFFFFFFFu, p, off);
-    if (lane == 0) ws.shared_gate[t0 + warp] = 1.0f / (1.0f + expf(-p));
-  }
+  // shared-expert gate of this CTA's tokens: warp w takes token t0 + w
+  if (d.Is > 0 && warp < nt) shared_gate_token(hidden, w_sg, d, ws, t0 + warp, lane);
 
-  // The batch-wide results and the FFN work list, each expert written by one
-  // thread of the grid.  Entries [0, n_se) are the shared expert's (expert
-  // -1, token order); the routed ones follow.
-  const int U = flag_scan[E];
-  const int n_entries = entry_base[E];
-  const int n_se = d.S;
-  const int gtid = blockIdx.x * blockDim.x + tid, gstride = gridDim.x * blockDim.x;
-  for (int e = gtid; e < E; e += gstride) {
-    ws.counts[e] = cnt_all[e];
-    ws.offsets[e] = offs[e];
-    if (union_flag[e]) ws.union_ids[flag_scan[e]] = e;
-    if (e >= U) ws.union_ids[e] = -1;
-    const int n_e = offs[e + 1] - offs[e];
-    for (int c = 0; c < chunk_cnt[e]; ++c) {
-      const int base = c * d.tok_chunk;
-      ws.entries[n_se + entry_base[e] + c] =
-          make_int4(e, offs[e] + base, min(d.tok_chunk, n_e - base), 0);
-    }
-  }
-  for (int sidx = gtid; sidx < n_se; sidx += gstride)
-    ws.entries[sidx] = make_int4(-1, sidx * d.tok_chunk, min(d.tok_chunk, B - sidx * d.tok_chunk), 0);
-  for (int i = gtid; i < n_se + n_entries; i += gstride) ws.entry_done[i] = 0;
-  if (blockIdx.x == 0 && tid == 0) {
-    const int t1_items = gate_up_tiles(d);
-    const int t2_items = down_tiles(d);
-    const int t1s_items = d.Is / kGateRows;
-    ws.offsets[E] = offs[E];
-    ws.ctrl[kCtrlUnionSize] = U;
-    ws.ctrl[kCtrlNumEntries] = n_se + n_entries;
-    ws.ctrl[kCtrlItems1] = n_entries * t1_items;
-    ws.ctrl[kCtrlTotalItems] = n_se * (t1s_items + t2_items) + n_entries * (t1_items + t2_items);
-    ws.ctrl[kCtrlWorkCounter] = 0;
-  }
+  publish_groups(d, ws, cnt_all, offs, flag_scan, entry_base, blockIdx.x * blockDim.x + tid,
+                 gridDim.x * blockDim.x);
   __syncthreads();
   if (blockIdx.x == 0 && tid == 0 && bad) atomicOr(&ws.ctrl[kCtrlErr], bad);
 #ifdef SLIMWISE_TRACE
@@ -257,8 +274,235 @@ __global__ void __launch_bounds__(kGroupThreads)
 #endif
 }
 
+// --------------------------------------------------------------------------
+// Large batches
+// --------------------------------------------------------------------------
+// The kernel above recounts the whole batch in every CTA, work that grows with
+// B^2: 42 us at B = 2048 and 312 us at B = 8192 (Qwen3.6-shaped layer).  From
+// kGroupTiledMin tokens on, two kernels do the same with work linear in B:
+//   group_count_kernel  the histogram of each tile of the batch (at most
+//                       kGroupTiles tiles of 128 tokens or a multiple), one
+//                       CTA per tile;
+//   group_place_kernel  a CTA per part of a tile sums the tiles' histograms
+//                       (a few hundred KB from L2) into the experts' offsets
+//                       and its tile's base in each expert, ranks the tile's
+//                       slots by expert with one bit mask per (expert, 32
+//                       tokens), and copies its part's hidden rows out.
+// The copy (B k H bf16 written) is then what bounds the stage.
+constexpr int kGroupTiles = 64;       // most tiles of the batch
+constexpr int kGroupTile = 128;       // tokens ranked together
+constexpr int kTileWords = kGroupTile / 32;
+
+// Blocks of 128 tokens per tile, and tiles of the batch.
+__host__ __device__ inline int group_tile_blocks(int B) {
+  return (B + kGroupTile * kGroupTiles - 1) / (kGroupTile * kGroupTiles);
+}
+__host__ __device__ inline int group_tile_count(int B) {
+  const int tile = kGroupTile * group_tile_blocks(B);
+  return (B + tile - 1) / tile;
+}
+
+__device__ __forceinline__ int checked_id(int e, int E, int *bad) {
+  if (e < 0 || e >= E) {  // only possible for caller-given selections
+    *bad = SLIMWISE_DEVERR_BAD_TOPK;
+    e = min(max(e, 0), E - 1);
+  }
+  return e;
+}
+
+// tile_cnt[tile][e]: selections of expert e by the tile's tokens.
+__global__ void __launch_bounds__(kGroupThreads)
+    group_count_kernel(Dims d, Ws ws, int32_t *__restrict__ tile_cnt) {
+  __shared__ int cnt[kMaxExperts];
+  __shared__ int bad;
+  for (int e = threadIdx.x; e < d.E; e += blockDim.x) cnt[e] = 0;
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+  pdl_wait_primary();
+  pdl_launch_dependents();
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && threadIdx.x == 0)
+    trace_stamp(ws, ws.ctrl[kCtrlTraceStep] - 1, kTrGroupStart);
+#endif
+  const int tile = kGroupTile * group_tile_blocks(d.B);
+  const int s0 = blockIdx.x * tile * d.k, s1 = min(d.B, (int)(blockIdx.x + 1) * tile) * d.k;
+  for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x)
+    atomicAdd(&cnt[checked_id(ws.topk_idx[s], d.E, &bad)], 1);
+  __syncthreads();
+  for (int e = threadIdx.x; e < d.E; e += blockDim.x)
+    tile_cnt[(size_t)blockIdx.x * d.E + e] = cnt[e];
+  if (threadIdx.x == 0 && bad) atomicOr(&ws.ctrl[kCtrlErr], bad);
+}
+
+// blockIdx.x = tile, blockIdx.y = part: tokens [y part, (y + 1) part) of every
+// 128-token block of the tile.  Dynamic shared memory: see place_smem_bytes.
+__global__ void __launch_bounds__(kGroupThreads)
+    group_place_kernel(const __nv_bfloat16 *__restrict__ hidden, const float *__restrict__ w_sg,
+                       Dims d, Ws ws, const int32_t *__restrict__ tile_cnt, int part,
+                       int do_gather) {
+  extern __shared__ int gsm[];
+  const int B = d.B, k = d.k, E = d.E, H = d.H;
+  int *total = gsm;                    // [E] selections in the batch
+  int *base = total + E;               // [E] next grouped position of this tile
+  int *offs = base + E;                // [E + 1]
+  int *flag = offs + E + 1;            // [E + 1] union flags, then their scan
+  int *chunks = flag + E + 1;          // [E + 1] entries, then their scan
+  uint32_t *mask = reinterpret_cast<uint32_t *>(chunks + E + 1);  // [E][kTileWords]
+  int *pos_s = reinterpret_cast<int *>(mask + (size_t)E * kTileWords);  // [part][k]
+
+  pdl_wait_primary();
+  pdl_launch_dependents();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = gridDim.x;
+  const int blocks = group_tile_blocks(B);
+  const int vecs = H / 8;
+
+  for (int e = tid; e < E; e += blockDim.x) {
+    int before = 0, all = 0;
+    constexpr int kBatch = 16;
+    for (int c0 = 0; c0 < T; c0 += kBatch) {
+      int v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        v[u] = c0 + u < T ? __ldcg(tile_cnt + (size_t)(c0 + u) * E + e) : 0;
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        all += v[u];
+        if (c0 + u < (int)blockIdx.x) before += v[u];
+      }
+    }
+    total[e] = all;
+    base[e] = before;
+    flag[e] = all > 0 ? 1 : 0;
+    chunks[e] = (all + d.tok_chunk - 1) / d.tok_chunk;
+  }
+  __syncthreads();
+  if (warp == 0) warp_exclusive_scan(total, offs, E, lane);
+  if (warp == 1) warp_exclusive_scan(flag, flag, E, lane);
+  if (warp == 2) warp_exclusive_scan(chunks, chunks, E, lane);
+  __syncthreads();
+  for (int e = tid; e < E; e += blockDim.x) base[e] += offs[e];
+
+  for (int b = 0; b < blocks; ++b) {
+    const int t0 = ((int)blockIdx.x * blocks + b) * kGroupTile;
+    if (t0 >= B) break;
+    const int nt = min(kGroupTile, B - t0);
+    for (int i = tid; i < E * kTileWords; i += blockDim.x) mask[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < nt * k; i += blockDim.x) {
+      const int e = min(max(ws.topk_idx[(size_t)t0 * k + i], 0), E - 1);
+      const int t = i / k;
+      atomicOr(&mask[e * kTileWords + (t >> 5)], 1u << (t & 31));
+    }
+    __syncthreads();
+    // this part's tokens [p0, p1) of the block
+    const int p0 = (int)blockIdx.y * part, p1 = min(nt, p0 + part);
+    for (int i = tid; i < (p1 - p0) * k; i += blockDim.x) {
+      const int t = p0 + i / k;
+      const int s = (t0 + p0) * k + i;
+      const int e = min(max(ws.topk_idx[s], 0), E - 1);
+      int p = base[e];
+#pragma unroll
+      for (int w = 0; w < kTileWords; ++w) {
+        const uint32_t m = mask[e * kTileWords + w];
+        if (w < (t >> 5)) p += __popc(m);
+        else if (w == (t >> 5)) p += __popc(m & ((1u << (t & 31)) - 1u));
+      }
+      pos_s[i] = p;
+      ws.pos[s] = p;
+      ws.perm[p] = s;
+    }
+    __syncthreads();
+    if (do_gather) {
+      // each hidden row of the part to its k grouped positions (and, for the
+      // shared expert, to its token-order copy): a warp takes 128 vectors of
+      // a row, its four loads issued before the stores
+      constexpr int kVec = 4;
+      const int groups = (vecs + 32 * kVec - 1) / (32 * kVec);
+      for (int g = warp; g < (p1 - p0) * groups; g += kGroupThreads / 32) {
+        const int tt = g / groups, v0 = (g - tt * groups) * 32 * kVec + lane;
+        const uint4 *src = reinterpret_cast<const uint4 *>(hidden + (size_t)(t0 + p0 + tt) * H);
+        uint4 v[kVec];
+#pragma unroll
+        for (int u = 0; u < kVec; ++u)
+          if (v0 + 32 * u < vecs) v[u] = __ldg(src + v0 + 32 * u);
+        for (int j = 0; j < k; ++j) {
+          uint4 *dst = reinterpret_cast<uint4 *>(ws.xp + (size_t)pos_s[tt * k + j] * H);
+#pragma unroll
+          for (int u = 0; u < kVec; ++u)
+            if (v0 + 32 * u < vecs) dst[v0 + 32 * u] = v[u];
+        }
+        if (d.Is > 0) {
+          uint4 *dst = reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + p0 + tt) * H);
+#pragma unroll
+          for (int u = 0; u < kVec; ++u)
+            if (v0 + 32 * u < vecs) dst[v0 + 32 * u] = v[u];
+        }
+      }
+      if (d.Is > 0)
+        for (int tt = warp; tt < p1 - p0; tt += kGroupThreads / 32)
+          shared_gate_token(hidden, w_sg, d, ws, t0 + p0 + tt, lane);
+    }
+    __syncthreads();
+    // the tile's next block continues after this one
+    if (b + 1 < blocks) {
+      for (int e = tid; e < E; e += blockDim.x) {
+        int n = 0;
+#pragma unroll
+        for (int w = 0; w < kTileWords; ++w) n += __popc(mask[e * kTileWords + w]);
+        base[e] += n;
+      }
+      __syncthreads();
+    }
+  }
+
+  const int gtid = ((int)blockIdx.y * T + (int)blockIdx.x) * blockDim.x + tid;
+  publish_groups(d, ws, total, offs, flag, chunks, gtid, (int)(gridDim.x * gridDim.y * blockDim.x));
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0)
+    trace_stamp(ws, ws.ctrl[kCtrlTraceStep] - 1, kTrGroupEnd);
+#endif
+}
+
+// Tokens of a block per CTA of group_place_kernel: enough CTAs for the GPU at
+// the smallest batches, fewer recounts of the tile at the largest.
+inline int group_part_tokens(int B) { return B <= 1024 ? 4 : B <= 4096 ? 8 : 16; }
+
+size_t place_smem_bytes(const Dims &d, int part) {
+  return (size_t)(5 * d.E + 3 + d.E * kTileWords + part * d.k) * 4;
+}
+
+cudaError_t launch_group_tiled(const __nv_bfloat16 *hidden, const float *w_shared_gate, Dims d,
+                               Ws ws, bool pdl, bool gather, cudaStream_t stream) {
+  // the tiles' histograms go where the call's expert outputs will be:
+  // E / 32 bytes a token at most against k H bf16
+  int32_t *tile_cnt = reinterpret_cast<int32_t *>(ws.y);
+  const int tiles = group_tile_count(d.B), part = group_part_tokens(d.B);
+  const size_t smem = place_smem_bytes(d, part);
+  cudaError_t err = cudaFuncSetAttribute(group_place_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kGroupThreads);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.gridDim = dim3(tiles);
+  err = cudaLaunchKernelEx(&cfg, group_count_kernel, d, ws, tile_cnt);
+  if (err != cudaSuccess) return err;
+  cfg.gridDim = dim3(tiles, kGroupTile / part);
+  cfg.dynamicSmemBytes = smem;
+  return cudaLaunchKernelEx(&cfg, group_place_kernel, hidden, w_shared_gate, d, ws,
+                            (const int32_t *)tile_cnt, part, gather ? 1 : 0);
+}
+
 cudaError_t launch_group_gather(const __nv_bfloat16 *hidden, const float *w_shared_gate,
                                 Dims d, Ws ws, bool pdl, bool gather, cudaStream_t stream) {
+  if (d.B >= kGroupTiledMin)
+    return launch_group_tiled(hidden, w_shared_gate, d, ws, pdl, gather, stream);
   cudaLaunchConfig_t cfg = {};
   const int tpc = group_tokens_per_cta(d.B);
   cfg.gridDim = dim3((d.B + tpc - 1) / tpc);

@@ -1,0 +1,72 @@
+"""Large batches (prompt chunks, calibration batches) against the oracle: the
+tiled grouping kernels at the edges of their range and of their tiles, and
+whole layers whose experts take several work entries."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_34117_gb300 as sw
+from paper_2609_34117_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    sw.build.build()
+    oracle.build()
+
+
+# 768 tokens is where the tiled kernels start; tiles are 128 tokens up to
+# 8192 of them, then 256 (8193: one token in the last tile's first block)
+@pytest.mark.parametrize("B,E,k", [(767, 16, 2), (768, 16, 2), (769, 128, 8), (1025, 1024, 32),
+                                   (4097, 256, 8), (8192, 128, 8), (8193, 16, 1),
+                                   (20000, 100, 4)])
+def test_group_large_batches(B, E, k):
+    rng = np.random.default_rng(B)
+    sel = np.argsort(rng.random((B, E)) * np.linspace(0.2, 1.0, E), axis=1)[:, :k].astype(np.int32)
+    g = sw.slimwise_moe_group(torch.from_numpy(sel).to(DEV), E)
+    ref = oracle.group_by_expert(sel, E)
+    U = ref["union_size"]
+    assert int(g["union_size"].item()) == U
+    for name in ("counts", "offsets", "perm", "pos"):
+        assert np.array_equal(g[name].cpu().numpy(), ref[name]), name
+    ids = g["union_ids"].cpu().numpy()
+    assert np.array_equal(ids[:U], ref["union_ids"]) and np.all(ids[U:] == -1)
+
+
+def _check(got, ref):
+    got = got.float().cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 1e-2 * np.linalg.norm(ref)
+    assert np.abs(got - ref).max() <= 3e-2
+
+
+# grouped rows of a ragged hidden width; experts of several entries with an
+# odd remainder, one of them selected by every token; the shared expert
+@pytest.mark.parametrize("H,E,I,k,B,shared", [(640, 24, 192, 3, 777, 0), (256, 16, 128, 2, 1031, 0),
+                                              (256, 16, 128, 2, 1500, 128), (512, 8, 128, 4, 2051, 0)])
+def test_layer_large_batches(H, E, I, k, B, shared):
+    shape = synth.LayerShape(hidden=H, num_experts=E, inter=I, top_k=k)
+    w_gu, w_d = synth.expert_weights(shape, 1)
+    wr = synth.router_weight(shape, 1)
+    bias = torch.zeros(E)
+    bias[E // 2] = 20.0
+    x, wr = synth.apply_popularity_bias(synth.hidden_states(B, shape, 2), wr, bias)
+    args = [t.to(DEV) for t in (x, wr)] + [None] + [t.to(DEV) for t in (w_gu, w_d)] + [k]
+    host = [synth.bf16_bits(x), wr.numpy(), None, synth.bf16_bits(w_gu), synth.bf16_bits(w_d), k]
+    toks = np.sort(np.random.default_rng(B).choice(B, size=200, replace=False)).astype(np.int32)
+    if shared:
+        w_sg, gu, dn = synth.shared_expert(H, shared, 3)
+        out = sw.slimwise_moe_decode_shared(*args, w_sg.to(DEV), gu.to(DEV), dn.to(DEV))
+        ref = oracle.moe_decode_shared(*host, w_sg.numpy(), synth.bf16_bits(gu), synth.bf16_bits(dn), toks)
+    else:
+        out = sw.slimwise_moe_decode_full(args[0], args[1], *args[3:])
+        ref = oracle.moe_decode_sampled(*host, toks)
+    _check(out[toks], ref["out"])
+    r = sw.slimwise_moe_route(args[0], args[1], None, k, E)
+    assert np.array_equal(r["topk_idx"].cpu().numpy(), ref["idx"])
