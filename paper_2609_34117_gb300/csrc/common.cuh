@@ -20,6 +20,8 @@ namespace slimwise {
 constexpr int kBlockK = 64;          // K elements per pipeline stage (128 B of bf16)
 constexpr int kTileRows = 128;       // MMA M: weight rows per work item
 constexpr int kGateRows = 64;        // gate rows (and as many up rows) per gate/up item
+constexpr int kUnitRows = 16;        // rows of a weight unit: 8 gate + 8 up, or 16 down
+constexpr int kTileUnits = kTileRows / kUnitRows;
 constexpr int kMaxTokTile = 256;     // MMA N limit: tokens of one expert per item
 constexpr int kTokBox = 16;          // token rows per MMA N step
 constexpr int kTokBoxSizes = 16;     // token-row TMA boxes of kTokBox * (m + 1) rows, m < 16
@@ -245,15 +247,19 @@ cudaError_t launch_group_gather(const __nv_bfloat16 *hidden, const float *w_shar
                                 Dims d, Ws ws, bool pdl, bool gather, cudaStream_t stream);
 
 struct FfnMaps {
-  CUtensorMap w_gu;                 // [E*2I rows, H cols] bf16, box 64 x 64
-  CUtensorMap w_down;               // [E*H rows, I cols] bf16, box 64 x 64
+  // Weights, 5-D {K columns, 8 rows, 2, units, experts}, box {64, 8, 2, 4, 1}:
+  // a unit is 16 rows of a weight tile, 8 gate rows and the 8 matching up
+  // rows of W_gu, or 16 consecutive rows of W_down; a box is 4 units, half a
+  // 128-row tile.
+  CUtensorMap w_gu;                 // [E, 2I, H] bf16
+  CUtensorMap w_down;               // [E, H, I] bf16
   // token rows: box 64 x 16 (m + 1), or 64 x 8 (m + 1) for pair items (each
   // CTA of the pair loads half of an item's rows)
   CUtensorMap xp[kTokBoxSizes];     // [B*k rows, H cols] bf16
   CUtensorMap act[kTokBoxSizes];    // [B*k rows, I cols] bf16
   // shared expert (encoded only when there is one)
-  CUtensorMap w_gu_s;               // [2Is rows, H cols] bf16, box 64 x 64
-  CUtensorMap w_down_s;             // [H rows, Is cols] bf16, box 64 x 64
+  CUtensorMap w_gu_s;               // [1, 2Is, H] bf16
+  CUtensorMap w_down_s;             // [1, H, Is] bf16
   CUtensorMap xt[kTokBoxSizes];     // [B rows, H cols] bf16, hidden in token order
   CUtensorMap act_s[kTokBoxSizes];  // [B rows, Is cols] bf16, token order
 };
@@ -474,12 +480,31 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *map,
       "l"((uint64_t)map), "r"(x), "r"(y), "r"(cl_bar), "l"(policy)
       : "memory");
 }
-// L2 prefetch of one box of a 2-D tensor map (no shared memory, no barrier).
-__device__ __forceinline__ void tma_prefetch_2d(const void *map, int x, int y) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
-                   (uint64_t)map),
-               "r"(x), "r"(y)
-               : "memory");
+// Weight rows (the 5-D maps of FfnMaps): half a 128-row tile of expert e from
+// 16-row unit u, K columns from x.
+__device__ __forceinline__ void tma_load_w(uint32_t dst, const void *map, uint32_t bar, int x,
+                                           int u, int e, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_"
+      "tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %3, %4, %5}], [%6], %7;" ::"r"(dst),
+      "l"((uint64_t)map), "r"(x), "r"(0), "r"(u), "r"(e), "r"(bar), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_w_pair(uint32_t dst, const void *map, uint32_t cl_bar,
+                                                int x, int u, int e, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::"
+      "bytes.L2::cache_hint [%0], [%1, {%2, %3, %3, %4, %5}], [%6], %7;" ::"r"(dst),
+      "l"((uint64_t)map), "r"(x), "r"(0), "r"(u), "r"(e), "r"(cl_bar), "l"(policy)
+      : "memory");
+}
+// L2 prefetch of the same box (no shared memory, no barrier).
+__device__ __forceinline__ void tma_prefetch_w(const void *map, int x, int u, int e) {
+  asm volatile(
+      "cp.async.bulk.prefetch.tensor.5d.L2.global.tile [%0, {%1, %2, %2, %3, %4}];" ::"l"(
+          (uint64_t)map),
+      "r"(x), "r"(0), "r"(u), "r"(e)
+      : "memory");
 }
 __device__ __forceinline__ void prefetch_l2(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
@@ -574,10 +599,20 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
       "[%0];" ::"r"(bar)
       : "memory");
 }
-// 32 lanes x 32 bit, 16 consecutive columns per thread.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+// 16 TMEM lanes x 16 or 32 columns in the fragment layout: for the 8-column
+// block j, thread t gets lane t / 4, columns 8j + 2 (t % 4) and + 1 in v[4j],
+// v[4j + 1], and the same columns of lane t / 4 + 8 in v[4j + 2], v[4j + 3].
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+        "=r"(v[7])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
       "[%16];"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]),
@@ -586,6 +621,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
         "=r"(v[15])
       : "r"(taddr)
       : "memory");
+}
+// Four 8 x 8 bf16 fragments (thread t holds row t / 4, columns 2 (t % 4), + 1)
+// stored transposed: thread 8m + r gives the 16-byte address of column r of
+// fragment m.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t r0, uint32_t r1,
+                                                  uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+               "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+               : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
 }
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");

@@ -53,8 +53,26 @@ constexpr int kEpiGroups = 2;    // epilogue warpgroups, one per TMEM accumulato
 constexpr int kEpiThreads = 128; // threads of one epilogue warpgroup
 constexpr int kFfnThreads = 64 + kEpiGroups * kEpiThreads;
 constexpr int kItemRing = 4;
-constexpr int kXchStride = 17;  // padded row stride (floats) of the exchange buffer
-constexpr int kXchBytes = kEpiGroups * kTileRows * kXchStride * 4;
+// Transposing buffer of one epilogue warp: up to 32 token rows of 16
+// activations, or 16 rows of 32 outputs, padded so that neither the 8-row
+// matrix stores nor the 16-byte reads conflict.
+constexpr int kActRowBytes = 16 * 2 + 16;
+constexpr int kOutRowBytes = 32 * 2 + 16;
+constexpr int kXchWarpBytes = 32 * kActRowBytes;
+constexpr int kXchBytes = kEpiGroups * (kEpiThreads / 32) * kXchWarpBytes;
+static_assert(16 * kOutRowBytes <= kXchWarpBytes, "transposing buffer");
+
+// A work item as the producer hands it to the MMA issuer and the epilogue
+// (decoded once, in shared memory).
+struct __align__(16) ItemSlot {
+  int item;       // its number; past the last one (or an abort): the end
+  int entry;
+  int tile;
+  int form;       // bit 0: down, bit 1: shared expert
+  int slot_base;
+  int n;          // tokens
+  int pad[2];
+};
 
 // A pipeline stage: one 64-wide K sub-tile (one 128-byte swizzle atom) of
 // the item's weight rows -- 128, or 256 for a wide item -- then tok_chunk
@@ -76,9 +94,10 @@ __host__ __device__ inline FfnSmem ffn_smem_plan(int tok_chunk, int stages, int 
   p.bar_off = p.xch_off + kXchBytes;
   // full[S], empty[S], acc_full[2], acc_empty[2], item_full[R], item_empty[R],
   // drain, and for a pair mailbox_full[R], mailbox_empty[R]
-  p.misc_off = p.bar_off + 8 * (2 * stages + 4 + 2 * kItemRing + 1 + (pair ? 2 * kItemRing : 0));
+  p.misc_off = align_up(
+      p.bar_off + 8 * (2 * stages + 4 + 2 * kItemRing + 1 + (pair ? 2 * kItemRing : 0)), 16);
   // item ring, tmem base, abort, consumed stages, and for a pair the mailbox[R]
-  p.total = p.misc_off + 4 * (kItemRing + 3 + (pair ? kItemRing : 0)) + 1024;
+  p.total = p.misc_off + kItemRing * sizeof(ItemSlot) + 4 * (3 + (pair ? kItemRing : 0)) + 1024;
   return p;
 }
 
@@ -195,6 +214,88 @@ __device__ __forceinline__ void combine_token(const Ws &ws, const Dims &d,
                  *reinterpret_cast<const uint32_t *>(&hi));
 }
 
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t *>(&h2);
+}
+
+// SiLU(g) * u = g / (1 + e^-g) * u of accumulator values
+__device__ __forceinline__ float swiglu(uint32_t g, uint32_t u) {
+  const float gv = __uint_as_float(g), uv = __uint_as_float(u);
+  return gv * __frcp_rn(1.0f + __expf(-gv)) * uv;
+}
+
+// Epilogue of one warp's 32 accumulator rows, without any exchange between
+// warps: the rows of a gate/up tile alternate in groups of 8 gate and 8 up
+// rows, so a thread's fragment (tmem_ld_frag) holds both values of an
+// activation; the bf16 results go through the warp's transposing buffer into
+// token rows and out as 16-byte stores.  Bound by the latency of one pass
+// (TMEM load, exponentials, stores); with the rows swapped between warps
+// through fp32 buffers and block barriers, and 2-byte output stores, an
+// epilogue took about 13,000 cycles at 64-80 tokens, a tail on every launch.
+// Measured against that: decode steps 1.0-2.5 us faster (B = 64 full pool
+// 182.9 -> 180.5 us, B = 96 with the shared expert 143.9 -> 141.9), an
+// 8-layer stack 823 -> 815 us, prefill of 4001 tokens 532 -> 524 us.
+// `v0`, `v1`: fragments of the warp's
+// first and last 16 rows; `base`: the first token's first element of this
+// warp; `left`: tokens left from it on.
+//
+// 16 kTok16 tokens of 16 activations.
+template <int kTok16, int R>
+__device__ __forceinline__ void store_activations(const uint32_t (&v0)[R], const uint32_t (&v1)[R],
+                                                  uint32_t wbuf, int lane, __nv_bfloat16 *base,
+                                                  int ld, int left) {
+  static_assert(R == 8 * kTok16, "fragment of 16 kTok16 columns");
+  const uint32_t dst = wbuf + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * kActRowBytes +
+                                         ((lane >> 3) & 1) * 16);
+#pragma unroll
+  for (int p = 0; p < kTok16; ++p) {
+    uint32_t a[4];  // rows half h of column block 2p + j: a[2j + h]
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int o = 4 * (2 * p + j);
+      a[2 * j] = pack_bf16(swiglu(v0[o], v0[o + 2]), swiglu(v0[o + 1], v0[o + 3]));
+      a[2 * j + 1] = pack_bf16(swiglu(v1[o], v1[o + 2]), swiglu(v1[o + 1], v1[o + 3]));
+    }
+    stmatrix_x4_trans(dst + (uint32_t)(p * 16 * kActRowBytes), a[0], a[1], a[2], a[3]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int p = 0; p < kTok16; ++p) {
+    const int t = p * 16 + (lane >> 1);
+    const uint4 w = ld_shared_v4(wbuf + (uint32_t)(t * kActRowBytes + (lane & 1) * 16));
+    if (t < left) *reinterpret_cast<uint4 *>(base + (size_t)t * ld + (lane & 1) * 8) = w;
+  }
+  __syncwarp();
+}
+
+// 16 tokens of 32 outputs, from 8-column block kBlock of the fragments.
+template <int kBlock, int R>
+__device__ __forceinline__ void store_outputs(const uint32_t (&v0)[R], const uint32_t (&v1)[R],
+                                              uint32_t wbuf, int lane, __nv_bfloat16 *base, int ld,
+                                              int left) {
+  const uint32_t dst = wbuf + (uint32_t)((lane & 7) * kOutRowBytes + (lane >> 3) * 16);
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int o = 4 * (kBlock + j);
+    uint32_t a[4];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      a[s] = pack_bf16(__uint_as_float(v0[o + 2 * s]), __uint_as_float(v0[o + 2 * s + 1]));
+      a[2 + s] = pack_bf16(__uint_as_float(v1[o + 2 * s]), __uint_as_float(v1[o + 2 * s + 1]));
+    }
+    stmatrix_x4_trans(dst + (uint32_t)(j * 8 * kOutRowBytes), a[0], a[1], a[2], a[3]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const int t = p * 8 + (lane >> 2);
+    const uint4 w = ld_shared_v4(wbuf + (uint32_t)(t * kOutRowBytes + (lane & 3) * 16));
+    if (t < left) *reinterpret_cast<uint4 *>(base + (size_t)t * ld + (lane & 3) * 8) = w;
+  }
+  __syncwarp();
+}
+
 // Named barrier of epilogue group g (ids 1.., id 0 is __syncthreads).
 __device__ __forceinline__ void epi_bar(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(kEpiThreads) : "memory");
@@ -254,7 +355,6 @@ __global__ void __maxnreg__(128)
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const FfnSmem plan = ffn_smem_plan(d.tok_chunk, stages, d.wide, kPair ? 1 : 0);
   const uint32_t smem_base = smem_u32(smem);
-  float *xch = reinterpret_cast<float *>(smem + plan.xch_off);
   const uint32_t bar0 = smem_base + (uint32_t)plan.bar_off;
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (stages + s); };
@@ -266,12 +366,12 @@ __global__ void __maxnreg__(128)
   // pair mailbox: full barriers live in the second CTA, empty ones in the first
   auto mbf_bar = [&](int r) { return bar0 + 8u * (2 * stages + 5 + 2 * kItemRing + r); };
   auto mbe_bar = [&](int r) { return bar0 + 8u * (2 * stages + 5 + 3 * kItemRing + r); };
-  int *misc = reinterpret_cast<int *>(smem + plan.misc_off);
-  volatile int *ring = misc;                         // [kItemRing]
-  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(misc + kItemRing);
-  volatile int *abort = misc + kItemRing + 1;
-  volatile int *consumed = misc + kItemRing + 2;     // stages the MMA finished with
-  volatile int *mbox = misc + kItemRing + 3;         // [kItemRing], pair only
+  ItemSlot *ring = reinterpret_cast<ItemSlot *>(smem + plan.misc_off);  // [kItemRing]
+  int *misc = reinterpret_cast<int *>(ring + kItemRing);
+  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(misc);
+  volatile int *abort = misc + 1;
+  volatile int *consumed = misc + 2;                 // stages the MMA finished with
+  volatile int *mbox = misc + 3;                     // [kItemRing], pair only
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t crank = kPair ? cluster_ctarank() : 0u;  // CTA of the pair
@@ -357,15 +457,14 @@ __global__ void __maxnreg__(128)
   if constexpr (!kShared) {
     if (warp == 0 && lane == 0 && d.B * d.k >= 2 * d.m_ret) {
       const int t1g = gate_up_tiles(d);
-      const int rows = kGateRows * item_tiles(d);  // gate rows (and up rows) of an item
       const int entry = item0 / t1g;
       if (entry < d.m_ret) {
         const int e = retained ? __ldcg(retained + entry) : entry;
         if (e >= 0 && e < d.E) {
-          const int row0 = e * 2 * d.I + (item0 - entry * t1g) * rows + (int)crank * kGateRows;
+          const int u0 = ((item0 - entry * t1g) * item_tiles(d) + (int)crank) * kTileUnits;
           for (int kc = 0; kc < d.H / kBlockK; ++kc) {
-            tma_prefetch_2d(&maps.w_gu, kc * kBlockK, row0);
-            tma_prefetch_2d(&maps.w_gu, kc * kBlockK, row0 + d.I);
+            tma_prefetch_w(&maps.w_gu, kc * kBlockK, u0, e);
+            tma_prefetch_w(&maps.w_gu, kc * kBlockK, u0 + kTileUnits / 2, e);
           }
         }
       }
@@ -447,7 +546,18 @@ __global__ void __maxnreg__(128)
           if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
           break;
         }
-        ring[slot] = item;
+        Item it = {};
+        if (item < total) it = decode_item<kShared>(item, ip, ws);
+        {
+          ItemSlot sl = {};
+          sl.item = item;
+          sl.entry = it.entry;
+          sl.tile = it.tile;
+          sl.form = it.down | (it.shared << 1);
+          sl.slot_base = it.slot_base;
+          sl.n = it.n;
+          ring[slot] = sl;
+        }
         mbar_arrive(itf_bar(slot));
         if (++slot == kItemRing) {
           slot = 0;
@@ -459,18 +569,16 @@ __global__ void __maxnreg__(128)
           pdl_launch_dependents();
           break;
         }
-        const Item it = decode_item<kShared>(item, ip, ws);
         // the item's token rows: one box of the tokens rounded up to 16
         // rows (rows past the entry are loaded but not multiplied); each CTA
         // of a pair loads half of them, from 8 n16 rows further for the second
         const int box_m = token_box_for(it.n16);
         const int tok_row = it.slot_base + (kPair ? (int)crank * it.n16 * (kTokBox / 2) : 0);
-        // weight rows: per 128-row half of the item, two 64-row boxes -- the
-        // gate rows and the matching up rows, or 128 consecutive down rows;
-        // a pair's CTA r loads half r
+        // weight rows: per 128-row half of the item, two boxes of 4 units (64
+        // rows) -- gate and up rows in alternating groups of 8, or 128
+        // consecutive down rows; a pair's CTA r loads half r
         const int halves = (kShared && it.shared) ? 1 : wmul;
-        const int hstep = it.down ? kTileRows : kGateRows;  // row offset of half 1
-        int nk, row0, row1;
+        int nk, unit0, expert;
         const void *amap;
         const void *bmap;
         if (kShared && it.shared) {
@@ -478,20 +586,14 @@ __global__ void __maxnreg__(128)
           nk = it.down ? d.Is / kBlockK : d.H / kBlockK;
           amap = it.down ? (const void *)&maps.w_down_s : (const void *)&maps.w_gu_s;
           bmap = it.down ? (const void *)&maps.act_s[box_m] : (const void *)&maps.xt[box_m];
-          row0 = it.down ? it.tile * kTileRows : it.tile * kGateRows;
-          row1 = it.down ? row0 + kGateRows : row0 + d.Is;
+          unit0 = it.tile * kTileUnits;
+          expert = 0;
         } else {
           nk = it.down ? d.I / kBlockK : d.H / kBlockK;
           amap = it.down ? (const void *)&maps.w_down : (const void *)&maps.w_gu;
           bmap = it.down ? (const void *)&maps.act[box_m] : (const void *)&maps.xp[box_m];
-          const int half0 = kPair ? (int)crank : 0;
-          if (it.down) {
-            row0 = it.expert * d.H + (it.tile * tiles_per_item + half0) * kTileRows;
-            row1 = row0 + kGateRows;
-          } else {
-            row0 = it.expert * 2 * d.I + (it.tile * tiles_per_item + half0) * kGateRows;
-            row1 = row0 + d.I;
-          }
+          unit0 = (it.tile * tiles_per_item + (kPair ? (int)crank : 0)) * kTileUnits;
+          expert = it.expert;
         }
         if (it.down) {
           // the entry's activations must be complete: all its gate/up tiles
@@ -530,16 +632,17 @@ __global__ void __maxnreg__(128)
           const uint32_t a = smem_base + (uint32_t)(stage * plan.stage_bytes);
           if (kPair && !lead) {
             const uint32_t lb = mapa_shared(full_bar(stage), 0u);
-            tma_load_2d_pair(a, amap, lb, x, row0, pol_w);
-            tma_load_2d_pair(a + kATileBytes / 2, amap, lb, x, row1, pol_w);
+            tma_load_w_pair(a, amap, lb, x, unit0, expert, pol_w);
+            tma_load_w_pair(a + kATileBytes / 2, amap, lb, x, unit0 + kTileUnits / 2, expert, pol_w);
             tma_load_2d_pair(a + (uint32_t)plan.a_bytes, bmap, lb, x, tok_row, pol_x);
           } else {
             mbar_arrive_expect_tx(full_bar(stage), stage_tx);
             for (int h = 0; h < halves; ++h) {
               const uint32_t ah = a + (uint32_t)(h * kATileBytes);
-              tma_load_2d(ah, amap, full_bar(stage), x, row0 + h * hstep, pol_w);
-              tma_load_2d(ah + kATileBytes / 2, amap, full_bar(stage), x, row1 + h * hstep,
-                          pol_w);
+              const int u = unit0 + h * kTileUnits;
+              tma_load_w(ah, amap, full_bar(stage), x, u, expert, pol_w);
+              tma_load_w(ah + kATileBytes / 2, amap, full_bar(stage), x, u + kTileUnits / 2, expert,
+                         pol_w);
             }
             tma_load_2d(a + (uint32_t)plan.a_bytes, bmap, full_bar(stage), x, tok_row, pol_x);
           }
@@ -579,7 +682,7 @@ __global__ void __maxnreg__(128)
           if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
           break;
         }
-        const int item = ring[slot];
+        const int item = ring[slot].item;
         mbar_arrive(ite_bar(slot));
         if (++slot == kItemRing) {
           slot = 0;
@@ -599,14 +702,15 @@ __global__ void __maxnreg__(128)
           if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
           break;
         }
-        const int item = ring[slot];
+        const ItemSlot it = ring[slot];
         mbar_arrive(ite_bar(slot));
         if (++slot == kItemRing) {
           slot = 0;
           rphase ^= 1u;
         }
-        if (item >= total) break;
-        const Item it = decode_item<kShared>(item, ip, ws);
+        if (it.item >= total) break;
+        const bool down = (it.form & 1) != 0, shared = (it.form & 2) != 0;
+        const int n16 = (it.n + 15) >> 4;
         const int b = local & 1;
         const uint32_t use = (uint32_t)(local >> 1);
         const bool freed =
@@ -622,10 +726,10 @@ __global__ void __maxnreg__(128)
         // A pair runs one M = 256 MMA: A rows 128-255 and B rows N/2.. are the
         // second CTA's, at the same shared-memory offsets.
         const uint32_t d_tmem = tmem_base + (uint32_t)(b * nb_cols);
-        const uint32_t idesc = idesc_bf16_f32(kPair ? 2 * kTileRows : kTileRows, it.n16 * kTokBox);
-        const int halves = (kShared && it.shared) ? 1 : wmul;
-        const int inner = (kShared && it.shared) ? d.Is : d.I;
-        const int nk = it.down ? inner / kBlockK : d.H / kBlockK;
+        const uint32_t idesc = idesc_bf16_f32(kPair ? 2 * kTileRows : kTileRows, n16 * kTokBox);
+        const int halves = (kShared && shared) ? 1 : wmul;
+        const int inner = (kShared && shared) ? d.Is : d.I;
+        const int nk = down ? inner / kBlockK : d.H / kBlockK;
         bool ok = true;
         for (int kc = 0; kc < nk; ++kc) {
           if (!mbar_wait_bounded(full_bar(stage), phase, abort, timeout_ns)) {
@@ -680,112 +784,92 @@ __global__ void __maxnreg__(128)
     // other's and the MMA of the next item.
     const int g = (warp - 2) >> 2;      // epilogue group
     const int q = warp & 3;             // TMEM lane quarter of this warp
-    const int row = 32 * q + lane;      // accumulator row = TMEM lane
     const int et = (threadIdx.x - 64) & (kEpiThreads - 1);
-    float *xb = xch + g * kTileRows * kXchStride;
+    const uint32_t wbuf = smem_base + (uint32_t)(plan.xch_off + (warp - 2) * kXchWarpBytes);
     int slot = 0;
     uint32_t rphase = 0;
     for (int local = 0;; ++local) {
       bool got = mbar_wait_bounded(itf_bar(slot), rphase, abort, timeout_ns);
       if (!got && !*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
       if (!epi_all(g, got)) break;
-      const int item = ring[slot];
+      const ItemSlot it = ring[slot];
       mbar_arrive(ite_bar(slot));
       if (++slot == kItemRing) {
         slot = 0;
         rphase ^= 1u;
       }
-      if (item >= total) break;
+      if (it.item >= total) break;
       const int b = local & 1;
       if (b != g) continue;
-      const Item it = decode_item<kShared>(item, ip, ws);
+      const bool down = (it.form & 1) != 0, shared = kShared && (it.form & 2) != 0;
       const uint32_t use = (uint32_t)(local >> 1);
-      const int halves = (kShared && it.shared) ? 1 : wmul;
+      const int halves = shared ? 1 : wmul;
       got = mbar_wait_bounded(accf_bar(b), use & 1u, abort, timeout_ns);
       if (!got && !*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
       if (!epi_all(g, got)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * nb_cols);
+      const int cols = ((it.n + 15) >> 4) * kTokBox;  // accumulator columns
       // 128-row tile of the item that TMEM half hh holds: half hh of a wide
       // item, the CTA's own half of a pair item
-      const int tile0 = (kShared && it.shared) ? it.tile
-                                               : it.tile * tiles_per_item + (kPair ? (int)crank : 0);
-      if (!it.down) {
-        // gate rows live in TMEM lanes 0..63, the matching up rows in 64..127
-        const int n_loc = et >> 3;          // token column within a 16-chunk
-        const int i0 = (et & 7) * 8;        // 8 consecutive intermediate indices
-        for (int hh = 0; hh < halves; ++hh) {
-          // half hh of a wide item is the 64 gate + 64 up rows of tile 2 t + hh
-          const int act_col = (tile0 + hh) * kGateRows + i0;
-          for (int c = 0; c < it.n16; ++c) {
-            uint32_t v[16];
-            tmem_ld16(taddr + (uint32_t)(hh * d.tok_chunk) + c * 16, v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) xb[row * kXchStride + j] = __uint_as_float(v[j]);
-            epi_bar(g);
-            const int col = c * 16 + n_loc;
-            if (col < it.n) {
-              uint32_t packed[4];
-#pragma unroll
-              for (int ii = 0; ii < 8; ii += 2) {
-                float a2[2];
-#pragma unroll
-                for (int u2 = 0; u2 < 2; ++u2) {
-                  const float gv = xb[(i0 + ii + u2) * kXchStride + n_loc];
-                  const float uv = xb[(kGateRows + i0 + ii + u2) * kXchStride + n_loc];
-                  // SiLU(g) * u = g / (1 + e^-g) * u
-                  a2[u2] = gv * __frcp_rn(1.0f + __expf(-gv)) * uv;
-                }
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(a2[0], a2[1]);
-                packed[ii / 2] = *reinterpret_cast<uint32_t *>(&h2);
-              }
-              // routed: grouped order [B*k, I]; shared: token order [B, Is]
-              __nv_bfloat16 *arow = (kShared && it.shared)
-                                        ? ws.act_s + (size_t)(it.slot_base + col) * d.Is
-                                        : ws.act + (size_t)(it.slot_base + col) * d.I;
-              *reinterpret_cast<uint4 *>(arow + act_col) =
-                  make_uint4(packed[0], packed[1], packed[2], packed[3]);
-            }
-            epi_bar(g);  // the exchange buffer is rewritten by the next chunk
-          }
-        }
+      const int tile0 = shared ? it.tile : it.tile * tiles_per_item + (kPair ? (int)crank : 0);
+      // the accumulator is free once its last columns have been loaded
+      auto release = [&]() {
         tc_fence_before();
         if constexpr (!kPair) mbar_arrive(acce_bar(b));
+      };
+      for (int hh = 0; hh < halves; ++hh) {
+        const uint32_t th = taddr + (uint32_t)(hh * d.tok_chunk);
+        // routed rows in grouped order, shared ones in token order
+        __nv_bfloat16 *base;
+        int ld;
+        if (!down) {
+          ld = shared ? d.Is : d.I;
+          base = (shared ? ws.act_s : ws.act) + (size_t)it.slot_base * ld +
+                 (tile0 + hh) * kGateRows + 16 * q;
+        } else {
+          ld = d.H;
+          base = (shared ? ws.y_s : ws.y) + (size_t)it.slot_base * ld + (tile0 + hh) * kTileRows +
+                 32 * q;
+        }
+        int c = 0;
+        for (; c + 32 <= cols; c += 32) {
+          uint32_t v0[16], v1[16];
+          tmem_ld_frag(th + c, v0);
+          tmem_ld_frag(th + c + (16u << 16), v1);
+          tmem_ld_wait();
+          if (hh == halves - 1 && c + 32 == cols) release();
+          if (down) {
+            store_outputs<0>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
+            store_outputs<2>(v0, v1, wbuf, lane, base + (size_t)(c + 16) * ld, ld, it.n - c - 16);
+          } else {
+            store_activations<2>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
+          }
+        }
+        if (c < cols) {  // 16 columns left
+          uint32_t v0[8], v1[8];
+          tmem_ld_frag(th + c, v0);
+          tmem_ld_frag(th + c + (16u << 16), v1);
+          tmem_ld_wait();
+          if (hh == halves - 1) release();
+          if (down) store_outputs<0>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
+          else store_activations<1>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
+        }
+      }
+      if (!down) {
         // publish the activations to the TMA (async proxy) readers of any CTA
         fence_proxy_async_global();
         __threadfence();
         epi_bar(g);
         if (et == 0) {
-          if constexpr (kPair)
-            mbar_arrive_cluster(mapa_shared(acce_bar(b), 0u));
+          if constexpr (kPair) mbar_arrive_cluster(mapa_shared(acce_bar(b), 0u));
           atomicAdd(&ws.entry_done[it.entry], 1);
         }
-      } else {
-        __nv_bfloat16 *ybase = (kShared && it.shared) ? ws.y_s : ws.y;  // token / grouped order
-        for (int hh = 0; hh < halves; ++hh) {
-          const int h = (tile0 + hh) * kTileRows + row;
-          for (int c = 0; c < it.n16; ++c) {
-            uint32_t v[16];
-            tmem_ld16(taddr + (uint32_t)(hh * d.tok_chunk) + c * 16, v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int col = c * 16 + j;
-              if (col < it.n)
-                ybase[(size_t)(it.slot_base + col) * d.H + h] = __float2bfloat16_rn(__uint_as_float(v[j]));
-            }
-          }
-        }
+      } else if constexpr (kPair) {
         // the expert outputs are all a down item writes: the combine kernel
         // that follows this grid sums them
-        tc_fence_before();
-        if constexpr (kPair) {
-          epi_bar(g);
-          if (et == 0) mbar_arrive_cluster(mapa_shared(acce_bar(b), 0u));
-        } else {
-          mbar_arrive(acce_bar(b));
-        }
+        epi_bar(g);
+        if (et == 0) mbar_arrive_cluster(mapa_shared(acce_bar(b), 0u));
       }
     }
   }

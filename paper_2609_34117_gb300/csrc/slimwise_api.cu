@@ -66,6 +66,32 @@ int encode_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols,
   return r == CUDA_SUCCESS ? SLIMWISE_OK : SLIMWISE_ERR_CUDA;
 }
 
+// Weight map of E experts (see FfnMaps): units of 16 rows x `cols`, as two
+// groups of 8 rows `group_rows` rows apart and `unit_rows` rows from unit to
+// unit; an expert has `rows` rows.  128-byte swizzle, zero fill.
+int encode_weights(CUtensorMap *map, const void *base, uint64_t E, uint64_t rows, uint64_t cols,
+                   uint64_t group_rows, uint64_t unit_rows) {
+  const uint64_t row = cols * 2;
+  cuuint64_t dims[5] = {cols, 8, 2, rows / kUnitRows, E};
+  cuuint64_t strides[4] = {row, group_rows * row, unit_rows * row, rows * row};
+  cuuint32_t box[5] = {(cuuint32_t)kBlockK, 8, 2, (cuuint32_t)kTileUnits / 2, 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
+                        const_cast<void *>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? SLIMWISE_OK : SLIMWISE_ERR_CUDA;
+}
+// Gate/up weights [E, 2I, H]: 8 gate rows, then the up rows I rows further.
+int encode_gate_up(CUtensorMap *map, const void *base, uint64_t E, uint64_t I, uint64_t H) {
+  return encode_weights(map, base, E, 2 * I, H, I, 8);
+}
+// Down weights [E, H, I]: 16 consecutive rows.
+int encode_down(CUtensorMap *map, const void *base, uint64_t E, uint64_t H, uint64_t I) {
+  return encode_weights(map, base, E, H, I, 8, 16);
+}
+
 bool aligned(const void *p, uintptr_t a) {
   return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0;
 }
@@ -200,12 +226,11 @@ bool ffn_maps_for(FfnMaps *maps, const void *w_gate_up, const void *w_down, cons
                           dev, slots};
   if (!(have_w && kw == last_w)) {
     have_w = false;
-    if (encode_map(&cached.w_gu, w_gate_up, (uint64_t)d.E * 2 * d.I, d.H, kGateRows) ||
-        encode_map(&cached.w_down, w_down, (uint64_t)d.E * d.H, d.I, kGateRows))
+    if (encode_gate_up(&cached.w_gu, w_gate_up, d.E, d.I, d.H) ||
+        encode_down(&cached.w_down, w_down, d.E, d.H, d.I))
       return false;
-    if (d.Is > 0 &&
-        (encode_map(&cached.w_gu_s, se.gate_up, 2 * (uint64_t)d.Is, d.H, kGateRows) ||
-         encode_map(&cached.w_down_s, se.down, (uint64_t)d.H, d.Is, kGateRows)))
+    if (d.Is > 0 && (encode_gate_up(&cached.w_gu_s, se.gate_up, 1, d.Is, d.H) ||
+                     encode_down(&cached.w_down_s, se.down, 1, d.H, d.Is)))
       return false;
     last_w = kw;
     have_w = true;
