@@ -217,6 +217,10 @@ __host__ __device__ inline int gate_up_tiles(const Dims &d) {
 __host__ __device__ inline int down_tiles(const Dims &d) {
   return d.H / (kTileRows * item_tiles(d));
 }
+// Gate/up items of one entry of the shared expert (0: none).
+__host__ __device__ inline int shared_gate_up_tiles(const Dims &d) {
+  return d.Is / (kGateRows * item_tiles(d));
+}
 // Wide items need whole 256-row tiles of both weights and no shared expert
 // (its items keep 128 rows, and a stage holds one kind of A tile).  Two
 // weight tiles then share each stage's token rows, which halves the token
@@ -323,6 +327,20 @@ __device__ __forceinline__ void pdl_wait_primary() {
 }
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// One thread of a converged warp (the same one at every call).  Copies and MMAs
+// are issued from a loop that the whole warp runs, under this predicate: their
+// operands then stay in uniform registers, where a loop run by lane 0 alone
+// moves each of them there for every instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
 }
 
 // mbarrier ------------------------------------------------------------------

@@ -53,6 +53,7 @@ constexpr int kEpiGroups = 2;    // epilogue warpgroups, one per TMEM accumulato
 constexpr int kEpiThreads = 128; // threads of one epilogue warpgroup
 constexpr int kFfnThreads = 64 + kEpiGroups * kEpiThreads;
 constexpr int kItemRing = 4;
+constexpr int kNoItem = 0x7FFFFFFF;  // past every item: no more work
 // Transposing buffer of one epilogue warp: up to 32 token rows of 16
 // activations, or 16 rows of 32 outputs, padded so that neither the 8-row
 // matrix stores nor the 16-byte reads conflict.
@@ -114,7 +115,6 @@ struct Item {
   int expert;
   int slot_base;
   int n;         // tokens
-  int n16;       // tokens rounded up to 16, / 16
 };
 
 // Work-item ranges of one launch, in the order they are handed out:
@@ -164,7 +164,6 @@ __device__ __forceinline__ Item decode_item(int item, const ItemPlan &ip, const 
   it.expert = en.x;
   it.slot_base = en.y;
   it.n = en.z;
-  it.n16 = (en.z + 15) >> 4;
   return it;
 }
 
@@ -349,7 +348,7 @@ __global__ void __maxnreg__(128)
                       int tmem_cols, int static_first, int early_dependents,
                       uint64_t timeout_ns,
                       int starve_first_down) {
-  static_assert(!(kPair && (kShared || kWide)), "pair items are routed 128-row tiles");
+  static_assert(!(kPair && kWide), "a pair item is a 128-row tile in each CTA");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -489,7 +488,7 @@ __global__ void __maxnreg__(128)
   ItemPlan ip;
   ip.r1 = __ldcg(&ws.ctrl[kCtrlItems1]);
   ip.t1 = t1;
-  ip.t1s = kShared ? d.Is / kGateRows : 0;
+  ip.t1s = kShared ? shared_gate_up_tiles(d) : 0;
   ip.t2 = t2;
   ip.S = kShared ? d.S : 0;
   const int nb_cols = ffn_acc_cols(d);  // TMEM columns per accumulator buffer
@@ -501,135 +500,144 @@ __global__ void __maxnreg__(128)
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
-      const uint64_t pol_w = l2_policy_evict_first();
-      const uint64_t pol_x = l2_policy_evict_last();
-      int stage = 0;
-      uint32_t phase = 0;
-      int slot = 0;
-      uint32_t rphase = 0;
-      int issued = 0;
-      // With every CTA of the grid resident (one per SM), CTA i's first item
-      // is item i (for pairs, cluster i's) and later ones come from the
-      // counter past the grid: the first item costs no atomic round trip after
-      // the dependency wait.
-      const int n_first = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-      bool first = static_first != 0;
-      for (;;) {
-        int item;
-        if (!kPair || lead) {
-          item = first ? item0
-                       : (static_first ? n_first : 0) + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
-          first = false;
-          if (*abort) item = 0x7FFFFFFF;
-          if constexpr (kPair) {
-            // hand the item to the second CTA; an item past the end (or the
-            // abort sentinel) ends its loop too
-            if (!mbar_wait_cluster_bounded(mbe_bar(slot), rphase ^ 1u, nullptr, timeout_ns)) {
-              if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-              break;
-            }
+    // The whole warp runs the loop (see elect_one); what depends on memory is
+    // read once per item and broadcast, so everything the copies take is
+    // uniform over the warp.
+    const uint64_t pol_w = l2_policy_evict_first();
+    const uint64_t pol_x = l2_policy_evict_last();
+    int stage = 0;
+    uint32_t phase = 0;
+    int slot = 0;
+    uint32_t rphase = 0;
+    int issued = 0;
+    // With every CTA of the grid resident (one per SM), CTA i's first item
+    // is item i (for pairs, cluster i's) and later ones come from the
+    // counter past the grid: the first item costs no atomic round trip after
+    // the dependency wait.
+    const int n_first = static_first ? (int)(kPair ? gridDim.x >> 1 : gridDim.x) : 0;
+    bool first = static_first != 0;
+    // a bounded wait of the warp: whether it completed on every lane
+    auto all_ok = [&](bool ok) {
+      if (!ok && !*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
+      return __all_sync(0xFFFFFFFFu, ok) != 0;
+    };
+    for (;;) {
+      int item = 0;
+      if (!kPair || lead) {
+        if (lane == 0) {
+          item = first ? item0 : n_first + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
+          if (*abort) item = kNoItem;
+        }
+        first = false;
+        if constexpr (kPair) {
+          // hand the item to the second CTA; an item past the end (or the
+          // abort sentinel) ends its loop too
+          if (!all_ok(mbar_wait_cluster_bounded(mbe_bar(slot), rphase ^ 1u, nullptr, timeout_ns)))
+            break;
+          if (lane == 0) {
             st_shared_cluster(mapa_shared(smem_u32((const void *)(mbox + slot)), 1u), item);
             mbar_arrive_cluster(mapa_shared(mbf_bar(slot), 1u));
           }
-        } else {
-          // the second CTA of a pair: the item its first CTA took
-          if (!mbar_wait_cluster_bounded(mbf_bar(slot), rphase, abort, timeout_ns)) {
-            if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-            break;
-          }
+        }
+      } else {
+        // the second CTA of a pair: the item its first CTA took
+        if (!all_ok(mbar_wait_cluster_bounded(mbf_bar(slot), rphase, abort, timeout_ns))) break;
+        if (lane == 0) {
           item = mbox[slot];
           mbar_arrive_cluster(mapa_shared(mbe_bar(slot), 0u));
-          if (*abort) item = 0x7FFFFFFF;
+          if (*abort) item = kNoItem;
         }
-        if (!mbar_wait_bounded(ite_bar(slot), rphase ^ 1u, abort, timeout_ns)) {
-          if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-          break;
-        }
-        Item it = {};
-        if (item < total) it = decode_item<kShared>(item, ip, ws);
-        {
-          ItemSlot sl = {};
-          sl.item = item;
-          sl.entry = it.entry;
-          sl.tile = it.tile;
-          sl.form = it.down | (it.shared << 1);
-          sl.slot_base = it.slot_base;
-          sl.n = it.n;
-          ring[slot] = sl;
-        }
+      }
+      item = __shfl_sync(0xFFFFFFFFu, item, 0);
+      if (!all_ok(mbar_wait_bounded(ite_bar(slot), rphase ^ 1u, abort, timeout_ns))) break;
+      Item it = {};
+      if (item < total) it = decode_item<kShared>(item, ip, ws);
+      it.expert = __shfl_sync(0xFFFFFFFFu, it.expert, 0);
+      it.slot_base = __shfl_sync(0xFFFFFFFFu, it.slot_base, 0);
+      it.n = __shfl_sync(0xFFFFFFFFu, it.n, 0);
+      if (lane == 0) {
+        ItemSlot sl = {};
+        sl.item = item;
+        sl.entry = it.entry;
+        sl.tile = it.tile;
+        sl.form = it.down | (it.shared << 1);
+        sl.slot_base = it.slot_base;
+        sl.n = it.n;
+        ring[slot] = sl;
         mbar_arrive(itf_bar(slot));
-        if (++slot == kItemRing) {
-          slot = 0;
-          rphase ^= 1u;
+      }
+      if (++slot == kItemRing) {
+        slot = 0;
+        rphase ^= 1u;
+      }
+      if (item >= total) {
+        // no work left for this CTA: the next kernel on the stream may start
+        // its launch (it waits for this grid's completion before reading)
+        pdl_launch_dependents();
+        break;
+      }
+      // the item's token rows: one box of the tokens rounded up to 16
+      // rows (rows past the entry are loaded but not multiplied); each CTA
+      // of a pair loads half of them, from 8 n16 rows further for the second
+      const int n16 = (it.n + 15) >> 4;
+      const int box_m = token_box_for(n16);
+      const int tok_row = it.slot_base + (kPair ? (int)crank * n16 * (kTokBox / 2) : 0);
+      // weight rows: per 128-row half of the item, two boxes of 4 units (64
+      // rows) -- gate and up rows in alternating groups of 8, or 128
+      // consecutive down rows; a pair's CTA r loads half r
+      const int halves = (kShared && it.shared) ? 1 : wmul;
+      const int unit0 = (it.tile * tiles_per_item + (kPair ? (int)crank : 0)) * kTileUnits;
+      int nk, expert;
+      const void *amap;
+      const void *bmap;
+      if (kShared && it.shared) {
+        // the shared expert: its own weights, tokens in batch order
+        nk = it.down ? d.Is / kBlockK : d.H / kBlockK;
+        amap = it.down ? (const void *)&maps.w_down_s : (const void *)&maps.w_gu_s;
+        bmap = it.down ? (const void *)&maps.act_s[box_m] : (const void *)&maps.xt[box_m];
+        expert = 0;
+      } else {
+        nk = it.down ? d.I / kBlockK : d.H / kBlockK;
+        amap = it.down ? (const void *)&maps.w_down : (const void *)&maps.w_gu;
+        bmap = it.down ? (const void *)&maps.act[box_m] : (const void *)&maps.xp[box_m];
+        expert = it.expert;
+      }
+      if (it.down) {
+        // the entry's activations must be complete: all its gate/up tiles
+        const int *done = &ws.entry_done[it.entry];
+        int need = ((kShared && it.shared) ? ip.t1s : t1) * (kPair ? 2 : 1);
+        // test only: the first routed down item waits for one gate/up tile
+        // more than exist, so its wait runs out (the timeout path)
+        if (starve_first_down && item == ip.S * ip.t1s + ip.r1) ++need;
+        bool ok = __all_sync(0xFFFFFFFFu, ld_acquire(done) >= need) != 0;
+        if (!ok) {
+          const uint64_t t0 = global_timer_ns();
+          while (!(ok = __all_sync(0xFFFFFFFFu, ld_acquire(done) >= need) != 0)) {
+            bool give_up = *abort != 0;
+            if (!give_up && global_timer_ns() - t0 > timeout_ns) {
+              raise_abort(abort, ws, SLIMWISE_DEVERR_DEPENDENCY_TIMEOUT);
+              give_up = true;
+            }
+            if (__any_sync(0xFFFFFFFFu, give_up)) break;
+            __nanosleep(128);
+          }
         }
-        if (item >= total) {
-          // no work left for this CTA: the next kernel on the stream may start
-          // its launch (it waits for this grid's completion before reading)
-          pdl_launch_dependents();
+        if (!ok) break;
+        fence_proxy_async_global();
+      }
+      // bytes the stage barrier expects: for a pair, both CTAs' copies
+      const uint32_t stage_tx =
+          kPair ? (uint32_t)(2 * kATileBytes + n16 * kTokBox * kBlockK * 2)
+                : (uint32_t)(halves * kATileBytes + n16 * kTokBox * kBlockK * 2);
+      bool ok = true;
+      for (int kc = 0; kc < nk; ++kc) {
+        if (!all_ok(mbar_wait_bounded(empty_bar(stage), phase ^ 1u, abort, timeout_ns))) {
+          ok = false;
           break;
         }
-        // the item's token rows: one box of the tokens rounded up to 16
-        // rows (rows past the entry are loaded but not multiplied); each CTA
-        // of a pair loads half of them, from 8 n16 rows further for the second
-        const int box_m = token_box_for(it.n16);
-        const int tok_row = it.slot_base + (kPair ? (int)crank * it.n16 * (kTokBox / 2) : 0);
-        // weight rows: per 128-row half of the item, two boxes of 4 units (64
-        // rows) -- gate and up rows in alternating groups of 8, or 128
-        // consecutive down rows; a pair's CTA r loads half r
-        const int halves = (kShared && it.shared) ? 1 : wmul;
-        int nk, unit0, expert;
-        const void *amap;
-        const void *bmap;
-        if (kShared && it.shared) {
-          // the shared expert: its own weights, tokens in batch order
-          nk = it.down ? d.Is / kBlockK : d.H / kBlockK;
-          amap = it.down ? (const void *)&maps.w_down_s : (const void *)&maps.w_gu_s;
-          bmap = it.down ? (const void *)&maps.act_s[box_m] : (const void *)&maps.xt[box_m];
-          unit0 = it.tile * kTileUnits;
-          expert = 0;
-        } else {
-          nk = it.down ? d.I / kBlockK : d.H / kBlockK;
-          amap = it.down ? (const void *)&maps.w_down : (const void *)&maps.w_gu;
-          bmap = it.down ? (const void *)&maps.act[box_m] : (const void *)&maps.xp[box_m];
-          unit0 = (it.tile * tiles_per_item + (kPair ? (int)crank : 0)) * kTileUnits;
-          expert = it.expert;
-        }
-        if (it.down) {
-          // the entry's activations must be complete: all its gate/up tiles
-          const int *done = &ws.entry_done[it.entry];
-          int need = (kShared && it.shared) ? ip.t1s : t1 * (kPair ? 2 : 1);
-          // test only: the first routed down item waits for one gate/up tile
-          // more than exist, so its wait runs out (the timeout path)
-          if (starve_first_down && item == ip.S * ip.t1s + ip.r1) ++need;
-          bool ok = ld_acquire(done) >= need;
-          if (!ok) {
-            const uint64_t t0 = global_timer_ns();
-            while (!(ok = ld_acquire(done) >= need)) {
-              if (*abort) break;
-              if (global_timer_ns() - t0 > timeout_ns) {
-                raise_abort(abort, ws, SLIMWISE_DEVERR_DEPENDENCY_TIMEOUT);
-                break;
-              }
-              __nanosleep(128);
-            }
-          }
-          if (!ok) break;
-          fence_proxy_async_global();
-        }
-        // bytes the stage barrier expects: for a pair, both CTAs' copies
-        const uint32_t stage_tx =
-            kPair ? (uint32_t)(2 * kATileBytes + it.n16 * kTokBox * kBlockK * 2)
-                  : (uint32_t)(halves * kATileBytes + kTokBox * (box_m + 1) * kBlockK * 2);
-        bool ok = true;
-        for (int kc = 0; kc < nk; ++kc) {
-          if (!mbar_wait_bounded(empty_bar(stage), phase ^ 1u, abort, timeout_ns)) {
-            if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-            ok = false;
-            break;
-          }
-          const int x = kc * kBlockK;
-          const uint32_t a = smem_base + (uint32_t)(stage * plan.stage_bytes);
+        const int x = kc * kBlockK;
+        const uint32_t a = smem_base + (uint32_t)(stage * plan.stage_bytes);
+        if (elect_one()) {
           if (kPair && !lead) {
             const uint32_t lb = mapa_shared(full_bar(stage), 0u);
             tma_load_w_pair(a, amap, lb, x, unit0, expert, pol_w);
@@ -646,14 +654,17 @@ __global__ void __maxnreg__(128)
             }
             tma_load_2d(a + (uint32_t)plan.a_bytes, bmap, full_bar(stage), x, tok_row, pol_x);
           }
-          ++issued;
-          if (++stage == stages) {
-            stage = 0;
-            phase ^= 1u;
-          }
         }
-        if (!ok) break;
+        __syncwarp();
+        ++issued;
+        if (++stage == stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
+      if (!ok) break;
+    }
+    if (lane == 0) {
       if (kPair && !lead) {
         // The second CTA's stages complete on the first CTA's barriers; the
         // first CTA's MMAs read them and their commits arrive here.  Wait
@@ -672,77 +683,61 @@ __global__ void __maxnreg__(128)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && kPair && !lead) {
+    // the whole warp runs the loop here too
+    int stage = 0;
+    uint32_t phase = 0;
+    int slot = 0;
+    uint32_t rphase = 0;
+    int n_consumed = 0;
+    auto all_ok = [&](bool ok) {
+      if (!ok && !*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
+      return __all_sync(0xFFFFFFFFu, ok) != 0;
+    };
+    for (int local = 0;; ++local) {
+      if (!all_ok(mbar_wait_bounded(itf_bar(slot), rphase, abort, timeout_ns))) break;
+      const int item = __shfl_sync(0xFFFFFFFFu, ring[slot].item, 0);
+      const int form = __shfl_sync(0xFFFFFFFFu, ring[slot].form, 0);
+      const int n16 = (__shfl_sync(0xFFFFFFFFu, ring[slot].n, 0) + 15) >> 4;
+      if (lane == 0) mbar_arrive(ite_bar(slot));
+      if (++slot == kItemRing) {
+        slot = 0;
+        rphase ^= 1u;
+      }
+      if (item >= total) break;
       // the second CTA of a pair issues no MMA: it only keeps its item ring
       // moving
-      int slot = 0;
-      uint32_t rphase = 0;
-      for (;;) {
-        if (!mbar_wait_bounded(itf_bar(slot), rphase, abort, timeout_ns)) {
-          if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-          break;
-        }
-        const int item = ring[slot].item;
-        mbar_arrive(ite_bar(slot));
-        if (++slot == kItemRing) {
-          slot = 0;
-          rphase ^= 1u;
-        }
-        if (item >= total) break;
-      }
-    } else if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int slot = 0;
-      uint32_t rphase = 0;
-      int n_consumed = 0;
-      bool issued_any = false;
-      for (int local = 0;; ++local) {
-        if (!mbar_wait_bounded(itf_bar(slot), rphase, abort, timeout_ns)) {
-          if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-          break;
-        }
-        const ItemSlot it = ring[slot];
-        mbar_arrive(ite_bar(slot));
-        if (++slot == kItemRing) {
-          slot = 0;
-          rphase ^= 1u;
-        }
-        if (it.item >= total) break;
-        const bool down = (it.form & 1) != 0, shared = (it.form & 2) != 0;
-        const int n16 = (it.n + 15) >> 4;
-        const int b = local & 1;
-        const uint32_t use = (uint32_t)(local >> 1);
-        const bool freed =
-            kPair ? mbar_wait_cluster_bounded(acce_bar(b), (use & 1u) ^ 1u, abort, timeout_ns)
-                  : mbar_wait_bounded(acce_bar(b), (use & 1u) ^ 1u, abort, timeout_ns);
-        if (!freed) {
-          if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
+      if (kPair && !lead) continue;
+      const bool down = (form & 1) != 0, shared = (form & 2) != 0;
+      const int b = local & 1;
+      const uint32_t use = (uint32_t)(local >> 1);
+      const bool freed =
+          kPair ? mbar_wait_cluster_bounded(acce_bar(b), (use & 1u) ^ 1u, abort, timeout_ns)
+                : mbar_wait_bounded(acce_bar(b), (use & 1u) ^ 1u, abort, timeout_ns);
+      if (!all_ok(freed)) break;
+      tc_fence_after();
+      // half h of the item: A = the stage's weight rows [128 h, 128 h + 128),
+      // D = columns [h tok_chunk, ...) of the buffer; B = the token rows.
+      // A pair runs one M = 256 MMA: A rows 128-255 and B rows N/2.. are the
+      // second CTA's, at the same shared-memory offsets.
+      const uint32_t d_tmem = tmem_base + (uint32_t)(b * nb_cols);
+      const uint32_t idesc = idesc_bf16_f32(kPair ? 2 * kTileRows : kTileRows, n16 * kTokBox);
+      const int halves = (kShared && shared) ? 1 : wmul;
+      const int inner = (kShared && shared) ? d.Is : d.I;
+      const int nk = down ? inner / kBlockK : d.H / kBlockK;
+      bool ok = true;
+      for (int kc = 0; kc < nk; ++kc) {
+        if (!all_ok(mbar_wait_bounded(full_bar(stage), phase, abort, timeout_ns))) {
+          ok = false;
           break;
         }
         tc_fence_after();
-        // half h of the item: A = the stage's weight rows [128 h, 128 h + 128),
-        // D = columns [h tok_chunk, ...) of the buffer; B = the token rows.
-        // A pair runs one M = 256 MMA: A rows 128-255 and B rows N/2.. are the
-        // second CTA's, at the same shared-memory offsets.
-        const uint32_t d_tmem = tmem_base + (uint32_t)(b * nb_cols);
-        const uint32_t idesc = idesc_bf16_f32(kPair ? 2 * kTileRows : kTileRows, n16 * kTokBox);
-        const int halves = (kShared && shared) ? 1 : wmul;
-        const int inner = (kShared && shared) ? d.Is : d.I;
-        const int nk = down ? inner / kBlockK : d.H / kBlockK;
-        bool ok = true;
-        for (int kc = 0; kc < nk; ++kc) {
-          if (!mbar_wait_bounded(full_bar(stage), phase, abort, timeout_ns)) {
-            if (!*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
-            ok = false;
-            break;
-          }
-          tc_fence_after();
 #ifdef SLIMWISE_TRACE
-          if (blockIdx.x == 0 && n_consumed == 0) trace_stamp(ws, tr_step, kTrFfnFirstData);
+        if (blockIdx.x == 0 && lane == 0 && n_consumed == 0) trace_stamp(ws, tr_step, kTrFfnFirstData);
 #endif
-          const uint32_t a = smem_base + (uint32_t)(stage * plan.stage_bytes);
-          const uint32_t bs = a + (uint32_t)plan.a_bytes;
+        const uint32_t a = smem_base + (uint32_t)(stage * plan.stage_bytes);
+        const uint32_t bs = a + (uint32_t)plan.a_bytes;
+        ++n_consumed;
+        if (elect_one()) {
           if constexpr (kPair) {
 #pragma unroll
             for (int kk = 0; kk < kBlockK / 16; ++kk)
@@ -759,22 +754,27 @@ __global__ void __maxnreg__(128)
             }
             tc_commit(empty_bar(stage));
           }
-          issued_any = true;
-          *consumed = ++n_consumed;
-          if (++stage == stages) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          *consumed = n_consumed;
         }
-        if (!ok) break;
+        __syncwarp();
+        if (++stage == stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      if (!ok) break;
+      if (elect_one()) {
         if constexpr (kPair) tc_commit_pair(accf_bar(b), (uint16_t)3);
         else tc_commit(accf_bar(b));
       }
-      if (*abort && issued_any) {
+      __syncwarp();
+    }
+    if (__any_sync(0xFFFFFFFFu, *abort != 0) && n_consumed > 0) {
+      if (elect_one()) {
         if constexpr (kPair) tc_commit_pair(drain_bar, (uint16_t)1);
         else tc_commit(drain_bar);
-        mbar_wait_timeout(drain_bar, 0, 10000000ull);
       }
+      mbar_wait_timeout(drain_bar, 0, 10000000ull);
     }
     __syncwarp();
   } else {
@@ -812,7 +812,7 @@ __global__ void __maxnreg__(128)
       const int cols = ((it.n + 15) >> 4) * kTokBox;  // accumulator columns
       // 128-row tile of the item that TMEM half hh holds: half hh of a wide
       // item, the CTA's own half of a pair item
-      const int tile0 = shared ? it.tile : it.tile * tiles_per_item + (kPair ? (int)crank : 0);
+      const int tile0 = it.tile * tiles_per_item + (kPair ? (int)crank : 0);
       // the accumulator is free once its last columns have been loaded
       auto release = [&]() {
         tc_fence_before();
@@ -955,12 +955,13 @@ int ffn_stages_for(int tok_chunk, int wide, int pair, size_t smem_limit) {
 }
 
 // Clusters of two FFN CTAs that can be resident at once (the pairs' SMs must
-// share a GPC), kept per device and shared-memory size.
+// share a GPC), kept per kernel, device and shared-memory size.
 cudaError_t pair_clusters_resident(const void *kernel, size_t smem, int dev, int *n) {
+  thread_local const void *last_kernel = nullptr;
   thread_local int last_dev = -1;
   thread_local size_t last_smem = 0;
   thread_local int last_n = 0;
-  if (dev == last_dev && smem == last_smem) {
+  if (kernel == last_kernel && dev == last_dev && smem == last_smem) {
     *n = last_n;
     return cudaSuccess;
   }
@@ -979,6 +980,7 @@ cudaError_t pair_clusters_resident(const void *kernel, size_t smem, int dev, int
   cudaError_t err = cudaOccupancyMaxActiveClusters(&c, kernel, &cfg);
   if (err != cudaSuccess) return err;
   if (c < 1) return cudaErrorInvalidConfiguration;
+  last_kernel = kernel;
   last_dev = dev;
   last_smem = smem;
   last_n = c;
@@ -1013,10 +1015,12 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
   if (d.wide && (d.Is > 0 || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0 ||
                  d.tok_chunk > 128))
     return cudaErrorInvalidValue;
-  // pair items likewise, and never together with wide ones
-  if (d.pair && (d.wide || d.Is > 0 || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0))
+  // pair items on whole 256-row tiles too, and never together with wide ones
+  if (d.pair && (d.wide || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0 ||
+                 d.Is % (2 * kGateRows) != 0))
     return cudaErrorInvalidValue;
-  auto kernel = d.Is > 0   ? expert_ffn_kernel<true, false, false>
+  auto kernel = d.Is > 0 ? (d.pair ? expert_ffn_kernel<true, false, true>
+                                   : expert_ffn_kernel<true, false, false>)
                 : d.pair ? expert_ffn_kernel<false, false, true>
                 : d.wide ? expert_ffn_kernel<false, true, false>
                          : expert_ffn_kernel<false, false, false>;

@@ -110,7 +110,7 @@ __device__ __forceinline__ void publish_groups(const Dims &d, const Ws &ws, cons
   if (gtid == 0) {
     const int t1_items = gate_up_tiles(d);
     const int t2_items = down_tiles(d);
-    const int t1s_items = d.Is / kGateRows;
+    const int t1s_items = shared_gate_up_tiles(d);
     ws.offsets[E] = offs[E];
     ws.ctrl[kCtrlUnionSize] = U;
     ws.ctrl[kCtrlNumEntries] = n_se + n_entries;

@@ -141,7 +141,8 @@ Dims make_dims(const slimwise_moe_shape *s, int32_t top_k, int32_t m_ret, int32_
 
 // The caller's choice of work-item form (slimwise_decode_opts.ffn_items).
 void apply_item_form(Dims *d, int32_t form) {
-  const bool can_pair = d->Is == 0 && d->I % (2 * kGateRows) == 0 && d->H % (2 * kTileRows) == 0;
+  const bool can_pair = d->I % (2 * kGateRows) == 0 && d->H % (2 * kTileRows) == 0 &&
+                        d->Is % (2 * kGateRows) == 0;
   if (form > 0 && can_pair) {
     d->pair = 1;
     d->wide = 0;
