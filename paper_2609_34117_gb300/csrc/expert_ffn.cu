@@ -107,6 +107,12 @@ __host__ __device__ inline FfnSmem ffn_smem_plan(int tok_chunk, int stages, int 
 // of the next): at most 512 columns, so wide items need tok_chunk <= 128.
 __host__ __device__ inline int ffn_acc_cols(const Dims &d) { return (d.wide ? 2 : 1) * d.tok_chunk; }
 
+// Claiming ahead pays from this token chunk on: a full-pool layer of 8192
+// tokens 849 -> 830 us, 4001 tokens 468 -> 461, 2048 tokens (chunk 176) 302 ->
+// 298; nothing at chunks of 16-112, and 3 us lost at B = 1, where CTAs have
+// two items each.
+constexpr int kAheadMinChunk = 128;
+
 struct Item {
   int down;      // 0: gate/up, 1: down
   int shared;    // 1: the shared expert (token order), 0: a routed expert
@@ -340,7 +346,14 @@ __device__ __forceinline__ void raise_abort(volatile int *abort, Ws &ws, int bit
 // the MMA commits arrive on the stage and accumulator barriers of both CTAs;
 // each CTA's epilogue reads its own TMEM lanes (its 128 weight rows) and
 // releases the accumulator to the first CTA's MMA issuer.
-template <bool kShared, bool kWide, bool kPair>
+//
+// kAhead: a CTA claims its next item when the current one starts, and fetches
+// its work entry, and looks whether a down item's activations are complete,
+// while the current one still streams, so that an item boundary costs none of
+// these round trips.  Large token chunks only (kAheadMinChunk): their items
+// are many per CTA, and an unstarted item held back at the end of the launch
+// is a small share of it.
+template <bool kShared, bool kWide, bool kPair, bool kAhead>
 __global__ void __maxnreg__(128)
     expert_ffn_kernel(const __grid_constant__ FfnMaps maps, Dims d, Ws ws,
                       __nv_bfloat16 *__restrict__ out,
@@ -349,6 +362,7 @@ __global__ void __maxnreg__(128)
                       uint64_t timeout_ns,
                       int starve_first_down) {
   static_assert(!(kPair && kWide), "a pair item is a 128-row tile in each CTA");
+  static_assert(!(kAhead && kPair), "a pair's items are handed from CTA to CTA");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -521,9 +535,29 @@ __global__ void __maxnreg__(128)
       if (!ok && !*abort) raise_abort(abort, ws, SLIMWISE_DEVERR_PIPELINE_TIMEOUT);
       return __all_sync(0xFFFFFFFFu, ok) != 0;
     };
-    for (;;) {
+    // work entry of an item, uniform over the warp
+    auto fetch = [&](int i) {
+      Item r = {};
+      if (i < total) r = decode_item<kShared>(i, ip, ws);
+      r.expert = __shfl_sync(0xFFFFFFFFu, r.expert, 0);
+      r.slot_base = __shfl_sync(0xFFFFFFFFu, r.slot_base, 0);
+      r.n = __shfl_sync(0xFFFFFFFFu, r.n, 0);
+      return r;
+    };
+    // gate/up tiles an entry's down items wait for
+    auto tiles_needed = [&](const Item &i) {
+      return ((kShared && i.shared) ? ip.t1s : t1) * (kPair ? 2 : 1);
+    };
+    // kAhead: the next item (claimed: on lane 0 until it is fetched), its
+    // entry, and whether its activations were seen complete
+    int next = 0;
+    Item next_it = {};
+    bool next_ready = false;
+    for (bool started = false;; started = true) {
       int item = 0;
-      if (!kPair || lead) {
+      if (kAhead && started) {
+        item = __any_sync(0xFFFFFFFFu, *abort != 0) ? kNoItem : next;
+      } else if (!kPair || lead) {
         if (lane == 0) {
           item = first ? item0 : n_first + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
           if (*abort) item = kNoItem;
@@ -550,11 +584,8 @@ __global__ void __maxnreg__(128)
       }
       item = __shfl_sync(0xFFFFFFFFu, item, 0);
       if (!all_ok(mbar_wait_bounded(ite_bar(slot), rphase ^ 1u, abort, timeout_ns))) break;
-      Item it = {};
-      if (item < total) it = decode_item<kShared>(item, ip, ws);
-      it.expert = __shfl_sync(0xFFFFFFFFu, it.expert, 0);
-      it.slot_base = __shfl_sync(0xFFFFFFFFu, it.slot_base, 0);
-      it.n = __shfl_sync(0xFFFFFFFFu, it.n, 0);
+      const Item it = (kAhead && started) ? next_it : fetch(item);
+      const bool ready = kAhead && started && next_ready;
       if (lane == 0) {
         ItemSlot sl = {};
         sl.item = item;
@@ -602,10 +633,11 @@ __global__ void __maxnreg__(128)
         bmap = it.down ? (const void *)&maps.act[box_m] : (const void *)&maps.xp[box_m];
         expert = it.expert;
       }
-      if (it.down) {
+      if (kAhead && lane == 0) next = n_first + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
+      if (it.down && !ready) {
         // the entry's activations must be complete: all its gate/up tiles
         const int *done = &ws.entry_done[it.entry];
-        int need = ((kShared && it.shared) ? ip.t1s : t1) * (kPair ? 2 : 1);
+        int need = tiles_needed(it);
         // test only: the first routed down item waits for one gate/up tile
         // more than exist, so its wait runs out (the timeout path)
         if (starve_first_down && item == ip.S * ip.t1s + ip.r1) ++need;
@@ -631,6 +663,16 @@ __global__ void __maxnreg__(128)
                 : (uint32_t)(halves * kATileBytes + n16 * kTokBox * kBlockK * 2);
       bool ok = true;
       for (int kc = 0; kc < nk; ++kc) {
+        if (kAhead && kc == (2 * nk) / 3) {
+          next = __shfl_sync(0xFFFFFFFFu, next, 0);
+          next_it = fetch(next);
+          next_ready = false;
+          if (next < total && next_it.down && !starve_first_down) {
+            next_ready = __all_sync(0xFFFFFFFFu, ld_acquire(&ws.entry_done[next_it.entry]) >=
+                                                     tiles_needed(next_it)) != 0;
+            if (next_ready) fence_proxy_async_global();
+          }
+        }
         if (!all_ok(mbar_wait_bounded(empty_bar(stage), phase ^ 1u, abort, timeout_ns))) {
           ok = false;
           break;
@@ -1019,11 +1061,14 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
   if (d.pair && (d.wide || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0 ||
                  d.Is % (2 * kGateRows) != 0))
     return cudaErrorInvalidValue;
-  auto kernel = d.Is > 0 ? (d.pair ? expert_ffn_kernel<true, false, true>
-                                   : expert_ffn_kernel<true, false, false>)
-                : d.pair ? expert_ffn_kernel<false, false, true>
-                : d.wide ? expert_ffn_kernel<false, true, false>
-                         : expert_ffn_kernel<false, false, false>;
+  const bool ahead = d.tok_chunk >= kAheadMinChunk;
+  auto kernel = d.Is > 0 ? (d.pair  ? expert_ffn_kernel<true, false, true, false>
+                            : ahead ? expert_ffn_kernel<true, false, false, true>
+                                    : expert_ffn_kernel<true, false, false, false>)
+                : d.pair  ? expert_ffn_kernel<false, false, true, false>
+                : d.wide  ? expert_ffn_kernel<false, true, false, false>
+                : ahead   ? expert_ffn_kernel<false, false, false, true>
+                          : expert_ffn_kernel<false, false, false, false>;
   err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int tmem_cols = 32;
