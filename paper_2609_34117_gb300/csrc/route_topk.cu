@@ -177,6 +177,131 @@ __device__ __forceinline__ void take_winner(uint32_t whi, uint32_t wlo, int j, i
   }
 }
 
+// The grid's last CTA reports bad and repeated retained ids and resets the
+// error word of this call.
+__device__ __forceinline__ void report_retained(const int32_t *__restrict__ retained, const Dims &d,
+                                                const Ws &ws) {
+  __shared__ uint32_t seen[kMaxExperts / 32];
+  __shared__ int bad;
+  for (int i = threadIdx.x; i < kMaxExperts / 32; i += blockDim.x) seen[i] = 0;
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+  for (int r = threadIdx.x; r < d.m_ret; r += blockDim.x) {
+    int e = retained ? retained[r] : r;
+    if (e < 0 || e >= d.E) {
+      atomicOr(&bad, SLIMWISE_DEVERR_BAD_RETAINED);
+    } else {
+      uint32_t bit = 1u << (e & 31);
+      if (atomicOr(&seen[e >> 5], bit) & bit)
+        atomicOr(&bad, SLIMWISE_DEVERR_DUPLICATE_RETAINED);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) ws.ctrl[kCtrlErr] = bad;
+}
+
+// Top-k and gates of token t, by one warp, from its logits z[0, m') over the
+// retained ids: NC candidates per lane in registers (m' <= 32 NC), or NC = 0
+// for larger pools.
+template <int NC>
+__device__ __forceinline__ void topk_token(const float *z, const int32_t *ids, const Dims &d,
+                                           const Ws &ws, int t, int lane) {
+  const int m = d.m_ret, k = d.k;
+  float my_z = 0.0f;
+  int my_e = 0;
+  if constexpr (NC > 0) {
+    // this lane's candidates r = lane + 32 i (i < NC) as 64-bit keys
+    // (order-preserving logit bits, complemented id; 0 = none), kept sorted
+    // descending in registers -- every index below is a compile-time one;
+    // all loads are issued before any is used
+    float zc[NC];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int r = lane + 32 * i;
+      if (r < m) {
+        zc[i] = z[r];
+      }
+    }
+    unsigned long long key[NC];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int r = lane + 32 * i;
+      key[i] = r < m ? ((unsigned long long)logit_order_bits(zc[i]) << 32) |
+                           (unsigned long long)(0xFFFFFFFFu - (uint32_t)ids[r])
+                     : 0ull;
+#pragma unroll
+      for (int j = i; j > 0; --j)
+        if (key[j] > key[j - 1]) {
+          const unsigned long long tmp = key[j];
+          key[j] = key[j - 1];
+          key[j - 1] = tmp;
+        }
+    }
+    // k rounds: the warp's largest head key wins and its lane pops it
+    for (int j = 0; j < k; ++j) {
+      const unsigned long long mine = key[0];
+      const uint32_t hi = (uint32_t)(mine >> 32), lo = (uint32_t)mine;
+      const uint32_t whi = __reduce_max_sync(0xFFFFFFFFu, hi);
+      const uint32_t wlo = __reduce_max_sync(0xFFFFFFFFu, hi == whi ? lo : 0u);
+      const unsigned long long win = ((unsigned long long)whi << 32) | wlo;
+      // pop every copy of the winner (repeated retained ids give equal keys)
+      for (int pops = 0; pops < NC && key[0] == win && win != 0ull; ++pops) {
+#pragma unroll
+        for (int i = 0; i + 1 < NC; ++i) key[i] = key[i + 1];
+        key[NC - 1] = 0ull;
+      }
+      take_winner(whi, wlo, j, lane, ids, d, my_z, my_e);
+    }
+  } else {
+    // large pools: the lane's candidates sorted in a local array
+    unsigned long long key[kMaxExperts / 32];
+    int nc = 0;
+    for (int r0 = lane; r0 < m; r0 += 128) {
+      float zc[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + 32 * u;
+        if (r < m) {
+          zc[u] = z[r];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + 32 * u;
+        if (r < m) {
+          const unsigned long long kv = ((unsigned long long)logit_order_bits(zc[u]) << 32) |
+                                        (unsigned long long)(0xFFFFFFFFu - (uint32_t)ids[r]);
+          int i = nc++;
+          while (i > 0 && key[i - 1] < kv) {
+            key[i] = key[i - 1];
+            --i;
+          }
+          key[i] = kv;
+        }
+      }
+    }
+    int head = 0;
+    for (int j = 0; j < k; ++j) {
+      const unsigned long long mine = head < nc ? key[head] : 0ull;
+      const uint32_t hi = (uint32_t)(mine >> 32), lo = (uint32_t)mine;
+      const uint32_t whi = __reduce_max_sync(0xFFFFFFFFu, hi);
+      const uint32_t wlo = __reduce_max_sync(0xFFFFFFFFu, hi == whi ? lo : 0u);
+      const unsigned long long win = ((unsigned long long)whi << 32) | wlo;
+      while (head < nc && key[head] == win) ++head;
+      take_winner(whi, wlo, j, lane, ids, d, my_z, my_e);
+    }
+  }
+  // g_j = exp(z_j - z_1) / sum_j' exp(z_j' - z_1), the sum in j order.
+  const float z1 = __shfl_sync(0xFFFFFFFFu, my_z, 0);
+  const float w = (lane < k) ? expf(my_z - z1) : 0.0f;
+  float denom = 0.0f;
+  for (int j = 0; j < k; ++j) denom += __shfl_sync(0xFFFFFFFFu, w, j);
+  if (lane < k) {
+    ws.topk_idx[(size_t)t * k + lane] = my_e;
+    ws.topk_gate[(size_t)t * k + lane] = w / denom;
+  }
+}
+
 // TB tokens per cluster; NC candidates per lane in the register top-k
 // (m' <= 32 NC), or NC = 0 for the general top-k of larger pools.
 template <int TB, int NC>
@@ -189,7 +314,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2)
   extern __shared__ __align__(16) unsigned char smem[];
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank();
-  const int H = d.H, m = d.m_ret, k = d.k;
+  const int H = d.H, m = d.m_ret;
   const int slice = (m + kClusterCtas - 1) / kClusterCtas;
   constexpr int kOwn = (TB + kClusterCtas - 1) / kClusterCtas;  // tokens whose top-k a CTA runs
   XT *xs = reinterpret_cast<XT *>(smem);
@@ -227,32 +352,12 @@ __global__ void __launch_bounds__(kRouteThreads, 2)
   const int nt = min(TB, d.B - t0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // Retained ids, clamped into [0, E) so a bad id cannot fault; the grid's
-  // last CTA also reports bad and repeated ids and resets the error word of
-  // this call.
+  // Retained ids, clamped into [0, E) so a bad id cannot fault.
   for (int r = threadIdx.x; r < m; r += blockDim.x) {
     int e = retained ? retained[r] : r;
     ids[r] = min(max(e, 0), d.E - 1);
   }
-  if (blockIdx.x == gridDim.x - 1) {
-    __shared__ uint32_t seen[kMaxExperts / 32];
-    __shared__ int bad;
-    for (int i = threadIdx.x; i < kMaxExperts / 32; i += blockDim.x) seen[i] = 0;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    for (int r = threadIdx.x; r < m; r += blockDim.x) {
-      int e = retained ? retained[r] : r;
-      if (e < 0 || e >= d.E) {
-        atomicOr(&bad, SLIMWISE_DEVERR_BAD_RETAINED);
-      } else {
-        uint32_t bit = 1u << (e & 31);
-        if (atomicOr(&seen[e >> 5], bit) & bit)
-          atomicOr(&bad, SLIMWISE_DEVERR_DUPLICATE_RETAINED);
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) ws.ctrl[kCtrlErr] = bad;
-  }
+  if (blockIdx.x == gridDim.x - 1) report_retained(retained, d, ws);
 
   // Hidden rows of the cluster's tokens (16-byte vectors of 8 bf16), zero
   // past the batch.  Each thread issues TB loads before storing any, so the
@@ -393,102 +498,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2)
   // Top-k and gates: token tw of the cluster is handled by warp tw / 8 of the
   // cluster's CTA tw % 8, so the tokens' top-k run side by side.
   const int tw = warp * kClusterCtas + crank;
-  if (tw < nt) {
-    const int t = t0 + tw;
-    float my_z = 0.0f;
-    int my_e = 0;
-    if constexpr (NC > 0) {
-      // this lane's candidates r = lane + 32 i (i < NC) as 64-bit keys
-      // (order-preserving logit bits, complemented id; 0 = none), kept sorted
-      // descending in registers -- every index below is a compile-time one;
-      // all loads are issued before any is used
-      float zc[NC];
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const int r = lane + 32 * i;
-        if (r < m) {
-          zc[i] = zs[(size_t)warp * m + r];
-        }
-      }
-      unsigned long long key[NC];
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const int r = lane + 32 * i;
-        key[i] = r < m ? ((unsigned long long)logit_order_bits(zc[i]) << 32) |
-                             (unsigned long long)(0xFFFFFFFFu - (uint32_t)ids[r])
-                       : 0ull;
-#pragma unroll
-        for (int j = i; j > 0; --j)
-          if (key[j] > key[j - 1]) {
-            const unsigned long long tmp = key[j];
-            key[j] = key[j - 1];
-            key[j - 1] = tmp;
-          }
-      }
-      // k rounds: the warp's largest head key wins and its lane pops it
-      for (int j = 0; j < k; ++j) {
-        const unsigned long long mine = key[0];
-        const uint32_t hi = (uint32_t)(mine >> 32), lo = (uint32_t)mine;
-        const uint32_t whi = __reduce_max_sync(0xFFFFFFFFu, hi);
-        const uint32_t wlo = __reduce_max_sync(0xFFFFFFFFu, hi == whi ? lo : 0u);
-        const unsigned long long win = ((unsigned long long)whi << 32) | wlo;
-        // pop every copy of the winner (repeated retained ids give equal keys)
-        for (int pops = 0; pops < NC && key[0] == win && win != 0ull; ++pops) {
-#pragma unroll
-          for (int i = 0; i + 1 < NC; ++i) key[i] = key[i + 1];
-          key[NC - 1] = 0ull;
-        }
-        take_winner(whi, wlo, j, lane, ids, d, my_z, my_e);
-      }
-    } else {
-      // large pools: the lane's candidates sorted in a local array
-      unsigned long long key[kMaxExperts / 32];
-      int nc = 0;
-      for (int r0 = lane; r0 < m; r0 += 128) {
-        float zc[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + 32 * u;
-          if (r < m) {
-            zc[u] = zs[(size_t)warp * m + r];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int r = r0 + 32 * u;
-          if (r < m) {
-            const unsigned long long kv = ((unsigned long long)logit_order_bits(zc[u]) << 32) |
-                                          (unsigned long long)(0xFFFFFFFFu - (uint32_t)ids[r]);
-            int i = nc++;
-            while (i > 0 && key[i - 1] < kv) {
-              key[i] = key[i - 1];
-              --i;
-            }
-            key[i] = kv;
-          }
-        }
-      }
-      int head = 0;
-      for (int j = 0; j < k; ++j) {
-        const unsigned long long mine = head < nc ? key[head] : 0ull;
-        const uint32_t hi = (uint32_t)(mine >> 32), lo = (uint32_t)mine;
-        const uint32_t whi = __reduce_max_sync(0xFFFFFFFFu, hi);
-        const uint32_t wlo = __reduce_max_sync(0xFFFFFFFFu, hi == whi ? lo : 0u);
-        const unsigned long long win = ((unsigned long long)whi << 32) | wlo;
-        while (head < nc && key[head] == win) ++head;
-        take_winner(whi, wlo, j, lane, ids, d, my_z, my_e);
-      }
-    }
-    // g_j = exp(z_j - z_1) / sum_j' exp(z_j' - z_1), the sum in j order.
-    const float z1 = __shfl_sync(0xFFFFFFFFu, my_z, 0);
-    const float w = (lane < k) ? expf(my_z - z1) : 0.0f;
-    float denom = 0.0f;
-    for (int j = 0; j < k; ++j) denom += __shfl_sync(0xFFFFFFFFu, w, j);
-    if (lane < k) {
-      ws.topk_idx[(size_t)t * k + lane] = my_e;
-      ws.topk_gate[(size_t)t * k + lane] = w / denom;
-    }
-  }
+  if (tw < nt) topk_token<NC>(zs + (size_t)warp * m, ids, d, ws, t0 + tw, lane);
 #ifdef SLIMWISE_TRACE
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     trace_stamp(ws, tr_step, kTrRouteEnd);
@@ -538,9 +548,238 @@ cudaError_t launch_route_nc(const __nv_bfloat16 *hidden, const float *router_w,
   return launch_route_tb<TB, 0>(hidden, router_w, retained, d, ws, pdl, stream);
 }
 
+// --------------------------------------------------------------------------
+// Large batches
+// --------------------------------------------------------------------------
+// A cluster of the kernel above reads the whole router for its 16 tokens and
+// spends more issue slots on loads and conversions than on multiply-adds.
+// There (route_tiled says where) the logits are a tiled product on the fp32
+// units, in the same canonical order, and a second kernel runs the top-k:
+//   route_logits_kernel  32 tokens x 16 retained experts per CTA, the K range
+//                        streamed in 128-wide chunks through a 4-stage
+//                        cp.async ring.  Lane l of every warp holds partial
+//                        sum l of its 8 tokens x 16 experts (128 registers),
+//                        so 24 shared-memory loads feed 256 packed
+//                        multiply-adds a chunk; the butterfly over the lanes
+//                        runs as a transposing reduction (each step halves
+//                        the values a lane carries: 124 shuffles for 128
+//                        logits, not 640).  z goes to global scratch.
+//   route_select_kernel  one warp per token over z.
+// Bound by the fp32 multiply-adds: 8192 tokens x 256 experts run at 73 % of
+// the 32 T/s that a register-only loop reaches here, two CTAs of 4 warps per
+// SM (one of 8 warps: 57 %, all of them waiting for each chunk together;
+// 16 tokens x 8 experts per warp: 70 %).
+constexpr int kTileTok = 32;
+constexpr int kTileRow = 16;
+constexpr int kTileThreads = 128;
+constexpr int kTileStages = 4;
+constexpr int kWarpTok = 8;    // tokens of one warp (4 warps: the tile's 32)
+constexpr int kWarpRow = 16;   // experts of one warp
+constexpr int kTileXBytes = kTileTok * 128 * 2;
+constexpr int kTileWBytes = kTileRow * 128 * 4;
+constexpr int kTileSmem = kTileStages * (kTileXBytes + kTileWBytes);
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes)
+               : "memory");
+}
+
+// One step of the transposing reduction: of 2 n values a lane keeps n, those
+// of its half, each added to its partner's.
+template <int kOff, int kN, int kSize>
+__device__ __forceinline__ void reduce_step(float (&a)[kSize], int lane) {
+  const bool upper = (lane & kOff) != 0;
+#pragma unroll
+  for (int i = 0; i < kN; ++i) {
+    const float give = upper ? a[i] : a[i + kN], keep = upper ? a[i + kN] : a[i];
+    a[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, kOff);
+  }
+}
+
+__global__ void __launch_bounds__(kTileThreads, 2)
+    route_logits_kernel(const __nv_bfloat16 *__restrict__ hidden,
+                        const float *__restrict__ router_w,
+                        const int32_t *__restrict__ retained, Dims d, Ws ws,
+                        float *__restrict__ z) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  pdl_wait_primary();
+  pdl_launch_dependents();
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    const int tr_step = ws.ctrl[kCtrlTraceStep];
+    trace_stamp(ws, tr_step, kTrRouteStart);
+    reinterpret_cast<uint64_t *>(ws.ctrl + kCtrlWords)[(tr_step & (kTraceSteps - 1)) * kTrSlots + kTrFfnEnd] = 0;
+  }
+#endif
+  const int H = d.H, m = d.m_ret, nchunks = H / 128;
+  const int t0 = blockIdx.x * kTileTok, r0 = blockIdx.y * kTileRow;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t xs = smem_u32(smem), wsm = xs + kTileStages * kTileXBytes;
+
+  // this thread's 16-byte vectors of a chunk: four of the hidden rows (rows
+  // tid / 16 + 8 u; tokens past the batch are zero) and four of the router
+  // rows (rows warp + 4 u; rows past the pool repeat its last one and are
+  // dropped at the end)
+  const int xrow = tid >> 4, xcol = tid & 15;
+  const __nv_bfloat16 *xsrc[4];
+  const float *wsrc[4];
+  uint32_t xbytes[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int t = t0 + xrow + 8 * u;
+    xbytes[u] = t < d.B ? 16u : 0u;
+    xsrc[u] = hidden + (size_t)(t < d.B ? t : 0) * H + xcol * 8;
+    const int r = min(r0 + warp + 4 * u, m - 1);
+    const int e = min(max(retained ? __ldg(retained + r) : r, 0), d.E - 1);
+    wsrc[u] = router_w + (size_t)e * H + lane * 4;
+  }
+  auto load_chunk = [&](int c) {
+    const int st = c % kTileStages;
+    const uint32_t xd = xs + st * kTileXBytes + xrow * 256 + xcol * 16;
+    const uint32_t wd = wsm + st * kTileWBytes + warp * 512 + lane * 16;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      cp_async16(xd + u * 8 * 256, xsrc[u] + c * 128, xbytes[u]);
+      cp_async16(wd + u * 4 * 512, wsrc[u] + c * 128, 16u);
+    }
+  };
+#pragma unroll
+  for (int c = 0; c < kTileStages - 1; ++c) {
+    if (c < nchunks) load_chunk(c);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+
+  float acc[kWarpRow][kWarpTok];
+#pragma unroll
+  for (int r = 0; r < kWarpRow; ++r)
+#pragma unroll
+    for (int t = 0; t < kWarpTok; ++t) acc[r][t] = 0.0f;
+  const unsigned char *xw = smem + (size_t)warp * kWarpTok * 256 + lane * 8;
+  const unsigned char *ww = smem + kTileStages * kTileXBytes + lane * 16;
+  for (int c = 0; c < nchunks; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kTileStages - 2) : "memory");
+    __syncthreads();  // chunk c is here, and chunk c - 1 has been read by all
+    if (c + kTileStages - 1 < nchunks) load_chunk(c + kTileStages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int st = c % kTileStages;
+    float x[4][kWarpTok];
+#pragma unroll
+    for (int t = 0; t < kWarpTok; ++t) {
+      const uint2 v = *reinterpret_cast<const uint2 *>(xw + st * kTileXBytes + t * 256);
+      x[0][t] = __uint_as_float(v.x << 16);
+      x[1][t] = __uint_as_float(v.x & 0xFFFF0000u);
+      x[2][t] = __uint_as_float(v.y << 16);
+      x[3][t] = __uint_as_float(v.y & 0xFFFF0000u);
+    }
+#pragma unroll
+    for (int r = 0; r < kWarpRow; ++r) {
+      const float4 w = *reinterpret_cast<const float4 *>(ww + st * kTileWBytes + r * 512);
+      const float wq[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int t = 0; t < kWarpTok; t += 2)
+          ffma2_acc(acc[r][t], acc[r][t + 1], x[q][t], x[q][t + 1], wq[q]);
+    }
+  }
+
+  // the xor butterfly (offsets 16 .. 1) of all 128 sums: at each step a lane
+  // keeps half of its values and hands the others to its partner; value
+  // v = 16 t + r ends on lane v / 4
+  float a[kWarpTok * kWarpRow];
+#pragma unroll
+  for (int v = 0; v < kWarpTok * kWarpRow; ++v) a[v] = acc[v % kWarpRow][v / kWarpRow];
+  reduce_step<16, 64>(a, lane);
+  reduce_step<8, 32>(a, lane);
+  reduce_step<4, 16>(a, lane);
+  reduce_step<2, 8>(a, lane);
+  reduce_step<1, 4>(a, lane);
+  const int t = t0 + warp * kWarpTok + (lane >> 2), r = r0 + (lane & 3) * 4;
+  if (t < d.B) {
+    float *dst = z + (size_t)t * m + r;
+    if ((m & 3) == 0 && r + 4 <= m) {
+      *reinterpret_cast<float4 *>(dst) = make_float4(a[0], a[1], a[2], a[3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r + u < m) dst[u] = a[u];
+    }
+  }
+}
+
+template <int NC>
+__global__ void __launch_bounds__(kRouteThreads)
+    route_select_kernel(const int32_t *__restrict__ retained, Dims d, Ws ws,
+                        const float *__restrict__ z) {
+  __shared__ int32_t ids[kMaxExperts];
+  pdl_wait_primary();
+  pdl_launch_dependents();
+  for (int r = threadIdx.x; r < d.m_ret; r += blockDim.x)
+    ids[r] = min(max(retained ? retained[r] : r, 0), d.E - 1);
+  if (blockIdx.x == gridDim.x - 1) report_retained(retained, d, ws);
+  __syncthreads();
+  const int t = blockIdx.x * kRouteWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (t < d.B) topk_token<NC>(z + (size_t)t * d.m_ret, ids, d, ws, t, lane);
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const int tr_step = ws.ctrl[kCtrlTraceStep];
+    trace_stamp(ws, tr_step, kTrRouteEnd);
+    ws.ctrl[kCtrlTraceStep] = tr_step + 1;
+  }
+#endif
+}
+
+// Which calls take the tiled kernels (where the scratch rows hold the logits).
+// A wave of the cluster kernel is 608 tokens; below that the second launch has
+// to be earned by the multiply-adds B m' H.  Whole layers, cluster kernel
+// against tiled, H = 2048 unless said: m' = 128: B = 256 188.1 / 189.1 us,
+// 304 197.5 / 190.2, 512 205.1 / 202.0, 8192 828 / 727; m' = 256: B = 96
+// 233.2 / 232.9, 160 251.2 / 244.2, 8192 912 / 747; m' = 64: B = 400 112.2 /
+// 113.7, 500 116.7 / 116.8, 640 129.4 / 121.8; m' = 96: B = 304 155.9 / 150.5;
+// m' = 32: B = 513 76.4 / 80.1, 640 88.9 / 84.8; H = 4096, m' = 128: B = 200
+// 97.2 / 91.6.  Above 256 tokens the cluster kernel's clusters no longer all
+// find room at once, so less work earns it.  Pools above 256 experts gain from
+// a few tokens on: m' = 512, B = 32 77.6 / 75.4; m' = 1024, B = 16 93.4 / 85.8.
+inline bool route_tiled(const Dims &d) {
+  if ((size_t)d.m_ret * 4 > (size_t)d.k * d.H * 2) return false;
+  const double logits = (double)d.B * d.m_ret;
+  return d.B > 608 || logits * d.H >= (d.B > 256 ? 55e6 : 68e6) ||
+         (d.m_ret > 256 && logits >= 16384);
+}
+
+cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_w,
+                               const int32_t *retained, Dims d, Ws ws, bool pdl,
+                               cudaStream_t stream) {
+  // the logits go where the call's expert outputs will be (route_tiled)
+  float *z = reinterpret_cast<float *>(ws.y);
+  cudaError_t err = cudaFuncSetAttribute(
+      route_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
+  if (err != cudaSuccess) return err;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.gridDim = dim3((d.B + kTileTok - 1) / kTileTok, (d.m_ret + kTileRow - 1) / kTileRow);
+  cfg.blockDim = dim3(kTileThreads);
+  cfg.dynamicSmemBytes = kTileSmem;
+  err = cudaLaunchKernelEx(&cfg, route_logits_kernel, hidden, router_w, retained, d, ws, z);
+  if (err != cudaSuccess) return err;
+  cfg.gridDim = dim3((d.B + kRouteWarps - 1) / kRouteWarps);
+  cfg.blockDim = dim3(kRouteThreads);
+  cfg.dynamicSmemBytes = 0;
+  auto select = d.m_ret <= 128   ? route_select_kernel<4>
+                : d.m_ret <= 256 ? route_select_kernel<8>
+                                 : route_select_kernel<0>;
+  return cudaLaunchKernelEx(&cfg, select, retained, d, ws, (const float *)z);
+}
+
 cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w,
                               const int32_t *retained, Dims d, Ws ws, bool pdl,
                               cudaStream_t stream) {
+  if (route_tiled(d)) return launch_route_tiled(hidden, router_w, retained, d, ws, pdl, stream);
   int dev = 0, optin = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;

@@ -70,3 +70,32 @@ def test_layer_large_batches(H, E, I, k, B, shared):
     _check(out[toks], ref["out"])
     r = sw.slimwise_moe_route(args[0], args[1], None, k, E)
     assert np.array_equal(r["topk_idx"].cpu().numpy(), ref["idx"])
+
+
+# Tiled routing (more than 608 tokens, or enough work) in 32-token x 16-expert
+# tiles with ragged edges, the three top-k forms, a pool whose logits do not
+# fit the scratch rows (the cluster kernel keeps it), any order of the ids
+@pytest.mark.parametrize("H,E,k,B,m_prime", [(256, 16, 2, 609, 8), (2048, 512, 8, 33, 511),
+                                             (2048, 128, 8, 257, 121), (640, 40, 3, 769, 33),
+                                             (2048, 128, 8, 800, 128), (384, 256, 8, 1055, 201),
+                                             (256, 512, 32, 777, 300), (128, 1024, 1, 800, 1024)])
+def test_tiled_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
+    shape = synth.LayerShape(hidden=H, num_experts=E, inter=64, top_k=k)
+    x, wr = synth.hidden_states(B, shape, 3), synth.router_weight(shape, 4)
+    wr[E // 2] = wr[E // 3]  # equal logits: ties to the lowest id
+    ret = synth.retained_set(E, m_prime, 5, shuffle=True)
+    xd, wd, rd = x.to(DEV), wr.to(DEV), ret.to(DEV)
+    r = sw.slimwise_moe_route(xd, wd, rd, k, E)
+    idx, gates = oracle.route(oracle.router_logits(synth.bf16_bits(x), wr.numpy()), ret.numpy(), k)
+    assert np.array_equal(r["topk_idx"].cpu().numpy(), idx)
+    np.testing.assert_allclose(r["topk_gate"].cpu().numpy(), gates, rtol=4e-6, atol=1e-7)
+    # bit for bit what the cluster kernel gives (small batches), special values
+    # among them
+    xd[5], xd[B - 1, 7], xd[30, 9] = 0.0, float("inf"), float("nan")
+    r = sw.slimwise_moe_route(xd, wd, rd, k, E)
+    step = 28
+    for t0 in range(0, B, step):
+        s = sw.slimwise_moe_route(xd[t0:t0 + step].contiguous(), wd, rd, k, E)
+        assert torch.equal(s["topk_idx"], r["topk_idx"][t0:t0 + step])
+        assert torch.equal(s["topk_gate"].view(torch.int32),
+                           r["topk_gate"][t0:t0 + step].view(torch.int32))
