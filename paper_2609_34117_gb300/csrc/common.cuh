@@ -250,6 +250,15 @@ cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w
 cudaError_t launch_group_gather(const __nv_bfloat16 *hidden, const float *w_shared_gate,
                                 Dims d, Ws ws, bool pdl, bool gather, cudaStream_t stream);
 
+// Arrays of 4-byte words copied out by one launch (dst NULL: not wanted).
+constexpr int kMaxExports = 8;
+struct ExportList {
+  int32_t *dst[kMaxExports];
+  const int32_t *src[kMaxExports];
+  int n[kMaxExports];
+};
+cudaError_t launch_export(const ExportList &x, bool pdl, cudaStream_t stream);
+
 struct FfnMaps {
   // Weights, 5-D {K columns, 8 rows, 2, units, experts}, box {64, 8, 2, 4, 1}:
   // a unit is 16 rows of a weight tile, 8 gate rows and the 8 matching up

@@ -159,25 +159,25 @@ int check_workspace(const slimwise_moe_shape *s, int32_t top_k, void *ws,
   return ws_bytes >= L->total ? SLIMWISE_OK : SLIMWISE_ERR_WORKSPACE;
 }
 
-int copy_out(void *dst, const void *src, size_t bytes, cudaStream_t st) {
-  if (!dst || !bytes) return SLIMWISE_OK;
-  return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st) == cudaSuccess
-             ? SLIMWISE_OK
-             : SLIMWISE_ERR_CUDA;
-}
-
-int copy_group_outputs(const Ws &w, const Dims &d, cudaStream_t st, int32_t *counts,
-                       int32_t *offsets, int32_t *union_ids, int32_t *union_size,
-                       int32_t *perm, int32_t *pos) {
-  const size_t slots = (size_t)d.B * d.k;
-  int rc = SLIMWISE_OK;
-  if (!rc) rc = copy_out(counts, w.counts, (size_t)d.E * 4, st);
-  if (!rc) rc = copy_out(offsets, w.offsets, (size_t)(d.E + 1) * 4, st);
-  if (!rc) rc = copy_out(union_ids, w.union_ids, (size_t)d.E * 4, st);
-  if (!rc) rc = copy_out(union_size, w.ctrl + kCtrlUnionSize, 4, st);
-  if (!rc) rc = copy_out(perm, w.perm, slots * 4, st);
-  if (!rc) rc = copy_out(pos, w.pos, slots * 4, st);
-  return rc;
+// Copies the grouping results (and the routing's, where `idx` or `gate` is
+// given) to the caller's buffers.
+int copy_group_outputs(const Ws &w, const Dims &d, cudaStream_t st, bool pdl, int32_t *idx,
+                       float *gate, int32_t *counts, int32_t *offsets, int32_t *union_ids,
+                       int32_t *union_size, int32_t *perm, int32_t *pos) {
+  const int slots = d.B * d.k;
+  ExportList x = {
+      {idx, reinterpret_cast<int32_t *>(gate), counts, offsets, union_ids, union_size, perm, pos},
+      {w.topk_idx, reinterpret_cast<const int32_t *>(w.topk_gate), w.counts, w.offsets,
+       w.union_ids, w.ctrl + kCtrlUnionSize, w.perm, w.pos},
+      {slots, slots, d.E, d.E + 1, d.E, 1, slots, slots}};
+  for (int a = 0; a < kMaxExports; ++a)
+    if (!aligned(x.dst[a], 4)) {  // not a kernel's int32 array: copied by itself
+      if (cudaMemcpyAsync(x.dst[a], x.src[a], (size_t)x.n[a] * 4, cudaMemcpyDeviceToDevice, st) !=
+          cudaSuccess)
+        return SLIMWISE_ERR_CUDA;
+      x.dst[a] = nullptr;
+    }
+  return launch_export(x, pdl, st) == cudaSuccess ? SLIMWISE_OK : SLIMWISE_ERR_CUDA;
 }
 
 // The FFN kernel's tensor maps for one call.  Encoding them costs host time
@@ -505,15 +505,12 @@ int slimwise_moe_route(const void *hidden, const float *router_w,
   const Ws w = make_ws(workspace, L);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (launch_route_topk(static_cast<const __nv_bfloat16 *>(hidden), router_w, retained_idx,
-                        d, w, false, st) != cudaSuccess ||
-      launch_group_gather(static_cast<const __nv_bfloat16 *>(hidden), nullptr, d, w, false, false,
+                        d, w, true, st) != cudaSuccess ||
+      launch_group_gather(static_cast<const __nv_bfloat16 *>(hidden), nullptr, d, w, true, false,
                           st) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
-  const size_t slots = (size_t)d.B * d.k;
-  rc = copy_out(topk_idx, w.topk_idx, slots * 4, st);
-  if (!rc) rc = copy_out(topk_gate, w.topk_gate, slots * 4, st);
-  if (!rc) rc = copy_group_outputs(w, d, st, counts, offsets, union_ids, union_size, perm, pos);
-  return rc;
+  return copy_group_outputs(w, d, st, true, topk_idx, topk_gate, counts, offsets, union_ids,
+                            union_size, perm, pos);
 }
 
 int slimwise_moe_group(const int32_t *topk_idx, int32_t top_k, void *stream,
@@ -532,15 +529,18 @@ int slimwise_moe_group(const int32_t *topk_idx, int32_t top_k, void *stream,
   rc = device_info(&di);
   if (rc) return rc;
   const Dims d = make_dims(shape, top_k, shape->num_experts);
-  const Ws w = make_ws(workspace, L);
+  Ws w = make_ws(workspace, L);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const size_t slots = (size_t)d.B * d.k;
-  if (cudaMemsetAsync(w.ctrl + kCtrlErr, 0, 4, st) != cudaSuccess ||
-      cudaMemcpyAsync(w.topk_idx, topk_idx, slots * 4, cudaMemcpyDeviceToDevice, st) !=
-          cudaSuccess ||
-      launch_group_gather(nullptr, nullptr, d, w, false, false, st) != cudaSuccess)
+  if (cudaMemsetAsync(w.ctrl + kCtrlErr, 0, 4, st) != cudaSuccess) return SLIMWISE_ERR_CUDA;
+  if (aligned(topk_idx, 4))  // the kernels only read the selections
+    w.topk_idx = const_cast<int32_t *>(topk_idx);
+  else if (cudaMemcpyAsync(w.topk_idx, topk_idx, (size_t)d.B * d.k * 4, cudaMemcpyDeviceToDevice,
+                           st) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
-  return copy_group_outputs(w, d, st, counts, offsets, union_ids, union_size, perm, pos);
+  if (launch_group_gather(nullptr, nullptr, d, w, false, false, st) != cudaSuccess)
+    return SLIMWISE_ERR_CUDA;
+  return copy_group_outputs(w, d, st, true, nullptr, nullptr, counts, offsets, union_ids,
+                            union_size, perm, pos);
 }
 
 int slimwise_moe_device_status(const void *workspace, void *stream, int32_t *flags) {

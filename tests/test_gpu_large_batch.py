@@ -99,3 +99,25 @@ def test_tiled_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
         assert torch.equal(s["topk_idx"], r["topk_idx"][t0:t0 + step])
         assert torch.equal(s["topk_gate"].view(torch.int32),
                            r["topk_gate"][t0:t0 + step].view(torch.int32))
+
+
+@pytest.mark.parametrize("B,E,k", [(1, 16, 1), (5, 1024, 32), (300, 96, 8)])
+def test_routing_outputs_may_be_left_out(B, E, k):
+    # any output may be NULL; one written alone equals the same one among all
+    from paper_2609_34117_gb300 import binding
+    import ctypes
+    shape = synth.LayerShape(hidden=256, num_experts=E, inter=64, top_k=k)
+    x = synth.hidden_states(B, shape, 3).to(DEV)
+    wr = synth.router_weight(shape, 4).to(DEV)
+    r = sw.slimwise_moe_route(x, wr, None, k, E)
+    names = ("topk_idx", "topk_gate", "counts", "offsets", "union_ids", "union_size", "perm", "pos")
+    ws = sw.alloc_workspace(B, 256, E, 64, k)
+    s = binding.Shape(B, 256, E, 64)
+    for i, n in enumerate(names):
+        alone = torch.full_like(r[n], -7)
+        ptrs = [alone.data_ptr() if j == i else None for j in range(8)]
+        rc = binding.load().slimwise_moe_route(
+            x.data_ptr(), wr.data_ptr(), None, 0, k, torch.cuda.current_stream().cuda_stream,
+            ctypes.byref(s), ws.data_ptr(), ws.numel(), *ptrs)
+        assert rc == 0
+        assert torch.equal(alone, r[n]), n
