@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(kNormWarps * 32)
 }
 
 __global__ void __launch_bounds__(kSumThreads)
-    expert_sums_kernel(Ws ws, const float *__restrict__ norm2, double *__restrict__ stats) {
+    expert_sums_kernel(Ws ws, const float *__restrict__ norm2, double *__restrict__ stats,
+                       int slots) {
   __shared__ double part[kSumThreads / 32][3];
   pdl_wait_primary();
   const int e = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -74,7 +75,10 @@ __global__ void __launch_bounds__(kSumThreads)
   double mass = 0.0, ean = 0.0, reap = 0.0;
   for (int p = p0 + threadIdx.x; p < p1; p += kSumThreads) {
     const double nrm = sqrt((double)__ldcg(norm2 + p));
-    const double g = (double)__ldcg(&ws.topk_gate[__ldcg(&ws.perm[p])]);
+    // (a position that no slot took, after a token with repeated selections,
+    // holds anything: kept inside the batch)
+    const uint32_t s = min((uint32_t)__ldcg(&ws.perm[p]), (uint32_t)slots - 1u);
+    const double g = (double)__ldcg(&ws.topk_gate[s]);
     mass += g;
     ean += nrm;
     reap += g * nrm;
@@ -119,7 +123,7 @@ cudaError_t launch_expert_stats(Dims d, Ws ws, double *stats, cudaStream_t strea
   if (err != cudaSuccess) return err;
   cfg.gridDim = dim3(d.E);
   cfg.blockDim = dim3(kSumThreads);
-  return cudaLaunchKernelEx(&cfg, expert_sums_kernel, ws, (const float *)norm2, stats);
+  return cudaLaunchKernelEx(&cfg, expert_sums_kernel, ws, (const float *)norm2, stats, slots);
 }
 
 // Retained set: the m' experts of highest score, ties to the lowest id, ids
