@@ -67,6 +67,8 @@ def load(path: str | None = None) -> ctypes.CDLL:
     """Load libslimwise.so (or `path`, or $SLIMWISE_LIBRARY); raises if it has
     not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             p = path or library_path()
@@ -108,19 +110,21 @@ def _check(rc: int, what: str):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
+    # the raw handle: building a torch.cuda.Stream for the current stream took
+    # 2.9 of the 18 us that a call spends on the host
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _dev(t, dtype, name):
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
@@ -324,10 +328,13 @@ def slimwise_moe_decode_ex(hidden, router_w, retained_idx, w_gate_up, w_down, to
 
 
 def _group_outputs(B, k, E, device):
-    i32 = dict(dtype=torch.int32, device=device)
-    return {"counts": torch.empty(E, **i32), "offsets": torch.empty(E + 1, **i32),
-            "union_ids": torch.empty(E, **i32), "union_size": torch.empty(1, **i32),
-            "perm": torch.empty(B * k, **i32), "pos": torch.empty(B * k, **i32)}
+    empty, i32 = torch.empty, torch.int32
+    return {"counts": empty(E, dtype=i32, device=device),
+            "offsets": empty(E + 1, dtype=i32, device=device),
+            "union_ids": empty(E, dtype=i32, device=device),
+            "union_size": empty(1, dtype=i32, device=device),
+            "perm": empty(B * k, dtype=i32, device=device),
+            "pos": empty(B * k, dtype=i32, device=device)}
 
 
 def slimwise_moe_route(hidden, router_w, retained_idx, top_k, num_experts, inter=64,
@@ -345,11 +352,11 @@ def slimwise_moe_route(hidden, router_w, retained_idx, top_k, num_experts, inter
            "topk_gate": torch.empty((B, top_k), dtype=torch.float32, device=hidden.device)}
     res.update(_group_outputs(B, top_k, num_experts, hidden.device))
     n_ret = 0 if retained_idx is None else int(retained_idx.numel())
+    # the dict's order is the C arguments' order
     _check(load().slimwise_moe_route(
         _ptr(hidden), _ptr(router_w), _ptr(retained_idx), n_ret, int(top_k), _stream(stream),
-        ctypes.byref(s), _ptr(workspace), workspace.numel(),
-        *[_ptr(res[n]) for n in ("topk_idx", "topk_gate", "counts", "offsets", "union_ids",
-                                  "union_size", "perm", "pos")]), "slimwise_moe_route")
+        ctypes.byref(s), _ptr(workspace), workspace.numel(), *[t.data_ptr() for t in res.values()]),
+        "slimwise_moe_route")
     return res
 
 
