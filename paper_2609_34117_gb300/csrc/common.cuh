@@ -206,7 +206,12 @@ struct Dims {
   int S;          // shared-expert work entries: ceil(B / tok_chunk), 0 without one
   int wide;       // 1: a routed work item covers two adjacent 128-row weight tiles
   int pair;       // 1: the same two tiles, one per CTA of a 2-CTA cluster (M = 256 MMA)
+  int local;      // 1: no grouping kernel; the FFN and combine CTAs group the batch themselves
 };
+// Batches of at most kLocalTokens tokens are grouped inside the FFN and the
+// combine (expert_ffn.cu), from one bit mask of tokens per expert.
+constexpr int kLocalTokens = 64;
+constexpr int kLocalWords = kLocalTokens / 32;
 
 // Work items per entry: routed gate/up tiles (64 gate + 64 up rows each, or
 // twice that for wide items) and down tiles (128 rows of W_down, or 256).
@@ -269,6 +274,7 @@ struct FfnMaps {
   // token rows: box 64 x 16 (m + 1), or 64 x 8 (m + 1) for pair items (each
   // CTA of the pair loads half of an item's rows)
   CUtensorMap xp[kTokBoxSizes];     // [B*k rows, H cols] bf16
+  CUtensorMap hid;                  // the caller's hidden rows [B, H], box 64 x tok_chunk (local)
   CUtensorMap act[kTokBoxSizes];    // [B*k rows, I cols] bf16
   // shared expert (encoded only when there is one)
   CUtensorMap w_gu_s;               // [1, 2Is, H] bf16
@@ -285,8 +291,10 @@ constexpr uint64_t kDefaultWaitLimitNs = 1000000000ull;
 cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStream_t stream);
 // retained: the call's retained ids (NULL: the full pool or a compacted one),
 // read only to guess which weight tiles to warm in L2.
-cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
-                              __nv_bfloat16 *out, const int32_t *retained, int grid, bool pdl,
+// hidden, w_shared_gate: read only when the call groups locally (d.local).
+cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
+                              const float *w_shared_gate, Dims d, Ws ws,
+                              const int32_t *retained, int grid, bool pdl,
                               cudaStream_t stream, uint64_t timeout_ns = kDefaultWaitLimitNs,
                               int starve_first_down = 0);
 
@@ -689,6 +697,27 @@ __device__ __forceinline__ uint32_t idesc_bf16_f32(int M, int N) {
          | (1u << 10)                    // B format: bf16
          | ((uint32_t)(N >> 3) << 17)    // N / 8
          | ((uint32_t)(M >> 4) << 24);   // M / 16
+}
+// Sigmoid gate of the shared expert for token t, by one warp: lane l
+// accumulates elements 128c + 4l + q (c, q ascending) with fused
+// multiply-adds, then an xor butterfly over the lanes.
+__device__ __forceinline__ void shared_gate_token(const __nv_bfloat16 *__restrict__ hidden,
+                                                  const float *__restrict__ w_sg, const Dims &d,
+                                                  const Ws &ws, int t, int lane) {
+  const __nv_bfloat16 *xr = hidden + (size_t)t * d.H;
+  float p = 0.0f;
+  for (int c = 0; c < d.H / 128; ++c) {
+    const int h = 128 * c + 4 * lane;
+    const uint2 xv = *reinterpret_cast<const uint2 *>(xr + h);
+    const float4 wv = *reinterpret_cast<const float4 *>(w_sg + h);
+    p = fmaf(__uint_as_float(xv.x << 16), wv.x, p);
+    p = fmaf(__uint_as_float(xv.x & 0xFFFF0000u), wv.y, p);
+    p = fmaf(__uint_as_float(xv.y << 16), wv.z, p);
+    p = fmaf(__uint_as_float(xv.y & 0xFFFF0000u), wv.w, p);
+  }
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) p = p + __shfl_xor_sync(0xFFFFFFFFu, p, off);
+  if (lane == 0) ws.shared_gate[t] = 1.0f / (1.0f + expf(-p));
 }
 #endif  // __CUDACC__
 

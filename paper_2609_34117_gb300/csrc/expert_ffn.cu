@@ -72,7 +72,8 @@ struct __align__(16) ItemSlot {
   int form;       // bit 0: down, bit 1: shared expert
   int slot_base;
   int n;          // tokens
-  int pad[2];
+  int expert;
+  int pad;
 };
 
 // A pipeline stage: one 64-wide K sub-tile (one 128-byte swizzle atom) of
@@ -82,11 +83,18 @@ struct FfnSmem {
   int stages;
   int a_bytes;
   int stage_bytes;
-  size_t xch_off, bar_off, misc_off, total;
+  size_t xch_off, bar_off, misc_off, local_off, total;
 };
 
+// Local grouping of the batch in a CTA's shared memory: per expert the mask of
+// its tokens [E][kLocalWords] and, for the j-th selected expert, its id and its
+// first grouped position.
+__host__ __device__ inline size_t local_group_bytes(int E) {
+  return (size_t)E * (kLocalWords * 4 + 2 * 2);
+}
+
 __host__ __device__ inline FfnSmem ffn_smem_plan(int tok_chunk, int stages, int wide,
-                                                  int pair) {
+                                                  int pair, int local_experts) {
   FfnSmem p;
   p.stages = stages;
   p.a_bytes = kATileBytes * (wide ? 2 : 1);
@@ -97,8 +105,11 @@ __host__ __device__ inline FfnSmem ffn_smem_plan(int tok_chunk, int stages, int 
   // drain, and for a pair mailbox_full[R], mailbox_empty[R]
   p.misc_off = align_up(
       p.bar_off + 8 * (2 * stages + 4 + 2 * kItemRing + 1 + (pair ? 2 * kItemRing : 0)), 16);
-  // item ring, tmem base, abort, consumed stages, and for a pair the mailbox[R]
-  p.total = p.misc_off + kItemRing * sizeof(ItemSlot) + 4 * (3 + (pair ? kItemRing : 0)) + 1024;
+  // item ring, tmem base, abort, consumed stages, union size, and for a pair
+  // the mailbox[R]
+  p.local_off =
+      align_up(p.misc_off + kItemRing * sizeof(ItemSlot) + 4 * (4 + (pair ? kItemRing : 0)), 8);
+  p.total = p.local_off + local_group_bytes(local_experts) + 1024;
   return p;
 }
 
@@ -123,6 +134,60 @@ struct Item {
   int n;         // tokens
 };
 
+// The local grouping (local_group_bytes).
+struct LocalGroup {
+  uint32_t *mask;        // [E][kLocalWords] tokens of each expert
+  unsigned short *ids;   // [E] selected experts, ascending
+  unsigned short *base;  // [E] first grouped position of each of them
+  __device__ __forceinline__ int count(int e) const {
+    static_assert(kLocalWords == 2, "one 8-byte mask per expert");
+    const uint2 m = reinterpret_cast<const uint2 *>(mask)[e];
+    return __popc(m.x) + __popc(m.y);
+  }
+  // rank of token t among expert e's, or -1 when it is not one of them
+  __device__ __forceinline__ int rank(int e, int t) const {
+    const uint2 m = reinterpret_cast<const uint2 *>(mask)[e];
+    const uint32_t own = t < 32 ? m.x : m.y, bit = 1u << (t & 31);
+    if (!(own & bit)) return -1;
+    return __popc(own & (bit - 1u)) + (t < 32 ? 0 : __popc(m.x));
+  }
+};
+__device__ __forceinline__ LocalGroup local_group(void *p, int E) {
+  LocalGroup lg;
+  lg.mask = reinterpret_cast<uint32_t *>(p);
+  lg.ids = reinterpret_cast<unsigned short *>(lg.mask + (size_t)E * kLocalWords);
+  lg.base = lg.ids + E;
+  return lg;
+}
+// The tokens' masks from the selections, by all threads of the CTA (masks
+// zeroed before).  Ids are kept inside the pool.
+__device__ __forceinline__ void mark_tokens(const LocalGroup &lg, const Dims &d, const Ws &ws) {
+  for (int i = threadIdx.x; i < d.B * d.k; i += blockDim.x) {
+    const int e = min(max(__ldcg(&ws.topk_idx[i]), 0), d.E - 1), t = i / d.k;
+    atomicOr(&lg.mask[e * kLocalWords + (t >> 5)], 1u << (t & 31));
+  }
+}
+// Chunk c (experts 32 c ..) of the exclusive scan over the experts, by one warp
+// of any: `n` tokens of this lane's expert; returns the tokens (<< 16) and the
+// selected experts of all experts before it.
+__device__ __forceinline__ int scan_experts(const LocalGroup &lg, int E, int c, int lane, int &n) {
+  int before = 0;
+  for (int e = lane; e < 32 * c; e += 32) {
+    const int m = lg.count(e);
+    before += (m << 16) | (m > 0 ? 1 : 0);
+  }
+  before = __reduce_add_sync(0xFFFFFFFFu, before);
+  n = 32 * c + lane < E ? lg.count(32 * c + lane) : 0;
+  const int own = (n << 16) | (n > 0 ? 1 : 0);
+  int incl = own;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+    if (lane >= off) incl += o;
+  }
+  return before + incl - own;
+}
+
 // Work-item ranges of one launch, in the order they are handed out:
 //   [shared gate/up: S*t1s][routed gate/up: r1][shared down: S*t2][routed down]
 // Every gate/up item precedes every down item; the shared expert's items go
@@ -133,8 +198,9 @@ struct ItemPlan {
   int S;            // shared-expert entries (0: none); routed entries follow them
 };
 
-template <bool kShared>
-__device__ __forceinline__ Item decode_item(int item, const ItemPlan &ip, const Ws &ws) {
+template <bool kShared, bool kLocal>
+__device__ __forceinline__ Item decode_item(int item, const ItemPlan &ip, const Ws &ws,
+                                            const LocalGroup &lg, int B) {
   Item it;
   it.shared = 0;
   if constexpr (!kShared) {
@@ -165,6 +231,20 @@ __device__ __forceinline__ Item decode_item(int item, const ItemPlan &ip, const 
     const int e = j / t;
     it.tile = j - e * t;
     it.entry = it.shared ? e : ip.S + e;
+  }
+  if constexpr (kLocal) {
+    // one entry per selected expert (and one for the shared expert); a
+    // gate/up item multiplies every token of the batch, in token order
+    it.expert = -1;
+    it.slot_base = 0;
+    it.n = B;
+    if (!it.shared) {
+      const int j = it.entry - ip.S;
+      it.expert = lg.ids[j];
+      it.slot_base = lg.base[j];
+      if (it.down) it.n = lg.count(it.expert);
+    }
+    return it;
   }
   const int4 en = __ldcg(&ws.entries[it.entry]);
   it.expert = en.x;
@@ -245,11 +325,12 @@ __device__ __forceinline__ float swiglu(uint32_t g, uint32_t u) {
 // first and last 16 rows; `base`: the first token's first element of this
 // warp; `left`: tokens left from it on.
 //
-// 16 kTok16 tokens of 16 activations.
-template <int kTok16, int R>
+// 16 kTok16 tokens of 16 activations; row(t): row after `base` of the t-th of
+// them, -1 to leave it out.
+template <int kTok16, int R, class Row>
 __device__ __forceinline__ void store_activations(const uint32_t (&v0)[R], const uint32_t (&v1)[R],
                                                   uint32_t wbuf, int lane, __nv_bfloat16 *base,
-                                                  int ld, int left) {
+                                                  int ld, const Row &row) {
   static_assert(R == 8 * kTok16, "fragment of 16 kTok16 columns");
   const uint32_t dst = wbuf + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * kActRowBytes +
                                          ((lane >> 3) & 1) * 16);
@@ -269,7 +350,8 @@ __device__ __forceinline__ void store_activations(const uint32_t (&v0)[R], const
   for (int p = 0; p < kTok16; ++p) {
     const int t = p * 16 + (lane >> 1);
     const uint4 w = ld_shared_v4(wbuf + (uint32_t)(t * kActRowBytes + (lane & 1) * 16));
-    if (t < left) *reinterpret_cast<uint4 *>(base + (size_t)t * ld + (lane & 1) * 8) = w;
+    const int r = row(t);
+    if (r >= 0) *reinterpret_cast<uint4 *>(base + (size_t)r * ld + (lane & 1) * 8) = w;
   }
   __syncwarp();
 }
@@ -353,20 +435,36 @@ __device__ __forceinline__ void raise_abort(volatile int *abort, Ws &ws, int bit
 // these round trips.  Large token chunks only (kAheadMinChunk): their items
 // are many per CTA, and an unstarted item held back at the end of the launch
 // is a small share of it.
-template <bool kShared, bool kWide, bool kPair, bool kAhead>
+//
+// kLocal (at most kLocalTokens tokens): there is no grouping kernel.  Every CTA
+// marks the batch's selections in shared memory (one bit mask of tokens per
+// expert), lists the selected experts and their first grouped positions, and
+// takes one entry per expert from that list.  A gate/up item multiplies all
+// tokens of the batch, in token order, straight from the caller's hidden rows
+// (a box of at most 64 rows, 8 KB a stage; the MMA has room for them at any
+// batch), and its epilogue stores the rows of the expert's tokens in grouped
+// order, so a down item reads its own tokens' activations alone, as elsewhere.
+// With the grouping kernel, which costs a launch boundary and the copy of the
+// rows, against without, a step: m' = 32 B = 37 55.6 / 52.2 us, m' = 64 B = 1
+// 31.8 / 27.8, full pool B = 64 176.9 / 172.4, Qwen3.6-shaped layer with the
+// shared expert B = 32 120.8 / 114.4.
+template <bool kShared, bool kWide, bool kPair, bool kAhead, bool kLocal>
 __global__ void __maxnreg__(128)
-    expert_ffn_kernel(const __grid_constant__ FfnMaps maps, Dims d, Ws ws,
-                      __nv_bfloat16 *__restrict__ out,
+    expert_ffn_kernel(const __grid_constant__ FfnMaps maps,
+                      const __nv_bfloat16 *__restrict__ hidden,
+                      const float *__restrict__ w_shared_gate, Dims d, Ws ws,
                       const int32_t *__restrict__ retained, int stages,
                       int tmem_cols, int static_first, int early_dependents,
                       uint64_t timeout_ns,
                       int starve_first_down) {
   static_assert(!(kPair && kWide), "a pair item is a 128-row tile in each CTA");
   static_assert(!(kAhead && kPair), "a pair's items are handed from CTA to CTA");
+  static_assert(!(kLocal && (kWide || kPair || kAhead)), "small batches take plain items");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const FfnSmem plan = ffn_smem_plan(d.tok_chunk, stages, d.wide, kPair ? 1 : 0);
+  const FfnSmem plan =
+      ffn_smem_plan(d.tok_chunk, stages, d.wide, kPair ? 1 : 0, kLocal ? d.E : 0);
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar0 = smem_base + (uint32_t)plan.bar_off;
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -384,7 +482,9 @@ __global__ void __maxnreg__(128)
   volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(misc);
   volatile int *abort = misc + 1;
   volatile int *consumed = misc + 2;                 // stages the MMA finished with
-  volatile int *mbox = misc + 3;                     // [kItemRing], pair only
+  int *n_union = misc + 3;                           // selected experts, local grouping only
+  volatile int *mbox = misc + 4;                     // [kItemRing], pair only
+  const LocalGroup lg = local_group(smem + plan.local_off, kLocal ? d.E : 0);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t crank = kPair ? cluster_ctarank() : 0u;  // CTA of the pair
@@ -413,14 +513,17 @@ __global__ void __maxnreg__(128)
     *consumed = 0;
     mbar_fence_init();
   }
+  if constexpr (kLocal)
+    for (int i = threadIdx.x; i < d.E * kLocalWords; i += blockDim.x) lg.mask[i] = 0u;
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&maps.w_gu);
     tma_prefetch_desc(&maps.w_down);
+    if constexpr (kLocal) tma_prefetch_desc(&maps.hid);
     for (int m = 0; m < kTokBoxSizes && kTokBox * (m + 1) <= d.tok_chunk; ++m) {
-      tma_prefetch_desc(&maps.xp[m]);
+      if constexpr (!kLocal) tma_prefetch_desc(&maps.xp[m]);
       tma_prefetch_desc(&maps.act[m]);
       if constexpr (kShared) {
-        tma_prefetch_desc(&maps.xt[m]);
+        if constexpr (!kLocal) tma_prefetch_desc(&maps.xt[m]);
         tma_prefetch_desc(&maps.act_s[m]);
       }
     }
@@ -493,18 +596,45 @@ __global__ void __maxnreg__(128)
   if (early_dependents) pdl_launch_dependents();
 #ifdef SLIMWISE_TRACE
   const int tr_step = ws.ctrl[kCtrlTraceStep] - 1;
-  if (blockIdx.x == 0 && threadIdx.x == 0) trace_stamp(ws, tr_step, kTrFfnStart);
+  if (kLocal && blockIdx.x == 0 && threadIdx.x == 0) trace_stamp(ws, tr_step, kTrGroupStart);
+#endif
+  if constexpr (kLocal) {
+    mark_tokens(lg, d, ws);
+    __syncthreads();
+    for (int c = warp; 32 * c < d.E; c += blockDim.x / 32) {
+      int n;
+      const int before = scan_experts(lg, d.E, c, lane, n);
+      const int e = 32 * c + lane, j = before & 0xFFFF;
+      if (n > 0) {
+        lg.ids[j] = (unsigned short)e;
+        lg.base[j] = (unsigned short)(before >> 16);
+      }
+      if (e == d.E - 1) *n_union = j + (n > 0 ? 1 : 0);
+    }
+    __syncthreads();
+  }
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (kLocal) trace_stamp(ws, tr_step, kTrGroupEnd);
+    trace_stamp(ws, tr_step, kTrFfnStart);
+  }
 #endif
 
-  const int total = __ldcg(&ws.ctrl[kCtrlTotalItems]);
   const int t1 = gate_up_tiles(d);
   const int t2 = down_tiles(d);
   ItemPlan ip;
-  ip.r1 = __ldcg(&ws.ctrl[kCtrlItems1]);
   ip.t1 = t1;
   ip.t1s = kShared ? shared_gate_up_tiles(d) : 0;
   ip.t2 = t2;
   ip.S = kShared ? d.S : 0;
+  int total;
+  if constexpr (kLocal) {
+    ip.r1 = *n_union * t1;
+    total = ip.S * (ip.t1s + t2) + *n_union * (t1 + t2);
+  } else {
+    ip.r1 = __ldcg(&ws.ctrl[kCtrlItems1]);
+    total = __ldcg(&ws.ctrl[kCtrlTotalItems]);
+  }
   const int nb_cols = ffn_acc_cols(d);  // TMEM columns per accumulator buffer
   constexpr int wmul = kWide ? 2 : 1;   // 128-row halves of a routed item in this CTA
   // 128-row tiles of a routed item (across the pair): its gate/up items count
@@ -538,7 +668,7 @@ __global__ void __maxnreg__(128)
     // work entry of an item, uniform over the warp
     auto fetch = [&](int i) {
       Item r = {};
-      if (i < total) r = decode_item<kShared>(i, ip, ws);
+      if (i < total) r = decode_item<kShared, kLocal>(i, ip, ws, lg, d.B);
       r.expert = __shfl_sync(0xFFFFFFFFu, r.expert, 0);
       r.slot_base = __shfl_sync(0xFFFFFFFFu, r.slot_base, 0);
       r.n = __shfl_sync(0xFFFFFFFFu, r.n, 0);
@@ -594,6 +724,7 @@ __global__ void __maxnreg__(128)
         sl.form = it.down | (it.shared << 1);
         sl.slot_base = it.slot_base;
         sl.n = it.n;
+        sl.expert = it.expert;
         ring[slot] = sl;
         mbar_arrive(itf_bar(slot));
       }
@@ -612,7 +743,8 @@ __global__ void __maxnreg__(128)
       // of a pair loads half of them, from 8 n16 rows further for the second
       const int n16 = (it.n + 15) >> 4;
       const int box_m = token_box_for(n16);
-      const int tok_row = it.slot_base + (kPair ? (int)crank * n16 * (kTokBox / 2) : 0);
+      const int tok_row = (kLocal && !it.down ? 0 : it.slot_base) +
+                          (kPair ? (int)crank * n16 * (kTokBox / 2) : 0);
       // weight rows: per 128-row half of the item, two boxes of 4 units (64
       // rows) -- gate and up rows in alternating groups of 8, or 128
       // consecutive down rows; a pair's CTA r loads half r
@@ -633,6 +765,7 @@ __global__ void __maxnreg__(128)
         bmap = it.down ? (const void *)&maps.act[box_m] : (const void *)&maps.xp[box_m];
         expert = it.expert;
       }
+      if (kLocal && !it.down) bmap = (const void *)&maps.hid;  // the batch, in token order
       if (kAhead && lane == 0) next = n_first + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
       if (it.down && !ready) {
         // the entry's activations must be complete: all its gate/up tiles
@@ -828,6 +961,11 @@ __global__ void __maxnreg__(128)
     const int q = warp & 3;             // TMEM lane quarter of this warp
     const int et = (threadIdx.x - 64) & (kEpiThreads - 1);
     const uint32_t wbuf = smem_base + (uint32_t)(plan.xch_off + (warp - 2) * kXchWarpBytes);
+    // the shared expert's gates, where no grouping kernel computes them: one
+    // token per CTA, before its first accumulators are ready
+    if (kLocal && kShared && warp == 9)
+      for (int t = blockIdx.x; t < d.B; t += gridDim.x)
+        shared_gate_token(hidden, w_shared_gate, d, ws, t, lane);
     int slot = 0;
     uint32_t rphase = 0;
     for (int local = 0;; ++local) {
@@ -875,6 +1013,11 @@ __global__ void __maxnreg__(128)
                  32 * q;
         }
         int c = 0;
+        // row, after `base`, of the activations of accumulator column c + t
+        auto row_of = [&](int t) {
+          if (kLocal && !shared) return c + t < d.B ? lg.rank(it.expert, c + t) : -1;
+          return c + t < it.n ? c + t : -1;
+        };
         for (; c + 32 <= cols; c += 32) {
           uint32_t v0[16], v1[16];
           tmem_ld_frag(th + c, v0);
@@ -885,7 +1028,7 @@ __global__ void __maxnreg__(128)
             store_outputs<0>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
             store_outputs<2>(v0, v1, wbuf, lane, base + (size_t)(c + 16) * ld, ld, it.n - c - 16);
           } else {
-            store_activations<2>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
+            store_activations<2>(v0, v1, wbuf, lane, base, ld, row_of);
           }
         }
         if (c < cols) {  // 16 columns left
@@ -895,7 +1038,7 @@ __global__ void __maxnreg__(128)
           tmem_ld_wait();
           if (hh == halves - 1) release();
           if (down) store_outputs<0>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
-          else store_activations<1>(v0, v1, wbuf, lane, base + (size_t)c * ld, ld, it.n - c);
+          else store_activations<1>(v0, v1, wbuf, lane, base, ld, row_of);
         }
       }
       if (!down) {
@@ -943,9 +1086,10 @@ __global__ void __maxnreg__(128)
 // the FFN's expert outputs are complete.
 constexpr int kCombineThreads = 256;
 
-template <bool kShared>
+template <bool kShared, bool kLocal>
 __global__ void __launch_bounds__(kCombineThreads)
     combine_kernel(Dims d, Ws ws, __nv_bfloat16 *__restrict__ out) {
+  extern __shared__ __align__(8) uint32_t masks[];  // kLocal: [E][kLocalWords], then base [E]
   const int t2 = d.H / kCombineTile;
   const int lane = threadIdx.x & 31;
   const int wpc = kCombineThreads / 32;
@@ -953,12 +1097,34 @@ __global__ void __launch_bounds__(kCombineThreads)
   // One pair per warp (the grid covers them all).  Its grouped positions and
   // gates were written by the routing and grouping kernels, which finished
   // before the expert FFN started its work, so they are read before waiting
-  // for the FFN; only the expert outputs need the wait.
+  // for the FFN; only the expert outputs need the wait.  Without a grouping
+  // kernel the positions are worked out here, from the selections: an
+  // expert's first position is the number of tokens of the experts before it.
   const int pr = blockIdx.x * wpc + (threadIdx.x >> 5);
   const int t = pr / t2;
   int p = 0;
   float gj = 0.0f, sg = 0.0f;
-  if (pr < pairs) {
+  if constexpr (kLocal) {
+    LocalGroup lg;
+    lg.mask = masks;
+    lg.ids = nullptr;
+    lg.base = reinterpret_cast<unsigned short *>(masks + d.E * kLocalWords);  // by expert id
+    for (int i = threadIdx.x; i < d.E * kLocalWords; i += blockDim.x) masks[i] = 0u;
+    __syncthreads();
+    mark_tokens(lg, d, ws);
+    __syncthreads();
+    for (int c = threadIdx.x >> 5; 32 * c < d.E; c += wpc) {
+      int n;
+      const int before = scan_experts(lg, d.E, c, lane, n);
+      if (32 * c + lane < d.E) lg.base[32 * c + lane] = (unsigned short)(before >> 16);
+    }
+    __syncthreads();
+    if (pr < pairs && lane < d.k) {
+      const int e = min(max(__ldcg(&ws.topk_idx[(size_t)t * d.k + lane]), 0), d.E - 1);
+      gj = __ldcg(&ws.topk_gate[(size_t)t * d.k + lane]);
+      p = lg.base[e] + lg.rank(e, t);
+    }
+  } else if (pr < pairs) {
     if (lane < d.k) {
       p = __ldcg(&ws.pos[(size_t)t * d.k + lane]);
       gj = __ldcg(&ws.topk_gate[(size_t)t * d.k + lane]);
@@ -970,7 +1136,10 @@ __global__ void __launch_bounds__(kCombineThreads)
   // for SMs with this grid's (and, with 8-token routing clusters, wait for
   // whole GPCs), which cost up to 7 us at B = 288, m' = 32.  It starts when
   // this grid ends.
-  if (pr < pairs) combine_token<kShared>(ws, d, out, t, pr - t * t2, lane, p, gj, sg);
+  if (pr < pairs) {
+    if constexpr (kShared && kLocal) sg = __ldcg(&ws.shared_gate[t]);  // written by the FFN
+    combine_token<kShared>(ws, d, out, t, pr - t * t2, lane, p, gj, sg);
+  }
 }
 
 cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStream_t stream) {
@@ -979,20 +1148,22 @@ cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStre
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((pairs + wpc - 1) / wpc);
   cfg.blockDim = dim3(kCombineThreads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = d.local ? (size_t)d.E * (kLocalWords * 4 + 2) : 0;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (d.Is > 0) return cudaLaunchKernelEx(&cfg, combine_kernel<true>, d, ws, out);
-  return cudaLaunchKernelEx(&cfg, combine_kernel<false>, d, ws, out);
+  auto kernel = d.Is > 0 ? (d.local ? combine_kernel<true, true> : combine_kernel<true, false>)
+                         : (d.local ? combine_kernel<false, true> : combine_kernel<false, false>);
+  return cudaLaunchKernelEx(&cfg, kernel, d, ws, out);
 }
 
-int ffn_stages_for(int tok_chunk, int wide, int pair, size_t smem_limit) {
+int ffn_stages_for(const Dims &d, size_t smem_limit) {
+  const int le = d.local ? d.E : 0;
   int s = 12;
-  while (s > 2 && ffn_smem_plan(tok_chunk, s, wide, pair).total + 1024 > smem_limit) --s;
+  while (s > 2 && ffn_smem_plan(d.tok_chunk, s, d.wide, d.pair, le).total + 1024 > smem_limit) --s;
   return s;
 }
 
@@ -1030,8 +1201,9 @@ cudaError_t pair_clusters_resident(const void *kernel, size_t smem, int dev, int
   return cudaSuccess;
 }
 
-cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
-                              __nv_bfloat16 *out, const int32_t *retained, int grid, bool pdl,
+cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
+                              const float *w_shared_gate, Dims d, Ws ws,
+                              const int32_t *retained, int grid, bool pdl,
                               cudaStream_t stream, uint64_t timeout_ns,
                               int starve_first_down) {
   int dev = 0;
@@ -1049,8 +1221,9 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
     return cudaErrorInvalidValue;
   // the dependent combine kernel needs no shared memory: every byte the
   // block may opt into goes to pipeline stages
-  const int stages = ffn_stages_for(d.tok_chunk, d.wide, d.pair, (size_t)optin);
-  const size_t smem = ffn_smem_plan(d.tok_chunk, stages, d.wide, d.pair).total + 1024;
+  const int stages = ffn_stages_for(d, (size_t)optin);
+  const size_t smem =
+      ffn_smem_plan(d.tok_chunk, stages, d.wide, d.pair, d.local ? d.E : 0).total + 1024;
   if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
   // wide items only without a shared expert, on whole 256-row tiles, with
   // both accumulators of two buffers in the 512 TMEM columns
@@ -1062,13 +1235,15 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
                  d.Is % (2 * kGateRows) != 0))
     return cudaErrorInvalidValue;
   const bool ahead = d.tok_chunk >= kAheadMinChunk;
-  auto kernel = d.Is > 0 ? (d.pair  ? expert_ffn_kernel<true, false, true, false>
-                            : ahead ? expert_ffn_kernel<true, false, false, true>
-                                    : expert_ffn_kernel<true, false, false, false>)
-                : d.pair  ? expert_ffn_kernel<false, false, true, false>
-                : d.wide  ? expert_ffn_kernel<false, true, false, false>
-                : ahead   ? expert_ffn_kernel<false, false, false, true>
-                          : expert_ffn_kernel<false, false, false, false>;
+  auto kernel = d.Is > 0 ? (d.local   ? expert_ffn_kernel<true, false, false, false, true>
+                            : d.pair  ? expert_ffn_kernel<true, false, true, false, false>
+                            : ahead   ? expert_ffn_kernel<true, false, false, true, false>
+                                      : expert_ffn_kernel<true, false, false, false, false>)
+                : d.local ? expert_ffn_kernel<false, false, false, false, true>
+                : d.pair  ? expert_ffn_kernel<false, false, true, false, false>
+                : d.wide  ? expert_ffn_kernel<false, true, false, false, false>
+                : ahead   ? expert_ffn_kernel<false, false, false, true, false>
+                          : expert_ffn_kernel<false, false, false, false, false>;
   err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int tmem_cols = 32;
@@ -1109,8 +1284,8 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, Dims d, Ws ws,
   cfg.numAttrs = na;
   const int static_first = grid <= resident ? 1 : 0;
   const int early_dependents = d.B > 64 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, maps, d, ws, out, retained, stages, tmem_cols,
-                            static_first, early_dependents, timeout_ns, starve_first_down);
+  return cudaLaunchKernelEx(&cfg, kernel, maps, hidden, w_shared_gate, d, ws, retained, stages,
+                            tmem_cols, static_first, early_dependents, timeout_ns, starve_first_down);
 }
 
 }  // namespace slimwise

@@ -60,28 +60,6 @@ __device__ int warp_exclusive_scan(const int *vals, int *outp, int n, int lane) 
   return total;
 }
 
-// Sigmoid gate of the shared expert for token t, by one warp: lane l
-// accumulates elements 128c + 4l + q (c, q ascending) with fused
-// multiply-adds, then an xor butterfly over the lanes.
-__device__ __forceinline__ void shared_gate_token(const __nv_bfloat16 *__restrict__ hidden,
-                                                  const float *__restrict__ w_sg, const Dims &d,
-                                                  const Ws &ws, int t, int lane) {
-  const __nv_bfloat16 *xr = hidden + (size_t)t * d.H;
-  float p = 0.0f;
-  for (int c = 0; c < d.H / 128; ++c) {
-    const int h = 128 * c + 4 * lane;
-    const uint2 xv = *reinterpret_cast<const uint2 *>(xr + h);
-    const float4 wv = *reinterpret_cast<const float4 *>(w_sg + h);
-    p = fmaf(__uint_as_float(xv.x << 16), wv.x, p);
-    p = fmaf(__uint_as_float(xv.x & 0xFFFF0000u), wv.y, p);
-    p = fmaf(__uint_as_float(xv.y << 16), wv.z, p);
-    p = fmaf(__uint_as_float(xv.y & 0xFFFF0000u), wv.w, p);
-  }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) p = p + __shfl_xor_sync(0xFFFFFFFFu, p, off);
-  if (lane == 0) ws.shared_gate[t] = 1.0f / (1.0f + expf(-p));
-}
-
 // The batch-wide results and the FFN work list, each expert written by one of
 // the grid's gstride threads.  cnt[e] selections, offs/flag_scan/entry_base
 // the exclusive scans (with totals at [E]) of the counts, of the union flags

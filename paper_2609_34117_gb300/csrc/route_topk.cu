@@ -178,7 +178,7 @@ __device__ __forceinline__ void take_winner(uint32_t whi, uint32_t wlo, int j, i
 }
 
 // The grid's last CTA reports bad and repeated retained ids and resets the
-// error word of this call.
+// error word (and, for a call that groups locally, the counters).
 __device__ __forceinline__ void report_retained(const int32_t *__restrict__ retained, const Dims &d,
                                                 const Ws &ws) {
   __shared__ uint32_t seen[kMaxExperts / 32];
@@ -198,6 +198,12 @@ __device__ __forceinline__ void report_retained(const int32_t *__restrict__ reta
   }
   __syncthreads();
   if (threadIdx.x == 0) ws.ctrl[kCtrlErr] = bad;
+  // without a grouping kernel the FFN's counters start here: at most one
+  // entry per expert, and the shared expert's
+  if (d.local) {
+    if (threadIdx.x == 0) ws.ctrl[kCtrlWorkCounter] = 0;
+    for (int i = threadIdx.x; i <= d.E; i += blockDim.x) ws.entry_done[i] = 0;
+  }
 }
 
 // Top-k and gates of token t, by one warp, from its logits z[0, m') over the

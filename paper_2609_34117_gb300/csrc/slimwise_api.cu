@@ -1,6 +1,7 @@
 // slimwise_api.cu -- the C ABI declared in include/slimwise_moe.h: argument
-// checks, workspace layout, TMA descriptors, and the four launches of one
-// decode MoE layer (route/top-k -> group/gather -> expert FFN -> combine).
+// checks, workspace layout, TMA descriptors, and the launches of one decode
+// MoE layer (route/top-k -> group/gather, above 64 tokens -> expert FFN ->
+// combine).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -114,7 +115,10 @@ int check_shape(const slimwise_moe_shape *s, int32_t top_k, int32_t m_ret) {
   return SLIMWISE_OK;
 }
 
-Dims make_dims(const slimwise_moe_shape *s, int32_t top_k, int32_t m_ret, int32_t Is = 0) {
+// form: the caller's choice of work-item form (slimwise_decode_opts.ffn_items);
+// grouped: the call needs the grouping kernel's results whatever its size.
+Dims make_dims(const slimwise_moe_shape *s, int32_t top_k, int32_t m_ret, int32_t Is = 0,
+               int32_t form = 0, bool grouped = false) {
   Dims d;
   d.B = s->num_tokens;
   d.H = s->hidden;
@@ -122,33 +126,26 @@ Dims make_dims(const slimwise_moe_shape *s, int32_t top_k, int32_t m_ret, int32_
   d.I = s->inter;
   d.k = top_k;
   d.m_ret = m_ret;
+  d.Is = Is;
+  // CTA-pair items only on request
+  d.pair = (form > 0 && d.I % (2 * kGateRows) == 0 && d.H % (2 * kTileRows) == 0 &&
+            Is % (2 * kGateRows) == 0) ? 1 : 0;
+  d.local = (d.B <= kLocalTokens && !d.pair && !grouped) ? 1 : 0;
   d.tok_chunk = token_chunk_for(d.B, top_k, m_ret);
-  if (Is > 0) {
+  if (d.local) {
+    d.tok_chunk = round16(d.B);  // every item multiplies the whole batch
+  } else if (Is > 0) {
     // the shared expert takes every token: at least 64 of them per entry, so
     // its weight tiles pass through the SMs B/64 times rather than B/16
     // (a larger token slot per stage, a few stages fewer for the routed items)
     const int want = pow2_at_least(d.B) < 64 ? pow2_at_least(d.B) : 64;
     if (d.tok_chunk < want) d.tok_chunk = want;
   }
-  d.Is = Is;
   d.S = Is > 0 ? (d.B + d.tok_chunk - 1) / d.tok_chunk : 0;
-  d.wide = (Is == 0 && d.I % (2 * kGateRows) == 0 && d.H % (2 * kTileRows) == 0 &&
-            d.tok_chunk >= kWideMinChunk && d.tok_chunk <= kWideMaxChunk &&
-            m_ret >= kWideMinPool) ? 1 : 0;
-  d.pair = 0;  // CTA-pair items only on request (apply_item_form)
+  d.wide = (!d.pair && !d.local && Is == 0 && d.I % (2 * kGateRows) == 0 &&
+            d.H % (2 * kTileRows) == 0 && d.tok_chunk >= kWideMinChunk &&
+            d.tok_chunk <= kWideMaxChunk && m_ret >= kWideMinPool) ? 1 : 0;
   return d;
-}
-
-// The caller's choice of work-item form (slimwise_decode_opts.ffn_items).
-void apply_item_form(Dims *d, int32_t form) {
-  const bool can_pair = d->I % (2 * kGateRows) == 0 && d->H % (2 * kTileRows) == 0 &&
-                        d->Is % (2 * kGateRows) == 0;
-  if (form > 0 && can_pair) {
-    d->pair = 1;
-    d->wide = 0;
-  } else if (form < 0) {
-    d->pair = 0;
-  }
 }
 
 int check_workspace(const slimwise_moe_shape *s, int32_t top_k, void *ws,
@@ -205,17 +202,17 @@ struct WeightMapsKey {
 };
 struct TokenMapsKey {
   const void *xp, *act, *xt, *act_s;
-  int H, I, Is, B, tok_chunk, pair, device;
+  int H, I, Is, B, tok_chunk, pair, local, device;
   uint64_t slots;
   bool operator==(const TokenMapsKey &o) const {
     return xp == o.xp && act == o.act && xt == o.xt && act_s == o.act_s && H == o.H &&
            I == o.I && Is == o.Is && B == o.B && tok_chunk == o.tok_chunk && pair == o.pair &&
-           device == o.device && slots == o.slots;
+           local == o.local && device == o.device && slots == o.slots;
   }
 };
 
-bool ffn_maps_for(FfnMaps *maps, const void *w_gate_up, const void *w_down, const Ws &w,
-                  const Dims &d, uint64_t slots, const SharedExpert &se) {
+bool ffn_maps_for(FfnMaps *maps, const void *hidden, const void *w_gate_up, const void *w_down,
+                  const Ws &w, const Dims &d, uint64_t slots, const SharedExpert &se) {
   thread_local bool have_w = false, have_t = false;
   thread_local WeightMapsKey last_w;
   thread_local TokenMapsKey last_t;
@@ -224,7 +221,7 @@ bool ffn_maps_for(FfnMaps *maps, const void *w_gate_up, const void *w_down, cons
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   const WeightMapsKey kw = {w_gate_up, w_down, se.gate_up, se.down, d.E, d.H, d.I, d.Is, dev};
   const TokenMapsKey kt = {w.xp, w.act, w.xt, w.act_s, d.H, d.I, d.Is, d.B, d.tok_chunk, d.pair,
-                          dev, slots};
+                          d.local, dev, slots};
   if (!(have_w && kw == last_w)) {
     have_w = false;
     if (encode_gate_up(&cached.w_gu, w_gate_up, d.E, d.I, d.H) ||
@@ -243,16 +240,20 @@ bool ffn_maps_for(FfnMaps *maps, const void *w_gate_up, const void *w_down, cons
     // as high (8 (b + 1) rows for 16 (b + 1) tokens)
     for (int b = 0; b < kTokBoxSizes && kTokBox * (b + 1) <= d.tok_chunk; ++b) {
       const uint32_t rows = (uint32_t)((d.pair ? kTokBox / 2 : kTokBox) * (b + 1));
-      if (encode_map(&cached.xp[b], w.xp, slots, d.H, rows) ||
+      if ((!d.local && encode_map(&cached.xp[b], w.xp, slots, d.H, rows)) ||
           encode_map(&cached.act[b], w.act, slots, d.I, rows))
         return false;
-      if (d.Is > 0 && (encode_map(&cached.xt[b], w.xt, (uint64_t)d.B, d.H, rows) ||
+      if (d.Is > 0 && ((!d.local && encode_map(&cached.xt[b], w.xt, (uint64_t)d.B, d.H, rows)) ||
                        encode_map(&cached.act_s[b], w.act_s, (uint64_t)d.B, d.Is, rows)))
         return false;
     }
     last_t = kt;
     have_t = true;
   }
+  // the hidden rows' map is made for each call: a program's hidden states
+  // need not stay at one address
+  if (d.local && encode_map(&cached.hid, hidden, (uint64_t)d.B, d.H, (uint32_t)d.tok_chunk))
+    return false;
   *maps = cached;
   return true;
 }
@@ -261,7 +262,7 @@ int decode_impl(const void *hidden, const float *router_w, const int32_t *retain
                 int32_t n_retained, const void *w_gate_up, const void *w_down,
                 int32_t top_k, void *out, void *stream, const slimwise_moe_shape *shape,
                 void *workspace, size_t workspace_bytes, const slimwise_decode_opts *opts,
-                const SharedExpert *shared = nullptr) {
+                const SharedExpert *shared = nullptr, bool grouped = false) {
   const int32_t m_ret = retained ? n_retained : (shape ? shape->num_experts : 0);
   int rc = check_shape(shape, top_k, m_ret);
   if (rc) return rc;
@@ -285,8 +286,7 @@ int decode_impl(const void *hidden, const float *router_w, const int32_t *retain
   rc = device_info(&di);
   if (rc) return rc;
 
-  Dims d = make_dims(shape, top_k, m_ret, se.inter);
-  if (opts) apply_item_form(&d, opts->ffn_items);
+  const Dims d = make_dims(shape, top_k, m_ret, se.inter, opts ? opts->ffn_items : 0, grouped);
   const Ws w = make_ws(workspace, L);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const bool pdl = !(opts && opts->disable_pdl);
@@ -295,13 +295,13 @@ int decode_impl(const void *hidden, const float *router_w, const int32_t *retain
 
   FfnMaps maps;
   const uint64_t slots = (uint64_t)d.B * d.k;
-  if (!ffn_maps_for(&maps, w_gate_up, w_down, w, d, slots, se)) return SLIMWISE_ERR_CUDA;
+  if (!ffn_maps_for(&maps, hidden, w_gate_up, w_down, w, d, slots, se)) return SLIMWISE_ERR_CUDA;
 
   if (launch_route_topk(static_cast<const __nv_bfloat16 *>(hidden), router_w, retained,
                         d, w, pdl, st) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
-  if (launch_group_gather(static_cast<const __nv_bfloat16 *>(hidden), se.gate, d, w, pdl, true,
-                          st) != cudaSuccess)
+  if (!d.local && launch_group_gather(static_cast<const __nv_bfloat16 *>(hidden), se.gate, d, w,
+                                      pdl, true, st) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
   const bool timed = opts && opts->ffn_begin && opts->ffn_end;
   if (timed && cudaEventRecord(static_cast<cudaEvent_t>(opts->ffn_begin), st) != cudaSuccess)
@@ -310,8 +310,8 @@ int decode_impl(const void *hidden, const float *router_w, const int32_t *retain
                                   ? (uint64_t)opts->wait_limit_ns
                                   : kDefaultWaitLimitNs;
   const int starve = (opts && opts->test_starve_first_down) ? 1 : 0;
-  if (launch_expert_ffn(maps, d, w, static_cast<__nv_bfloat16 *>(out), retained, grid,
-                        pdl && !timed, st, wait_limit, starve) != cudaSuccess)
+  if (launch_expert_ffn(maps, static_cast<const __nv_bfloat16 *>(hidden), se.gate, d, w, retained,
+                        grid, pdl && !timed, st, wait_limit, starve) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
   // the combine belongs to the timed span: the events bracket the expert FFN
   // and the combine of its outputs
@@ -397,14 +397,15 @@ int slimwise_moe_expert_stats(const void *hidden, const float *router_w,
   if (shape->num_tokens == 0) return SLIMWISE_OK;
   if (!stats) return SLIMWISE_ERR_INVALID_ARG;
   if (!aligned(stats, 8)) return SLIMWISE_ERR_UNSUPPORTED_SHAPE;
-  // the full-pool layer (its output is the calibration pass's layer output)
+  // the full-pool layer (its output is the calibration pass's layer output),
+  // with the grouping that the statistics read
   rc = decode_impl(hidden, router_w, nullptr, 0, w_gate_up, w_down, top_k, out, stream, shape,
-                   workspace, workspace_bytes, nullptr);
+                   workspace, workspace_bytes, nullptr, nullptr, true);
   if (rc) return rc;
   WsLayout L;
   rc = check_workspace(shape, top_k, workspace, workspace_bytes, &L);
   if (rc) return rc;
-  const Dims d = make_dims(shape, top_k, shape->num_experts);
+  const Dims d = make_dims(shape, top_k, shape->num_experts, 0, 0, true);
   return launch_expert_stats(d, make_ws(workspace, L), stats,
                              reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess
              ? SLIMWISE_OK
@@ -501,7 +502,7 @@ int slimwise_moe_route(const void *hidden, const float *router_w,
   DeviceInfo di;
   rc = device_info(&di);
   if (rc) return rc;
-  const Dims d = make_dims(shape, top_k, m_ret);
+  const Dims d = make_dims(shape, top_k, m_ret, 0, 0, true);
   const Ws w = make_ws(workspace, L);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (launch_route_topk(static_cast<const __nv_bfloat16 *>(hidden), router_w, retained_idx,
@@ -528,7 +529,7 @@ int slimwise_moe_group(const int32_t *topk_idx, int32_t top_k, void *stream,
   DeviceInfo di;
   rc = device_info(&di);
   if (rc) return rc;
-  const Dims d = make_dims(shape, top_k, shape->num_experts);
+  const Dims d = make_dims(shape, top_k, shape->num_experts, 0, 0, true);
   Ws w = make_ws(workspace, L);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(w.ctrl + kCtrlErr, 0, 4, st) != cudaSuccess) return SLIMWISE_ERR_CUDA;
