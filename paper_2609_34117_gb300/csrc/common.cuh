@@ -210,8 +210,11 @@ struct Dims {
 };
 // Batches of at most kLocalTokens tokens are grouped inside the FFN and the
 // combine (expert_ffn.cu), from one bit mask of tokens per expert.
-constexpr int kLocalTokens = 64;
-constexpr int kLocalWords = kLocalTokens / 32;
+constexpr int kLocalTokens = 96;
+// 32-token words of an expert's mask: 2 up to 64 tokens, else 4.
+__host__ __device__ inline int local_words(const Dims &d) {
+  return !d.local ? 0 : d.B <= 64 ? 2 : 4;
+}
 
 // Work items per entry: routed gate/up tiles (64 gate + 64 up rows each, or
 // twice that for wide items) and down tiles (128 rows of W_down, or 256).

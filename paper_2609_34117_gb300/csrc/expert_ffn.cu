@@ -87,14 +87,14 @@ struct FfnSmem {
 };
 
 // Local grouping of the batch in a CTA's shared memory: per expert the mask of
-// its tokens [E][kLocalWords] and, for the j-th selected expert, its id and its
-// first grouped position.
-__host__ __device__ inline size_t local_group_bytes(int E) {
-  return (size_t)E * (kLocalWords * 4 + 2 * 2);
+// its tokens [E][words] and, for the j-th selected expert, its id and its first
+// grouped position.
+__host__ __device__ inline size_t local_group_bytes(int E, int words) {
+  return words ? (size_t)E * (words * 4 + 2 * 2) : 0;
 }
 
 __host__ __device__ inline FfnSmem ffn_smem_plan(int tok_chunk, int stages, int wide,
-                                                  int pair, int local_experts) {
+                                                  int pair, int E, int words) {
   FfnSmem p;
   p.stages = stages;
   p.a_bytes = kATileBytes * (wide ? 2 : 1);
@@ -108,8 +108,8 @@ __host__ __device__ inline FfnSmem ffn_smem_plan(int tok_chunk, int stages, int 
   // item ring, tmem base, abort, consumed stages, union size, and for a pair
   // the mailbox[R]
   p.local_off =
-      align_up(p.misc_off + kItemRing * sizeof(ItemSlot) + 4 * (4 + (pair ? kItemRing : 0)), 8);
-  p.total = p.local_off + local_group_bytes(local_experts) + 1024;
+      align_up(p.misc_off + kItemRing * sizeof(ItemSlot) + 4 * (4 + (pair ? kItemRing : 0)), 16);
+  p.total = p.local_off + local_group_bytes(E, words) + 1024;
   return p;
 }
 
@@ -134,43 +134,68 @@ struct Item {
   int n;         // tokens
 };
 
-// The local grouping (local_group_bytes).
+// The local grouping (local_group_bytes); W mask words per expert.
+template <int W>
 struct LocalGroup {
-  uint32_t *mask;        // [E][kLocalWords] tokens of each expert
+  uint32_t *mask;        // [E][W] tokens of each expert
   unsigned short *ids;   // [E] selected experts, ascending
   unsigned short *base;  // [E] first grouped position of each of them
+  __device__ __forceinline__ void load(int e, uint32_t (&m)[W]) const {
+    static_assert(W == 2 || W == 4, "one 8- or 16-byte mask per expert");
+    if constexpr (W == 2) {
+      const uint2 v = reinterpret_cast<const uint2 *>(mask)[e];
+      m[0] = v.x; m[1] = v.y;
+    } else {
+      const uint4 v = reinterpret_cast<const uint4 *>(mask)[e];
+      m[0] = v.x; m[1] = v.y; m[2] = v.z; m[3] = v.w;
+    }
+  }
   __device__ __forceinline__ int count(int e) const {
-    static_assert(kLocalWords == 2, "one 8-byte mask per expert");
-    const uint2 m = reinterpret_cast<const uint2 *>(mask)[e];
-    return __popc(m.x) + __popc(m.y);
+    uint32_t m[W];
+    load(e, m);
+    int n = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) n += __popc(m[w]);
+    return n;
   }
   // rank of token t among expert e's, or -1 when it is not one of them
   __device__ __forceinline__ int rank(int e, int t) const {
-    const uint2 m = reinterpret_cast<const uint2 *>(mask)[e];
-    const uint32_t own = t < 32 ? m.x : m.y, bit = 1u << (t & 31);
-    if (!(own & bit)) return -1;
-    return __popc(own & (bit - 1u)) + (t < 32 ? 0 : __popc(m.x));
+    uint32_t m[W];
+    load(e, m);
+    const uint32_t bit = 1u << (t & 31);
+    int n = 0;
+    bool in = false;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      if (w == (t >> 5)) in = (m[w] & bit) != 0;
+      n += w < (t >> 5) ? __popc(m[w]) : w == (t >> 5) ? __popc(m[w] & (bit - 1u)) : 0;
+    }
+    return in ? n : -1;
   }
 };
-__device__ __forceinline__ LocalGroup local_group(void *p, int E) {
-  LocalGroup lg;
+template <int W>
+__device__ __forceinline__ LocalGroup<W> local_group(void *p, int E) {
+  LocalGroup<W> lg;
   lg.mask = reinterpret_cast<uint32_t *>(p);
-  lg.ids = reinterpret_cast<unsigned short *>(lg.mask + (size_t)E * kLocalWords);
+  lg.ids = reinterpret_cast<unsigned short *>(lg.mask + (size_t)E * W);
   lg.base = lg.ids + E;
   return lg;
 }
 // The tokens' masks from the selections, by all threads of the CTA (masks
 // zeroed before).  Ids are kept inside the pool.
-__device__ __forceinline__ void mark_tokens(const LocalGroup &lg, const Dims &d, const Ws &ws) {
+template <int W>
+__device__ __forceinline__ void mark_tokens(const LocalGroup<W> &lg, const Dims &d, const Ws &ws) {
   for (int i = threadIdx.x; i < d.B * d.k; i += blockDim.x) {
     const int e = min(max(__ldcg(&ws.topk_idx[i]), 0), d.E - 1), t = i / d.k;
-    atomicOr(&lg.mask[e * kLocalWords + (t >> 5)], 1u << (t & 31));
+    atomicOr(&lg.mask[e * W + (t >> 5)], 1u << (t & 31));
   }
 }
 // Chunk c (experts 32 c ..) of the exclusive scan over the experts, by one warp
 // of any: `n` tokens of this lane's expert; returns the tokens (<< 16) and the
 // selected experts of all experts before it.
-__device__ __forceinline__ int scan_experts(const LocalGroup &lg, int E, int c, int lane, int &n) {
+template <int W>
+__device__ __forceinline__ int scan_experts(const LocalGroup<W> &lg, int E, int c, int lane,
+                                            int &n) {
   int before = 0;
   for (int e = lane; e < 32 * c; e += 32) {
     const int m = lg.count(e);
@@ -198,9 +223,9 @@ struct ItemPlan {
   int S;            // shared-expert entries (0: none); routed entries follow them
 };
 
-template <bool kShared, bool kLocal>
+template <bool kShared, bool kLocal, int W>
 __device__ __forceinline__ Item decode_item(int item, const ItemPlan &ip, const Ws &ws,
-                                            const LocalGroup &lg, int B) {
+                                            const LocalGroup<W> &lg, int B) {
   Item it;
   it.shared = 0;
   if constexpr (!kShared) {
@@ -436,19 +461,20 @@ __device__ __forceinline__ void raise_abort(volatile int *abort, Ws &ws, int bit
 // are many per CTA, and an unstarted item held back at the end of the launch
 // is a small share of it.
 //
-// kLocal (at most kLocalTokens tokens): there is no grouping kernel.  Every CTA
+// kLocalWords > 0 (at most kLocalTokens tokens): there is no grouping kernel.  Every CTA
 // marks the batch's selections in shared memory (one bit mask of tokens per
 // expert), lists the selected experts and their first grouped positions, and
 // takes one entry per expert from that list.  A gate/up item multiplies all
 // tokens of the batch, in token order, straight from the caller's hidden rows
-// (a box of at most 64 rows, 8 KB a stage; the MMA has room for them at any
-// batch), and its epilogue stores the rows of the expert's tokens in grouped
+// (a box of at most 96 rows, 12 KB a stage), and its epilogue stores the rows of the expert's tokens in grouped
 // order, so a down item reads its own tokens' activations alone, as elsewhere.
 // With the grouping kernel, which costs a launch boundary and the copy of the
 // rows, against without, a step: m' = 32 B = 37 55.6 / 52.2 us, m' = 64 B = 1
 // 31.8 / 27.8, full pool B = 64 176.9 / 172.4, Qwen3.6-shaped layer with the
-// shared expert B = 32 120.8 / 114.4.
-template <bool kShared, bool kWide, bool kPair, bool kAhead, bool kLocal>
+// shared expert B = 32 120.8 / 114.4; 64 to 128 tokens, m' = 64: 64 99.4 /
+// 95.8, 96 100.2 / 98.1, 112 100.2 / 99.7, 128 100.1 / 101.4 (larger token
+// boxes take the ring's place and L2 reads; the line is drawn at 96).
+template <bool kShared, bool kWide, bool kPair, bool kAhead, int kLocalWords>
 __global__ void __maxnreg__(128)
     expert_ffn_kernel(const __grid_constant__ FfnMaps maps,
                       const __nv_bfloat16 *__restrict__ hidden,
@@ -457,6 +483,7 @@ __global__ void __maxnreg__(128)
                       int tmem_cols, int static_first, int early_dependents,
                       uint64_t timeout_ns,
                       int starve_first_down) {
+  constexpr bool kLocal = kLocalWords > 0;
   static_assert(!(kPair && kWide), "a pair item is a 128-row tile in each CTA");
   static_assert(!(kAhead && kPair), "a pair's items are handed from CTA to CTA");
   static_assert(!(kLocal && (kWide || kPair || kAhead)), "small batches take plain items");
@@ -464,7 +491,7 @@ __global__ void __maxnreg__(128)
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const FfnSmem plan =
-      ffn_smem_plan(d.tok_chunk, stages, d.wide, kPair ? 1 : 0, kLocal ? d.E : 0);
+      ffn_smem_plan(d.tok_chunk, stages, d.wide, kPair ? 1 : 0, d.E, kLocalWords);
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t bar0 = smem_base + (uint32_t)plan.bar_off;
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -484,7 +511,7 @@ __global__ void __maxnreg__(128)
   volatile int *consumed = misc + 2;                 // stages the MMA finished with
   int *n_union = misc + 3;                           // selected experts, local grouping only
   volatile int *mbox = misc + 4;                     // [kItemRing], pair only
-  const LocalGroup lg = local_group(smem + plan.local_off, kLocal ? d.E : 0);
+  const auto lg = local_group<kLocal ? kLocalWords : 2>(smem + plan.local_off, d.E);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t crank = kPair ? cluster_ctarank() : 0u;  // CTA of the pair
@@ -1086,10 +1113,11 @@ __global__ void __maxnreg__(128)
 // the FFN's expert outputs are complete.
 constexpr int kCombineThreads = 256;
 
-template <bool kShared, bool kLocal>
+template <bool kShared, int kLocalWords>
 __global__ void __launch_bounds__(kCombineThreads)
     combine_kernel(Dims d, Ws ws, __nv_bfloat16 *__restrict__ out) {
-  extern __shared__ __align__(8) uint32_t masks[];  // kLocal: [E][kLocalWords], then base [E]
+  constexpr bool kLocal = kLocalWords > 0;
+  extern __shared__ __align__(16) uint32_t masks[];  // kLocal: [E][kLocalWords], then base [E]
   const int t2 = d.H / kCombineTile;
   const int lane = threadIdx.x & 31;
   const int wpc = kCombineThreads / 32;
@@ -1105,7 +1133,7 @@ __global__ void __launch_bounds__(kCombineThreads)
   int p = 0;
   float gj = 0.0f, sg = 0.0f;
   if constexpr (kLocal) {
-    LocalGroup lg;
+    LocalGroup<kLocal ? kLocalWords : 2> lg;
     lg.mask = masks;
     lg.ids = nullptr;
     lg.base = reinterpret_cast<unsigned short *>(masks + d.E * kLocalWords);  // by expert id
@@ -1148,22 +1176,27 @@ cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStre
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((pairs + wpc - 1) / wpc);
   cfg.blockDim = dim3(kCombineThreads);
-  cfg.dynamicSmemBytes = d.local ? (size_t)d.E * (kLocalWords * 4 + 2) : 0;
+  const int words = local_words(d);
+  cfg.dynamicSmemBytes = d.local ? (size_t)d.E * (words * 4 + 2) : 0;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  auto kernel = d.Is > 0 ? (d.local ? combine_kernel<true, true> : combine_kernel<true, false>)
-                         : (d.local ? combine_kernel<false, true> : combine_kernel<false, false>);
+  auto kernel = d.Is > 0 ? (words == 2   ? combine_kernel<true, 2>
+                            : words == 4 ? combine_kernel<true, 4>
+                                         : combine_kernel<true, 0>)
+                         : (words == 2   ? combine_kernel<false, 2>
+                            : words == 4 ? combine_kernel<false, 4>
+                                         : combine_kernel<false, 0>);
   return cudaLaunchKernelEx(&cfg, kernel, d, ws, out);
 }
 
 int ffn_stages_for(const Dims &d, size_t smem_limit) {
-  const int le = d.local ? d.E : 0;
+  const int words = local_words(d);
   int s = 12;
-  while (s > 2 && ffn_smem_plan(d.tok_chunk, s, d.wide, d.pair, le).total + 1024 > smem_limit) --s;
+  while (s > 2 && ffn_smem_plan(d.tok_chunk, s, d.wide, d.pair, d.E, words).total + 1024 > smem_limit) --s;
   return s;
 }
 
@@ -1223,7 +1256,7 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
   // block may opt into goes to pipeline stages
   const int stages = ffn_stages_for(d, (size_t)optin);
   const size_t smem =
-      ffn_smem_plan(d.tok_chunk, stages, d.wide, d.pair, d.local ? d.E : 0).total + 1024;
+      ffn_smem_plan(d.tok_chunk, stages, d.wide, d.pair, d.E, local_words(d)).total + 1024;
   if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
   // wide items only without a shared expert, on whole 256-row tiles, with
   // both accumulators of two buffers in the 512 TMEM columns
@@ -1235,15 +1268,18 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
                  d.Is % (2 * kGateRows) != 0))
     return cudaErrorInvalidValue;
   const bool ahead = d.tok_chunk >= kAheadMinChunk;
-  auto kernel = d.Is > 0 ? (d.local   ? expert_ffn_kernel<true, false, false, false, true>
-                            : d.pair  ? expert_ffn_kernel<true, false, true, false, false>
-                            : ahead   ? expert_ffn_kernel<true, false, false, true, false>
-                                      : expert_ffn_kernel<true, false, false, false, false>)
-                : d.local ? expert_ffn_kernel<false, false, false, false, true>
-                : d.pair  ? expert_ffn_kernel<false, false, true, false, false>
-                : d.wide  ? expert_ffn_kernel<false, true, false, false, false>
-                : ahead   ? expert_ffn_kernel<false, false, false, true, false>
-                          : expert_ffn_kernel<false, false, false, false, false>;
+  const int words = local_words(d);
+  auto kernel = d.Is > 0 ? (words == 2  ? expert_ffn_kernel<true, false, false, false, 2>
+                            : words == 4 ? expert_ffn_kernel<true, false, false, false, 4>
+                            : d.pair     ? expert_ffn_kernel<true, false, true, false, 0>
+                            : ahead      ? expert_ffn_kernel<true, false, false, true, 0>
+                                         : expert_ffn_kernel<true, false, false, false, 0>)
+                : words == 2 ? expert_ffn_kernel<false, false, false, false, 2>
+                : words == 4 ? expert_ffn_kernel<false, false, false, false, 4>
+                : d.pair     ? expert_ffn_kernel<false, false, true, false, 0>
+                : d.wide     ? expert_ffn_kernel<false, true, false, false, 0>
+                : ahead      ? expert_ffn_kernel<false, false, false, true, 0>
+                             : expert_ffn_kernel<false, false, false, false, 0>;
   err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int tmem_cols = 32;

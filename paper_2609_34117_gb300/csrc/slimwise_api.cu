@@ -1,6 +1,6 @@
 // slimwise_api.cu -- the C ABI declared in include/slimwise_moe.h: argument
 // checks, workspace layout, TMA descriptors, and the launches of one decode
-// MoE layer (route/top-k -> group/gather, above 64 tokens -> expert FFN ->
+// MoE layer (route/top-k -> group/gather, above 96 tokens -> expert FFN ->
 // combine).
 #include <algorithm>
 #include <cmath>

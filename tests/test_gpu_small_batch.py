@@ -1,0 +1,49 @@
+"""Small batches, which the FFN and the combine group by themselves: mask-word
+and chunk edges (32, 64 and 96 tokens), pools that are not whole chunks of 32
+experts, the largest pool and selection, the shared expert."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_34117_gb300 as sw
+from paper_2609_34117_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    sw.build.build()
+    oracle.build()
+
+
+@pytest.mark.parametrize("B,E,k,shared", [(31, 33, 3, 0), (32, 16, 2, 128), (33, 100, 8, 0),
+                                          (64, 1024, 32, 0), (65, 40, 4, 128), (96, 1024, 8, 0),
+                                          (95, 16, 16, 0), (97, 40, 4, 128)])
+def test_layer_small_batches(B, E, k, shared):
+    H, I = 256, 128
+    shape = synth.LayerShape(hidden=H, num_experts=E, inter=I, top_k=k)
+    w_gu, w_d = synth.expert_weights(shape, 1)
+    wr = synth.router_weight(shape, 1)
+    x = synth.hidden_states(B, shape, 2)
+    args = [t.to(DEV) for t in (x, wr)] + [None] + [t.to(DEV) for t in (w_gu, w_d)] + [k]
+    host = [synth.bf16_bits(x), wr.numpy(), None, synth.bf16_bits(w_gu), synth.bf16_bits(w_d), k]
+    if shared:
+        w_sg, gu, dn = synth.shared_expert(H, shared, 3)
+        out = sw.slimwise_moe_decode_shared(*args, w_sg.to(DEV), gu.to(DEV), dn.to(DEV))
+        ref = oracle.moe_decode_shared(*host, w_sg.numpy(), synth.bf16_bits(gu), synth.bf16_bits(dn))
+    else:
+        out = sw.slimwise_moe_decode_full(args[0], args[1], *args[3:])
+        ref = oracle.moe_decode(*host)
+    got = out.float().cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref["out"]) <= 1e-2 * np.linalg.norm(ref["out"])
+    assert np.abs(got - ref["out"]).max() <= 3e-2
+    # in place: the output may be the hidden rows' own buffer
+    if not shared:
+        y = sw.slimwise_moe_decode_full(args[0], args[1], *args[3:], out=args[0])
+        assert torch.equal(y, out)
