@@ -445,12 +445,8 @@ int slimwise_moe_compact_layer(const void *w_gate_up, const void *w_down,
       !aligned(w_gate_up_c, 16) || !aligned(w_down_c, 16) || !aligned(router_w_c, 16) ||
       !aligned(retained_idx, 4) || !aligned(ids_c, 4))
     return SLIMWISE_ERR_UNSUPPORTED_SHAPE;
-  DeviceInfo di;
-  rc = device_info(&di);
-  if (rc) return rc;
   return launch_compact_layer(w_gate_up, w_down, router_w, retained_idx, n_retained,
-                              shape->num_experts, shape->hidden, shape->inter, di.sms,
-                              w_gate_up_c, w_down_c, router_w_c, ids_c,
+                              shape->num_experts, shape->hidden, shape->inter, w_gate_up_c, w_down_c, router_w_c, ids_c,
                               reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess
              ? SLIMWISE_OK
              : SLIMWISE_ERR_CUDA;
