@@ -561,8 +561,8 @@ cudaError_t launch_route_nc(const __nv_bfloat16 *hidden, const float *router_w,
 // spends more issue slots on loads and conversions than on multiply-adds.
 // There (route_tiled says where) the logits are a tiled product on the fp32
 // units, in the same canonical order, and a second kernel runs the top-k:
-//   route_logits_kernel  32 tokens x 16 retained experts per CTA, the K range
-//                        streamed in 128-wide chunks through a 4-stage
+//   route_logits_kernel  32 tokens (16 or 8 where those make too few CTAs) x
+//                        16 retained experts per CTA, the K range streamed in 128-wide chunks through a 4-stage
 //                        cp.async ring.  Lane l of every warp holds partial
 //                        sum l of its 8 tokens x 16 experts (128 registers),
 //                        so 24 shared-memory loads feed 256 packed
@@ -575,15 +575,14 @@ cudaError_t launch_route_nc(const __nv_bfloat16 *hidden, const float *router_w,
 // the 32 T/s that a register-only loop reaches here, two CTAs of 4 warps per
 // SM (one of 8 warps: 57 %, all of them waiting for each chunk together;
 // 16 tokens x 8 experts per warp: 70 %).
-constexpr int kTileTok = 32;
 constexpr int kTileRow = 16;
 constexpr int kTileThreads = 128;
 constexpr int kTileStages = 4;
-constexpr int kWarpTok = 8;    // tokens of one warp (4 warps: the tile's 32)
 constexpr int kWarpRow = 16;   // experts of one warp
-constexpr int kTileXBytes = kTileTok * 128 * 2;
+// WT tokens per warp (4 warps: 4 WT per tile).
 constexpr int kTileWBytes = kTileRow * 128 * 4;
-constexpr int kTileSmem = kTileStages * (kTileXBytes + kTileWBytes);
+__host__ __device__ constexpr int tile_x_bytes(int wt) { return 4 * wt * 128 * 2; }
+__host__ __device__ constexpr int tile_smem(int wt) { return kTileStages * (tile_x_bytes(wt) + kTileWBytes); }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes)
@@ -602,7 +601,8 @@ __device__ __forceinline__ void reduce_step(float (&a)[kSize], int lane) {
   }
 }
 
-__global__ void __launch_bounds__(kTileThreads, 2)
+template <int WT>
+__global__ void __launch_bounds__(kTileThreads, WT == 8 ? 2 : 3)
     route_logits_kernel(const __nv_bfloat16 *__restrict__ hidden,
                         const float *__restrict__ router_w,
                         const int32_t *__restrict__ retained, Dims d, Ws ws,
@@ -618,23 +618,28 @@ __global__ void __launch_bounds__(kTileThreads, 2)
   }
 #endif
   const int H = d.H, m = d.m_ret, nchunks = H / 128;
+  constexpr int kTileTok = 4 * WT, kTileXBytes = tile_x_bytes(WT);
+  constexpr int kXLoads = kTileTok * 16 / kTileThreads;  // WT / 2
   const int t0 = blockIdx.x * kTileTok, r0 = blockIdx.y * kTileRow;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t xs = smem_u32(smem), wsm = xs + kTileStages * kTileXBytes;
 
-  // this thread's 16-byte vectors of a chunk: four of the hidden rows (rows
+  // this thread's 16-byte vectors of a chunk: WT / 2 of the hidden rows (rows
   // tid / 16 + 8 u; tokens past the batch are zero) and four of the router
   // rows (rows warp + 4 u; rows past the pool repeat its last one and are
   // dropped at the end)
   const int xrow = tid >> 4, xcol = tid & 15;
-  const __nv_bfloat16 *xsrc[4];
+  const __nv_bfloat16 *xsrc[kXLoads];
   const float *wsrc[4];
-  uint32_t xbytes[4];
+  uint32_t xbytes[kXLoads];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < kXLoads; ++u) {
     const int t = t0 + xrow + 8 * u;
     xbytes[u] = t < d.B ? 16u : 0u;
     xsrc[u] = hidden + (size_t)(t < d.B ? t : 0) * H + xcol * 8;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
     const int r = min(r0 + warp + 4 * u, m - 1);
     const int e = min(max(retained ? __ldg(retained + r) : r, 0), d.E - 1);
     wsrc[u] = router_w + (size_t)e * H + lane * 4;
@@ -644,10 +649,9 @@ __global__ void __launch_bounds__(kTileThreads, 2)
     const uint32_t xd = xs + st * kTileXBytes + xrow * 256 + xcol * 16;
     const uint32_t wd = wsm + st * kTileWBytes + warp * 512 + lane * 16;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      cp_async16(xd + u * 8 * 256, xsrc[u] + c * 128, xbytes[u]);
-      cp_async16(wd + u * 4 * 512, wsrc[u] + c * 128, 16u);
-    }
+    for (int u = 0; u < kXLoads; ++u) cp_async16(xd + u * 8 * 256, xsrc[u] + c * 128, xbytes[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cp_async16(wd + u * 4 * 512, wsrc[u] + c * 128, 16u);
   };
 #pragma unroll
   for (int c = 0; c < kTileStages - 1; ++c) {
@@ -655,12 +659,12 @@ __global__ void __launch_bounds__(kTileThreads, 2)
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
 
-  float acc[kWarpRow][kWarpTok];
+  float acc[kWarpRow][WT];
 #pragma unroll
   for (int r = 0; r < kWarpRow; ++r)
 #pragma unroll
-    for (int t = 0; t < kWarpTok; ++t) acc[r][t] = 0.0f;
-  const unsigned char *xw = smem + (size_t)warp * kWarpTok * 256 + lane * 8;
+    for (int t = 0; t < WT; ++t) acc[r][t] = 0.0f;
+  const unsigned char *xw = smem + (size_t)warp * WT * 256 + lane * 8;
   const unsigned char *ww = smem + kTileStages * kTileXBytes + lane * 16;
   for (int c = 0; c < nchunks; ++c) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kTileStages - 2) : "memory");
@@ -668,9 +672,9 @@ __global__ void __launch_bounds__(kTileThreads, 2)
     if (c + kTileStages - 1 < nchunks) load_chunk(c + kTileStages - 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
     const int st = c % kTileStages;
-    float x[4][kWarpTok];
+    float x[4][WT];
 #pragma unroll
-    for (int t = 0; t < kWarpTok; ++t) {
+    for (int t = 0; t < WT; ++t) {
       const uint2 v = *reinterpret_cast<const uint2 *>(xw + st * kTileXBytes + t * 256);
       x[0][t] = __uint_as_float(v.x << 16);
       x[1][t] = __uint_as_float(v.x & 0xFFFF0000u);
@@ -684,30 +688,31 @@ __global__ void __launch_bounds__(kTileThreads, 2)
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int t = 0; t < kWarpTok; t += 2)
+        for (int t = 0; t < WT; t += 2)
           ffma2_acc(acc[r][t], acc[r][t + 1], x[q][t], x[q][t + 1], wq[q]);
     }
   }
 
-  // the xor butterfly (offsets 16 .. 1) of all 128 sums: at each step a lane
+  // the xor butterfly (offsets 16 .. 1) of all 16 WT sums: at each step a lane
   // keeps half of its values and hands the others to its partner; value
-  // v = 16 t + r ends on lane v / 4
-  float a[kWarpTok * kWarpRow];
+  // v = 16 t + r ends on lane v / (WT / 2)
+  constexpr int kVals = WT * kWarpRow, kOwn = WT / 2;
+  float a[kVals];
 #pragma unroll
-  for (int v = 0; v < kWarpTok * kWarpRow; ++v) a[v] = acc[v % kWarpRow][v / kWarpRow];
-  reduce_step<16, 64>(a, lane);
-  reduce_step<8, 32>(a, lane);
-  reduce_step<4, 16>(a, lane);
-  reduce_step<2, 8>(a, lane);
-  reduce_step<1, 4>(a, lane);
-  const int t = t0 + warp * kWarpTok + (lane >> 2), r = r0 + (lane & 3) * 4;
+  for (int v = 0; v < kVals; ++v) a[v] = acc[v % kWarpRow][v / kWarpRow];
+  reduce_step<16, kVals / 2>(a, lane);
+  reduce_step<8, kVals / 4>(a, lane);
+  reduce_step<4, kVals / 8>(a, lane);
+  reduce_step<2, kVals / 16>(a, lane);
+  reduce_step<1, kVals / 32>(a, lane);
+  const int t = t0 + warp * WT + lane * kOwn / kWarpRow, r = r0 + lane * kOwn % kWarpRow;
   if (t < d.B) {
     float *dst = z + (size_t)t * m + r;
-    if ((m & 3) == 0 && r + 4 <= m) {
-      *reinterpret_cast<float4 *>(dst) = make_float4(a[0], a[1], a[2], a[3]);
+    if (kOwn == 4 && (m & 3) == 0 && r + 4 <= m) {
+      *reinterpret_cast<float4 *>(dst) = make_float4(a[0], a[1 % kVals], a[2 % kVals], a[3 % kVals]);
     } else {
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < kOwn; ++u)
         if (r + u < m) dst[u] = a[u];
     }
   }
@@ -736,30 +741,38 @@ __global__ void __launch_bounds__(kRouteThreads)
 }
 
 // Which calls take the tiled kernels (where the scratch rows hold the logits).
-// A wave of the cluster kernel is 608 tokens; below that the second launch has
-// to be earned by the multiply-adds B m' H.  Whole layers, cluster kernel
-// against tiled, H = 2048 unless said: m' = 128: B = 256 188.1 / 189.1 us,
-// 304 197.5 / 190.2, 512 205.1 / 202.0, 8192 828 / 727; m' = 256: B = 96
-// 233.2 / 232.9, 160 251.2 / 244.2, 8192 912 / 747; m' = 64: B = 400 112.2 /
-// 113.7, 500 116.7 / 116.8, 640 129.4 / 121.8; m' = 96: B = 304 155.9 / 150.5;
-// m' = 32: B = 513 76.4 / 80.1, 640 88.9 / 84.8; H = 4096, m' = 128: B = 200
-// 97.2 / 91.6.  Above 256 tokens the cluster kernel's clusters no longer all
-// find room at once, so less work earns it.  Pools above 256 experts gain from
-// a few tokens on: m' = 512, B = 32 77.6 / 75.4; m' = 1024, B = 16 93.4 / 85.8.
+// Above 256 tokens the cluster kernel's clusters no longer find room all at
+// once, and every cluster evaluates the whole pool; below, the second launch
+// has to be earned.  Whole layers at H = 2048, cluster kernel / tiled, us:
+//   m' = 32    B = 256  64.9 / 65.8    400  70.7 / 70.2    600  85.8 / 79.5
+//   m' = 64    B = 256 105.4 / 106.0   304 114.5 / 107.8   500 116.5 / 114.1
+//   m' = 128   B = 128 182.0 / 182.8   200 187.6 / 186.5   304 197.5 / 189.4
+//   m' = 256   B = 16  101.0 / 101.6    64 206.1 / 204.8   128 239.1 / 237.3
+//   m' = 512   B = 4    40.2 / 38.1     32  72.1 / 67.4
+//   m' = 1024  B = 1    66.0 / 56.2     16  89.1 / 77.6
+// and B = 8192: m' = 128 828 / 727, m' = 256 912 / 747.
 inline bool route_tiled(const Dims &d) {
   if ((size_t)d.m_ret * 4 > (size_t)d.k * d.H * 2) return false;
-  const double logits = (double)d.B * d.m_ret;
-  return d.B > 608 || logits * d.H >= (d.B > 256 ? 55e6 : 68e6) ||
-         (d.m_ret > 256 && logits >= 16384);
+  return d.B > 256 || d.m_ret > 256 ||
+         (long long)d.B * d.m_ret >= (d.m_ret > 128 ? 16384 : 24576);
 }
 
 cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_w,
-                               const int32_t *retained, Dims d, Ws ws, bool pdl,
+                               const int32_t *retained, Dims d, Ws ws, bool pdl, int sms,
                                cudaStream_t stream) {
   // the logits go where the call's expert outputs will be (route_tiled)
   float *z = reinterpret_cast<float *>(ws.y);
-  cudaError_t err = cudaFuncSetAttribute(
-      route_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
+  // the smallest tiles that still leave at most one CTA per SM, the largest
+  // ones where there are more (m' = 64, tiles of 32, 16 and 8 tokens: B = 256
+  // 109.0 / 106.3 / 106.0 us, B = 500 116.5 / 114.1 / 114.2; m' = 128, B = 512
+  // 201.2 / 202.5 / 205.0)
+  const int row_tiles = (d.m_ret + kTileRow - 1) / kTileRow;
+  int wt = 2;
+  while (wt < 8 && (d.B + 4 * wt - 1) / (4 * wt) * row_tiles > sms) wt *= 2;
+  auto logits = wt == 8 ? route_logits_kernel<8>
+                : wt == 4 ? route_logits_kernel<4> : route_logits_kernel<2>;
+  cudaError_t err = cudaFuncSetAttribute(logits, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         tile_smem(wt));
   if (err != cudaSuccess) return err;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -768,10 +781,10 @@ cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  cfg.gridDim = dim3((d.B + kTileTok - 1) / kTileTok, (d.m_ret + kTileRow - 1) / kTileRow);
+  cfg.gridDim = dim3((d.B + 4 * wt - 1) / (4 * wt), row_tiles);
   cfg.blockDim = dim3(kTileThreads);
-  cfg.dynamicSmemBytes = kTileSmem;
-  err = cudaLaunchKernelEx(&cfg, route_logits_kernel, hidden, router_w, retained, d, ws, z);
+  cfg.dynamicSmemBytes = tile_smem(wt);
+  err = cudaLaunchKernelEx(&cfg, logits, hidden, router_w, retained, d, ws, z);
   if (err != cudaSuccess) return err;
   cfg.gridDim = dim3((d.B + kRouteWarps - 1) / kRouteWarps);
   cfg.blockDim = dim3(kRouteThreads);
@@ -785,10 +798,15 @@ cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_
 cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w,
                               const int32_t *retained, Dims d, Ws ws, bool pdl,
                               cudaStream_t stream) {
-  if (route_tiled(d)) return launch_route_tiled(hidden, router_w, retained, d, ws, pdl, stream);
   int dev = 0, optin = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
+  if (route_tiled(d)) {
+    int sms = 0;
+    err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (err != cudaSuccess) return err;
+    return launch_route_tiled(hidden, router_w, retained, d, ws, pdl, sms, stream);
+  }
   err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (err != cudaSuccess) return err;
   // wide hidden rows: fewer tokens per cluster until they fit in shared memory

@@ -72,11 +72,11 @@ def test_layer_large_batches(H, E, I, k, B, shared):
     assert np.array_equal(r["topk_idx"].cpu().numpy(), ref["idx"])
 
 
-# Tiled routing (more than 608 tokens, or enough work) in 32-token x 16-expert
-# tiles with ragged edges, the three top-k forms, a pool whose logits do not
+# Tiled routing in tiles of 32, 16 and 8 tokens x 16 experts with ragged edges, the three top-k forms, a pool whose logits do not
 # fit the scratch rows (the cluster kernel keeps it), any order of the ids
 @pytest.mark.parametrize("H,E,k,B,m_prime", [(256, 16, 2, 609, 8), (2048, 512, 8, 33, 511),
-                                             (2048, 128, 8, 257, 121), (640, 40, 3, 769, 33),
+                                             (2048, 1024, 8, 1, 1024), (2048, 128, 8, 257, 121),
+                                             (256, 16, 2, 5000, 8), (640, 40, 3, 769, 33),
                                              (2048, 128, 8, 800, 128), (384, 256, 8, 1055, 201),
                                              (256, 512, 32, 777, 300), (128, 1024, 1, 800, 1024)])
 def test_tiled_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
@@ -91,7 +91,7 @@ def test_tiled_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
     np.testing.assert_allclose(r["topk_gate"].cpu().numpy(), gates, rtol=4e-6, atol=1e-7)
     # bit for bit what the cluster kernel gives (small batches), special values
     # among them
-    xd[5], xd[B - 1, 7], xd[30, 9] = 0.0, float("inf"), float("nan")
+    xd[5 % B], xd[B - 1, 7], xd[30 % B, 9] = 0.0, float("inf"), float("nan")
     r = sw.slimwise_moe_route(xd, wd, rd, k, E)
     step = 28
     for t0 in range(0, B, step):
