@@ -170,7 +170,7 @@ struct Ws {
   __nv_bfloat16 *act;  // [B*k, I] SwiGLU activations in grouped order
   __nv_bfloat16 *y;    // [B*k, H] expert outputs in grouped order
   float *shared_gate;  // [B] sigmoid gate of the shared expert
-  __nv_bfloat16 *xt;   // [B, H] hidden rows, token order (shared-expert input)
+  __nv_bfloat16 *xt;   // [B, H] hidden rows, token order (shared expert in pair items)
   __nv_bfloat16 *act_s;  // [B, Is] shared-expert activations, token order
   __nv_bfloat16 *y_s;  // [B, H] shared-expert outputs, token order
 };
@@ -277,12 +277,14 @@ struct FfnMaps {
   // token rows: box 64 x 16 (m + 1), or 64 x 8 (m + 1) for pair items (each
   // CTA of the pair loads half of an item's rows)
   CUtensorMap xp[kTokBoxSizes];     // [B*k rows, H cols] bf16
-  CUtensorMap hid;                  // the caller's hidden rows [B, H], box 64 x tok_chunk (local)
+  // the caller's hidden rows [B, H], box 64 x tok_chunk: a local call's tokens,
+  // and the shared expert's
+  CUtensorMap hid;
   CUtensorMap act[kTokBoxSizes];    // [B*k rows, I cols] bf16
   // shared expert (encoded only when there is one)
   CUtensorMap w_gu_s;               // [1, 2Is, H] bf16
   CUtensorMap w_down_s;             // [1, H, Is] bf16
-  CUtensorMap xt[kTokBoxSizes];     // [B rows, H cols] bf16, hidden in token order
+  CUtensorMap xt[kTokBoxSizes];     // [B rows, H cols] bf16, hidden in token order (pairs)
   CUtensorMap act_s[kTokBoxSizes];  // [B rows, Is cols] bf16, token order
 };
 

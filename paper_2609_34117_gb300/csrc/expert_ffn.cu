@@ -545,12 +545,12 @@ __global__ void __maxnreg__(128)
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&maps.w_gu);
     tma_prefetch_desc(&maps.w_down);
-    if constexpr (kLocal) tma_prefetch_desc(&maps.hid);
+    if constexpr (kLocal || (kShared && !kPair)) tma_prefetch_desc(&maps.hid);
     for (int m = 0; m < kTokBoxSizes && kTokBox * (m + 1) <= d.tok_chunk; ++m) {
       if constexpr (!kLocal) tma_prefetch_desc(&maps.xp[m]);
       tma_prefetch_desc(&maps.act[m]);
       if constexpr (kShared) {
-        if constexpr (!kLocal) tma_prefetch_desc(&maps.xt[m]);
+        if constexpr (kPair) tma_prefetch_desc(&maps.xt[m]);
         tma_prefetch_desc(&maps.act_s[m]);
       }
     }
@@ -792,7 +792,10 @@ __global__ void __maxnreg__(128)
         bmap = it.down ? (const void *)&maps.act[box_m] : (const void *)&maps.xp[box_m];
         expert = it.expert;
       }
-      if (kLocal && !it.down) bmap = (const void *)&maps.hid;  // the batch, in token order
+      // the batch in token order, straight from the caller's hidden rows: boxes
+      // of tok_chunk rows
+      const bool from_hidden = !it.down && (kLocal || (kShared && !kPair && it.shared));
+      if (from_hidden) bmap = (const void *)&maps.hid;
       if (kAhead && lane == 0) next = n_first + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
       if (it.down && !ready) {
         // the entry's activations must be complete: all its gate/up tiles
@@ -820,7 +823,8 @@ __global__ void __maxnreg__(128)
       // bytes the stage barrier expects: for a pair, both CTAs' copies
       const uint32_t stage_tx =
           kPair ? (uint32_t)(2 * kATileBytes + n16 * kTokBox * kBlockK * 2)
-                : (uint32_t)(halves * kATileBytes + n16 * kTokBox * kBlockK * 2);
+                : (uint32_t)(halves * kATileBytes +
+                             (from_hidden ? d.tok_chunk : n16 * kTokBox) * kBlockK * 2);
       bool ok = true;
       for (int kc = 0; kc < nk; ++kc) {
         if (kAhead && kc == (2 * nk) / 3) {

@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(kGroupThreads)
         const int tt = i / vecs, vv = i % vecs;
         for (int j = 0; j < k; ++j)
           reinterpret_cast<uint4 *>(ws.xp + (size_t)my_pos[tt * k + j] * H)[vv] = hv[u];
-        // token-order copy for the shared expert (a stable address to map)
-        if (d.Is > 0) reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + tt) * H)[vv] = hv[u];
+        // pair items take the shared expert's rows from a token-order copy
+        if (d.Is > 0 && d.pair) reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + tt) * H)[vv] = hv[u];
       }
     }
   } else if (do_gather) {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kGroupThreads)
         if (i0 + u * blockDim.x < nt * vecs) {
           for (int j = 0; j < k; ++j)
             reinterpret_cast<uint4 *>(ws.xp + (size_t)my_pos[tt[u] * k + j] * H)[vv[u]] = v[u];
-          if (d.Is > 0) reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + tt[u]) * H)[vv[u]] = v[u];
+          if (d.Is > 0 && d.pair) reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + tt[u]) * H)[vv[u]] = v[u];
         }
       }
     }
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kGroupThreads)
     __syncthreads();
     if (do_gather) {
       // each hidden row of the part to its k grouped positions (and, for the
-      // shared expert, to its token-order copy): a warp takes 128 vectors of
+      // shared expert of pair items, to its token-order copy): a warp takes 128 vectors of
       // a row, its four loads issued before the stores
       constexpr int kVec = 4;
       const int groups = (vecs + 32 * kVec - 1) / (32 * kVec);
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kGroupThreads)
           for (int u = 0; u < kVec; ++u)
             if (v0 + 32 * u < vecs) dst[v0 + 32 * u] = v[u];
         }
-        if (d.Is > 0) {
+        if (d.Is > 0 && d.pair) {
           uint4 *dst = reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + p0 + tt) * H);
 #pragma unroll
           for (int u = 0; u < kVec; ++u)

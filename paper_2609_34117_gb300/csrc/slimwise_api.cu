@@ -243,7 +243,7 @@ bool ffn_maps_for(FfnMaps *maps, const void *hidden, const void *w_gate_up, cons
       if ((!d.local && encode_map(&cached.xp[b], w.xp, slots, d.H, rows)) ||
           encode_map(&cached.act[b], w.act, slots, d.I, rows))
         return false;
-      if (d.Is > 0 && ((!d.local && encode_map(&cached.xt[b], w.xt, (uint64_t)d.B, d.H, rows)) ||
+      if (d.Is > 0 && ((d.pair && encode_map(&cached.xt[b], w.xt, (uint64_t)d.B, d.H, rows)) ||
                        encode_map(&cached.act_s[b], w.act_s, (uint64_t)d.B, d.Is, rows)))
         return false;
     }
@@ -252,7 +252,9 @@ bool ffn_maps_for(FfnMaps *maps, const void *hidden, const void *w_gate_up, cons
   }
   // the hidden rows' map is made for each call: a program's hidden states
   // need not stay at one address
-  if (d.local && encode_map(&cached.hid, hidden, (uint64_t)d.B, d.H, (uint32_t)d.tok_chunk))
+  if ((d.local || (d.Is > 0 && !d.pair)) &&
+      encode_map(&cached.hid, hidden, (uint64_t)d.B, d.H,
+                 (uint32_t)d.tok_chunk))
     return false;
   *maps = cached;
   return true;
