@@ -101,7 +101,7 @@ enum TraceSlot {
 // Byte offsets of every workspace region (all 1024-byte aligned).
 struct WsLayout {
   size_t ctrl, topk_idx, topk_gate, counts, offsets, union_ids, entries,
-      entry_done, perm, pos, xp, act, y, shared_gate, xt, act_s, y_s, total;
+      entry_done, perm, pos, xp, act, y, shared_gate, spare, act_s, y_s, total;
   int32_t max_entries;
 };
 
@@ -144,11 +144,11 @@ inline WsLayout make_layout(int B, int H, int E, int I, int k, int Is = 0) {
   L.y = take(slots * H * 2);
   if (Is > 0) {
     L.shared_gate = take((size_t)B * 4);
-    L.xt = take((size_t)B * H * 2);
+    L.spare = take((size_t)B * H * 2);  // not used: part of the size callers know
     L.act_s = take((size_t)B * Is * 2);
     L.y_s = take((size_t)B * H * 2);
   } else {  // no shared expert: no space (these regions are never accessed)
-    L.shared_gate = L.xt = L.act_s = L.y_s = o;
+    L.shared_gate = L.spare = L.act_s = L.y_s = o;
   }
   L.total = o;
   return L;
@@ -170,7 +170,6 @@ struct Ws {
   __nv_bfloat16 *act;  // [B*k, I] SwiGLU activations in grouped order
   __nv_bfloat16 *y;    // [B*k, H] expert outputs in grouped order
   float *shared_gate;  // [B] sigmoid gate of the shared expert
-  __nv_bfloat16 *xt;   // [B, H] hidden rows, token order (shared expert in pair items)
   __nv_bfloat16 *act_s;  // [B, Is] shared-expert activations, token order
   __nv_bfloat16 *y_s;  // [B, H] shared-expert outputs, token order
 };
@@ -192,7 +191,6 @@ inline Ws make_ws(void *base, const WsLayout &L) {
   w.act = (__nv_bfloat16 *)(b + L.act);
   w.y = (__nv_bfloat16 *)(b + L.y);
   w.shared_gate = (float *)(b + L.shared_gate);
-  w.xt = (__nv_bfloat16 *)(b + L.xt);
   w.act_s = (__nv_bfloat16 *)(b + L.act_s);
   w.y_s = (__nv_bfloat16 *)(b + L.y_s);
   return w;
@@ -284,7 +282,6 @@ struct FfnMaps {
   // shared expert (encoded only when there is one)
   CUtensorMap w_gu_s;               // [1, 2Is, H] bf16
   CUtensorMap w_down_s;             // [1, H, Is] bf16
-  CUtensorMap xt[kTokBoxSizes];     // [B rows, H cols] bf16, hidden in token order (pairs)
   CUtensorMap act_s[kTokBoxSizes];  // [B rows, Is cols] bf16, token order
 };
 

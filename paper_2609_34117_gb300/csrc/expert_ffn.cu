@@ -484,7 +484,7 @@ __global__ void __maxnreg__(128)
                       uint64_t timeout_ns,
                       int starve_first_down) {
   constexpr bool kLocal = kLocalWords > 0;
-  static_assert(!(kPair && kWide), "a pair item is a 128-row tile in each CTA");
+  static_assert(!(kPair && (kShared || kWide)), "pair items are routed 128-row tiles");
   static_assert(!(kAhead && kPair), "a pair's items are handed from CTA to CTA");
   static_assert(!(kLocal && (kWide || kPair || kAhead)), "small batches take plain items");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -545,12 +545,11 @@ __global__ void __maxnreg__(128)
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&maps.w_gu);
     tma_prefetch_desc(&maps.w_down);
-    if constexpr (kLocal || (kShared && !kPair)) tma_prefetch_desc(&maps.hid);
+    if constexpr (kLocal || kShared) tma_prefetch_desc(&maps.hid);
     for (int m = 0; m < kTokBoxSizes && kTokBox * (m + 1) <= d.tok_chunk; ++m) {
       if constexpr (!kLocal) tma_prefetch_desc(&maps.xp[m]);
       tma_prefetch_desc(&maps.act[m]);
       if constexpr (kShared) {
-        if constexpr (kPair) tma_prefetch_desc(&maps.xt[m]);
         tma_prefetch_desc(&maps.act_s[m]);
       }
     }
@@ -784,7 +783,7 @@ __global__ void __maxnreg__(128)
         // the shared expert: its own weights, tokens in batch order
         nk = it.down ? d.Is / kBlockK : d.H / kBlockK;
         amap = it.down ? (const void *)&maps.w_down_s : (const void *)&maps.w_gu_s;
-        bmap = it.down ? (const void *)&maps.act_s[box_m] : (const void *)&maps.xt[box_m];
+        bmap = (const void *)&maps.act_s[box_m];
         expert = 0;
       } else {
         nk = it.down ? d.I / kBlockK : d.H / kBlockK;
@@ -794,7 +793,7 @@ __global__ void __maxnreg__(128)
       }
       // the batch in token order, straight from the caller's hidden rows: boxes
       // of tok_chunk rows
-      const bool from_hidden = !it.down && (kLocal || (kShared && !kPair && it.shared));
+      const bool from_hidden = !it.down && (kLocal || (kShared && it.shared));
       if (from_hidden) bmap = (const void *)&maps.hid;
       if (kAhead && lane == 0) next = n_first + atomicAdd(&ws.ctrl[kCtrlWorkCounter], 1);
       if (it.down && !ready) {
@@ -1267,15 +1266,13 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
   if (d.wide && (d.Is > 0 || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0 ||
                  d.tok_chunk > 128))
     return cudaErrorInvalidValue;
-  // pair items on whole 256-row tiles too, and never together with wide ones
-  if (d.pair && (d.wide || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0 ||
-                 d.Is % (2 * kGateRows) != 0))
+  // pair items likewise, and never together with wide ones
+  if (d.pair && (d.wide || d.Is > 0 || d.I % (2 * kGateRows) != 0 || d.H % (2 * kTileRows) != 0))
     return cudaErrorInvalidValue;
   const bool ahead = d.tok_chunk >= kAheadMinChunk;
   const int words = local_words(d);
   auto kernel = d.Is > 0 ? (words == 2  ? expert_ffn_kernel<true, false, false, false, 2>
                             : words == 4 ? expert_ffn_kernel<true, false, false, false, 4>
-                            : d.pair     ? expert_ffn_kernel<true, false, true, false, 0>
                             : ahead      ? expert_ffn_kernel<true, false, false, true, 0>
                                          : expert_ffn_kernel<true, false, false, false, 0>)
                 : words == 2 ? expert_ffn_kernel<false, false, false, false, 2>

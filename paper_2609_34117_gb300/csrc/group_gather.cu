@@ -231,8 +231,6 @@ __global__ void __launch_bounds__(kGroupThreads)
         const int tt = i / vecs, vv = i % vecs;
         for (int j = 0; j < k; ++j)
           reinterpret_cast<uint4 *>(ws.xp + (size_t)my_pos[tt * k + j] * H)[vv] = hv[u];
-        // pair items take the shared expert's rows from a token-order copy
-        if (d.Is > 0 && d.pair) reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + tt) * H)[vv] = hv[u];
       }
     }
   } else if (do_gather) {
@@ -254,7 +252,6 @@ __global__ void __launch_bounds__(kGroupThreads)
         if (i0 + u * blockDim.x < nt * vecs) {
           for (int j = 0; j < k; ++j)
             reinterpret_cast<uint4 *>(ws.xp + (size_t)my_pos[tt[u] * k + j] * H)[vv[u]] = v[u];
-          if (d.Is > 0 && d.pair) reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + tt[u]) * H)[vv[u]] = v[u];
         }
       }
     }
@@ -408,8 +405,7 @@ __global__ void __launch_bounds__(kGroupThreads)
     }
     __syncthreads();
     if (do_gather) {
-      // each hidden row of the part to its k grouped positions (and, for the
-      // shared expert of pair items, to its token-order copy): a warp takes 128 vectors of
+      // each hidden row of the part to its k grouped positions: a warp takes 128 vectors of
       // a row, its four loads issued before the stores
       constexpr int kVec = 4;
       const int groups = (vecs + 32 * kVec - 1) / (32 * kVec);
@@ -422,12 +418,6 @@ __global__ void __launch_bounds__(kGroupThreads)
           if (v0 + 32 * u < vecs) v[u] = __ldg(src + v0 + 32 * u);
         for (int j = 0; j < k; ++j) {
           uint4 *dst = reinterpret_cast<uint4 *>(ws.xp + (size_t)pos_s[tt * k + j] * H);
-#pragma unroll
-          for (int u = 0; u < kVec; ++u)
-            if (v0 + 32 * u < vecs) dst[v0 + 32 * u] = v[u];
-        }
-        if (d.Is > 0 && d.pair) {
-          uint4 *dst = reinterpret_cast<uint4 *>(ws.xt + (size_t)(t0 + p0 + tt) * H);
 #pragma unroll
           for (int u = 0; u < kVec; ++u)
             if (v0 + 32 * u < vecs) dst[v0 + 32 * u] = v[u];

@@ -128,8 +128,8 @@ Dims make_dims(const slimwise_moe_shape *s, int32_t top_k, int32_t m_ret, int32_
   d.m_ret = m_ret;
   d.Is = Is;
   // CTA-pair items only on request
-  d.pair = (form > 0 && d.I % (2 * kGateRows) == 0 && d.H % (2 * kTileRows) == 0 &&
-            Is % (2 * kGateRows) == 0) ? 1 : 0;
+  d.pair = (form > 0 && Is == 0 && d.I % (2 * kGateRows) == 0 && d.H % (2 * kTileRows) == 0)
+               ? 1 : 0;
   d.local = (d.B <= kLocalTokens && !d.pair && !grouped) ? 1 : 0;
   d.tok_chunk = token_chunk_for(d.B, top_k, m_ret);
   if (d.local) {
@@ -201,12 +201,12 @@ struct WeightMapsKey {
   }
 };
 struct TokenMapsKey {
-  const void *xp, *act, *xt, *act_s;
+  const void *xp, *act, *act_s;
   int H, I, Is, B, tok_chunk, pair, local, device;
   uint64_t slots;
   bool operator==(const TokenMapsKey &o) const {
-    return xp == o.xp && act == o.act && xt == o.xt && act_s == o.act_s && H == o.H &&
-           I == o.I && Is == o.Is && B == o.B && tok_chunk == o.tok_chunk && pair == o.pair &&
+    return xp == o.xp && act == o.act && act_s == o.act_s && H == o.H && I == o.I &&
+           Is == o.Is && B == o.B && tok_chunk == o.tok_chunk && pair == o.pair &&
            local == o.local && device == o.device && slots == o.slots;
   }
 };
@@ -220,7 +220,7 @@ bool ffn_maps_for(FfnMaps *maps, const void *hidden, const void *w_gate_up, cons
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   const WeightMapsKey kw = {w_gate_up, w_down, se.gate_up, se.down, d.E, d.H, d.I, d.Is, dev};
-  const TokenMapsKey kt = {w.xp, w.act, w.xt, w.act_s, d.H, d.I, d.Is, d.B, d.tok_chunk, d.pair,
+  const TokenMapsKey kt = {w.xp, w.act, w.act_s, d.H, d.I, d.Is, d.B, d.tok_chunk, d.pair,
                           d.local, dev, slots};
   if (!(have_w && kw == last_w)) {
     have_w = false;
@@ -243,8 +243,7 @@ bool ffn_maps_for(FfnMaps *maps, const void *hidden, const void *w_gate_up, cons
       if ((!d.local && encode_map(&cached.xp[b], w.xp, slots, d.H, rows)) ||
           encode_map(&cached.act[b], w.act, slots, d.I, rows))
         return false;
-      if (d.Is > 0 && ((d.pair && encode_map(&cached.xt[b], w.xt, (uint64_t)d.B, d.H, rows)) ||
-                       encode_map(&cached.act_s[b], w.act_s, (uint64_t)d.B, d.Is, rows)))
+      if (d.Is > 0 && encode_map(&cached.act_s[b], w.act_s, (uint64_t)d.B, d.Is, rows))
         return false;
     }
     last_t = kt;
@@ -252,7 +251,7 @@ bool ffn_maps_for(FfnMaps *maps, const void *hidden, const void *w_gate_up, cons
   }
   // the hidden rows' map is made for each call: a program's hidden states
   // need not stay at one address
-  if ((d.local || (d.Is > 0 && !d.pair)) &&
+  if ((d.local || d.Is > 0) &&
       encode_map(&cached.hid, hidden, (uint64_t)d.B, d.H,
                  (uint32_t)d.tok_chunk))
     return false;
