@@ -121,7 +121,7 @@ int slimwise_moe_decode_full(const void *hidden, const float *router_w,
  *                        the expert-FFN kernel and after the combine kernel
  *                        that follows it (NULL: none); used to time the two
  *                        alone.
- *   disable_pdl          1: launch the layer's four kernels with plain stream
+ *   disable_pdl          1: launch the layer's kernels with plain stream
  *                        ordering instead of programmatic dependent launch.
  *   grid_ctas            >0: persistent expert-FFN grid size (default: the
  *                        device's SM count).

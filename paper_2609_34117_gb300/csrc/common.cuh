@@ -68,7 +68,9 @@ __host__ __device__ inline int token_box_for(int n16) { return n16 - 1; }
 constexpr int kMinTokChunk = 16;     // smallest token_chunk_for(): bounds the entry count
 // Tokens per routing cluster.  One wave of routing CTAs (two per SM) holds
 // 38 clusters: above 152 tokens clusters of 4 need two waves, so every pool
-// takes 8 tokens per cluster there; above 304 tokens 16, staged as bf16.
+// takes 8 tokens per cluster there.  (Above 256 tokens only layers whose
+// logits do not fit the scratch rows still come here: 16 above 304, staged as
+// bf16.)
 inline int route_tokens_per_cluster(int B, int m_ret) {
   (void)m_ret;
   if (B <= 32) return 1;

@@ -10,23 +10,24 @@
 // epilogue warps.
 //
 // One persistent CTA per SM (320 threads):
-//   warp 0   producer (one thread): takes work items from a global counter,
-//            waits for a down item's activations, and issues each stage's
-//            copies -- the 128-row weight tile (two 64-row boxes) and the
-//            item's token rows (one box, its height the token count rounded
-//            up to 16 rows).  Each copy costs the issuing thread about 40 ns
-//            (a streaming probe), so a stage takes three copies whatever the
-//            number of tokens and the descriptors are chosen once per item;
-//            at that count the copy rate no longer bounds the kernel (a
-//            second issuing warp for the token box changed nothing).
-//   warp 1   MMA issuer (one thread) and TMEM owner; double-buffered
-//            accumulators so the epilogue of one item overlaps the next.
+//   warp 0   producer: takes work items from a global counter, decodes each
+//            once (the others read it from shared memory), waits for a down
+//            item's activations, and issues each stage's copies -- the
+//            128-row weight tile (two 64-row boxes) and the item's token rows
+//            (one box, its height the token count rounded up to 16 rows).
+//            The whole warp runs the loop and one elected thread issues, so
+//            the copies' operands stay in uniform registers; run by lane 0
+//            alone, decode steps were 1.5-4 us slower (B = 96 with the shared
+//            expert 141.9 against 137.8 us, an 8-layer stack 815 against 798).
+//   warp 1   MMA issuer (the same way) and TMEM owner; double-buffered
+//            accumulators so the epilogue of one item overlaps the next.  One
+//            commit per stage: a second one costs 70-140 cycles.
 //   warps 2-9 two epilogue warpgroups; group g handles the items of
 //            accumulator buffer g (every other item).
 // Work items, all of gate/up before any of down (so a down item only waits
 // for work that has already been handed out):
 //   gate/up (entry, i-tile): A = 64 gate rows + the matching 64 up rows of
-//            W_gu[e], K = H; epilogue computes act = SiLU(gate) * up (fp32),
+//            W_gu[e], alternating in groups of 8, K = H; epilogue computes act = SiLU(gate) * up (fp32),
 //            stores bf16 act in grouped order and counts the tile done.
 //   down    (entry, h-tile): A = 128 rows of W_down[e], K = I, B = act of the
 //            entry's tokens (after all its gate/up tiles are done); epilogue
@@ -582,8 +583,8 @@ __global__ void __maxnreg__(128)
       raise_abort(abort, ws, SLIMWISE_DEVERR_TMEM_PAIR);
   }
 
-  // While the grouping kernel runs (this grid may already be resident), warm
-  // L2 with this CTA's likely first work item: the gate/up tile that item
+  // While the routing or grouping kernel runs (this grid may already be
+  // resident), warm L2 with this CTA's likely first work item: the gate/up tile that item
   // number blockIdx.x (for a pair, the cluster's number) has when each
   // retained expert is selected and takes one entry.  The work list runs in
   // ascending expert order, so entry j is then the j-th retained expert
@@ -591,7 +592,8 @@ __global__ void __maxnreg__(128)
   // pool once B k >= 2 m'.  The guess uses only this call's inputs, so it is
   // as good for a stack of different layers as for one layer called again
   // (guessing from the previous call's work list cost a 10-layer skewed stack
-  // 3.8 %).  A wide item warms only its first 64 gate and 64 up rows: all of
+  // 3.8 %).  Without it steps of 16 to 256 tokens are 2-5 us slower (m' = 64
+  // B = 256 103.4 / 108.8 us).  A wide item warms only its first 64 gate and 64 up rows: all of
   // them would be 152 MB, more than L2 holds; each CTA of a pair warms its
   // own 64 gate and 64 up rows.  Prefetches only, every index bounded, so a
   // wrong guess costs bandwidth, never correctness.
@@ -613,7 +615,7 @@ __global__ void __maxnreg__(128)
     }
   }
 
-  // Everything below reads the grouping kernel's results.
+  // Everything below reads the routing and grouping kernels' results.
   pdl_wait_primary();
   // Above 64 tokens the combine kernel that follows may become resident now
   // (it waits for this grid to finish): measured 2-4 us faster per step at

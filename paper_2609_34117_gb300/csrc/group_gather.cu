@@ -24,6 +24,9 @@
 
 namespace slimwise {
 
+// Layers of at most 96 tokens do without this kernel (expert_ffn.cu), except
+// for statistics, pair items and routing-only calls.
+//
 // Tokens per CTA: one up to 64 tokens, two above.  Fewer tokens per CTA
 // spread the grouped-row copy over more SMs (one against two: up to 1.1 us a
 // step faster at B = 8-64), but every CTA recounts the whole batch's

@@ -2,6 +2,10 @@
 // renormalised gates (SlimWise Sec. 3.1, Eq. 2 and the renormalisation that
 // follows it).
 //
+// Two forms, chosen by route_tiled: small batches take the cluster kernel that
+// follows, larger ones (and large pools) a tiled product and a selecting
+// kernel further down.  Both give the same bits.
+//
 // A thread-block cluster of kClusterCtas CTAs handles TB tokens.  CTA r of
 // the cluster evaluates the logits of its slice of the retained experts for
 // those tokens and writes each one, through distributed shared memory, into
@@ -343,7 +347,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2)
   }
   // The inputs may come from the previous kernel on the stream.
   pdl_wait_primary();
-  // Let the grouping kernel become resident; it waits for this grid to end.
+  // Let the next kernel become resident; it waits for this grid to end.
   pdl_launch_dependents();
 #ifdef SLIMWISE_TRACE
   const int tr_step = ws.ctrl[kCtrlTraceStep];

@@ -2,7 +2,7 @@
 outputs bit for bit.
 
 A serving engine records a decode step once and replays it; the layer's
-launches (four kernels chained with programmatic dependent launch, their TMA
+launches (three or four kernels chained with programmatic dependent launch, their TMA
 descriptors passed by value) must replay correctly with new inputs copied
 into the captured buffers.  The kernels are deterministic, so the replayed
 outputs must equal the eager ones exactly.
