@@ -799,17 +799,513 @@ cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_
   return cudaLaunchKernelEx(&cfg, select, retained, d, ws, (const float *)z);
 }
 
+// --------------------------------------------------------------------------
+// Large batches on large pools
+// --------------------------------------------------------------------------
+// Only the k largest logits of a token are used, so there (route_filtered says
+// where) the tensor cores bound all of them and the fp32 units evaluate, in the
+// canonical order, only those that can be among the k:
+//   route_bound_kernel   128 tokens x 128 retained experts per CTA, tcgen05:
+//                        the router rows as a sum of two bf16 rows (split when
+//                        loaded), fp32 accumulation.  Writes the approximate
+//                        logits and the router rows' squared norms to scratch.
+//   route_refine_kernel  one warp per token: the k-th largest approximate
+//                        logit T of distinct experts, the canonical logit of
+//                        every expert whose approximate one reaches T - 2 b,
+//                        and the top-k of those.
+// b bounds |approximate - canonical| (filter_bound): k experts have canonical
+// logits of at least T - b, an expert left out has less, so the selections,
+// the gates and the order are the canonical ones bit for bit.  Where no bound
+// holds (a value that is not finite, norms that over- or underflow, fewer than
+// k distinct experts) every logit of the token is evaluated.
+// The bounding kernel (12 us at 4001 tokens x 128 experts) waits for its loads;
+// the refining one reads k router rows per token from L2, which bounds it at
+// large batches (8192 tokens x 256 experts: 0.55 GB), and is a chain of a few
+// such round trips at small ones.
+constexpr int kBoundThreads = 288;          // 8 loading / storing warps, 1 MMA warp
+constexpr int kBoundLoaders = 256;
+constexpr int kBoundTile = 128;             // tokens, and experts, of a CTA
+constexpr int kBoundK = 64;
+constexpr int kBoundOperand = kBoundTile * kBoundK * 2;
+constexpr int kBoundStages = 4;
+constexpr int kBoundParts = 4;              // most shares of K
+constexpr int kBoundSmem = kBoundStages * 3 * kBoundOperand + 1024;
+
+// Bound of |approximate - canonical logit| over the product of the norms of the
+// hidden and the router row (so of sum |x w|, by Cauchy-Schwarz):
+//   2^-17         the part of a weight that neither bf16 term holds (at most
+//                 2^-18 of it);
+//   (H/8) 2^-21   the tensor core's sum: one step per 16 elements of each term,
+//                 allowed 2^-21 of the sum of magnitudes (four units of fp32
+//                 truncation) each;
+//   (H/32+6) 2^-23  the canonical sum's own rounding, at least twice over.
+// Largest |approximate - exact| seen, of this bound: 0.4 % with normal rows, 3 %
+// with elements over e^+-6, 6 % with rows of one sign (H = 8192).
+__device__ __forceinline__ float filter_bound(int H) {
+  return 0x1p-17f + (float)(H / 8) * 0x1p-21f + (float)(H / 32 + 6) * 0x1p-23f;
+}
+
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c,
+                                             uint32_t e) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(e)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+__global__ void __launch_bounds__(kBoundThreads, 1)
+    route_bound_kernel(const __nv_bfloat16 *__restrict__ hidden,
+                       const float *__restrict__ router_w,
+                       const int32_t *__restrict__ retained, Dims d, Ws ws,
+                       float *__restrict__ z, float *__restrict__ norm2) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long bars[2 * kBoundStages + 1];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (kBoundStages + s); };
+  const uint32_t done_bar = bar0 + 8u * (2 * kBoundStages);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int s = 0; s < kBoundStages; ++s) {
+      mbar_init(full_bar(s), kBoundLoaders / 32);
+      mbar_init(empty_bar(s), 1);
+    }
+    mbar_init(done_bar, 1);
+    abort_flag = 0;
+    mbar_fence_init();
+  }
+  if (warp == 8) {
+    tmem_alloc(smem_u32(&tmem_slot), kBoundTile);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&tmem_slot);
+  volatile int *abort = &abort_flag;
+  pdl_wait_primary();
+  pdl_launch_dependents();
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
+    const int tr_step = ws.ctrl[kCtrlTraceStep];
+    trace_stamp(ws, tr_step, kTrRouteStart);
+    reinterpret_cast<uint64_t *>(ws.ctrl + kCtrlWords)[(tr_step & (kTraceSteps - 1)) * kTrSlots + kTrFfnEnd] = 0;
+  }
+#endif
+  // this CTA's share of K: an even number of blocks (H is a multiple of 128)
+  const int H = d.H, m = d.m_ret, nk = H / kBoundK / gridDim.z, k0 = blockIdx.z * nk * kBoundK;
+  z += (size_t)blockIdx.z * d.B * m;
+  norm2 += (size_t)blockIdx.z * m;
+  const int t0 = blockIdx.x * kBoundTile, r0 = blockIdx.y * kBoundTile;
+
+  if (warp < 8) {
+    // Each thread carries column block tid % 8 (8 elements) of rows tid / 8 +
+    // 32 u of both operands, from global memory through registers (one K block
+    // ahead) into the 128-byte swizzled tiles.  Rows past the batch or the
+    // pool are zero.
+    const int col = tid & 7, row = tid >> 3;
+    const __nv_bfloat16 *xsrc[4];
+    const float *wsrc[4];
+    bool xok[4], wok[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + row + 32 * u, r = r0 + row + 32 * u;
+      xok[u] = t < d.B;
+      wok[u] = r < m;
+      const int rr = wok[u] ? r : 0;
+      const int e = min(max(retained ? __ldg(retained + rr) : rr, 0), d.E - 1);
+      xsrc[u] = hidden + (size_t)(xok[u] ? t : 0) * H + k0 + col * 8;
+      wsrc[u] = router_w + (size_t)e * H + k0 + col * 8;
+    }
+    struct Block {
+      uint4 x[4];
+      float4 wa[4], wb[4];
+    };
+    auto fetch = [&](Block &b, int kc) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        b.x[u] = xok[u] ? __ldg(reinterpret_cast<const uint4 *>(xsrc[u] + kc * kBoundK))
+                        : make_uint4(0u, 0u, 0u, 0u);
+        const float4 *w = reinterpret_cast<const float4 *>(wsrc[u] + kc * kBoundK);
+        b.wa[u] = wok[u] ? __ldg(w) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        b.wb[u] = wok[u] ? __ldg(w + 1) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      }
+    };
+    float n2[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    auto put = [&](const Block &b, int kc) {
+      const int s = kc % kBoundStages;
+      const bool got = mbar_wait_bounded(
+          empty_bar(s), ((uint32_t)(kc / kBoundStages) & 1u) ^ 1u, abort, kDefaultWaitLimitNs);
+      if (!__all_sync(0xFFFFFFFFu, got)) {
+        *abort = 1;
+        return false;
+      }
+      const uint32_t base = smem + (uint32_t)(s * 3 * kBoundOperand);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int rw = row + 32 * u;
+        const uint32_t dst = base + (uint32_t)(rw * 128 + ((col ^ (rw & 7)) * 16));
+        const float w[8] = {b.wa[u].x, b.wa[u].y, b.wa[u].z, b.wa[u].w,
+                            b.wb[u].x, b.wb[u].y, b.wb[u].z, b.wb[u].w};
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          hi[q] = bf16_pair(w[2 * q], w[2 * q + 1]);
+          lo[q] = bf16_pair(w[2 * q] - __uint_as_float(hi[q] << 16),
+                            w[2 * q + 1] - __uint_as_float(hi[q] & 0xFFFF0000u));
+          n2[u] = fmaf(w[2 * q], w[2 * q], fmaf(w[2 * q + 1], w[2 * q + 1], n2[u]));
+        }
+        st_shared_v4(dst, b.x[u].x, b.x[u].y, b.x[u].z, b.x[u].w);
+        st_shared_v4(dst + kBoundOperand, hi[0], hi[1], hi[2], hi[3]);
+        st_shared_v4(dst + 2 * kBoundOperand, lo[0], lo[1], lo[2], lo[3]);
+      }
+      fence_proxy_async_shared();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full_bar(s));
+      return true;
+    };
+    // two K blocks in flight
+    Block even, odd;
+    fetch(even, 0);
+    fetch(odd, 1);
+    bool ok = true;
+    for (int kc = 0; kc < nk; kc += 2) {
+      ok = put(even, kc);
+      if (!ok) break;
+      if (kc + 2 < nk) fetch(even, kc + 2);
+      ok = put(odd, kc + 1);
+      if (!ok) break;
+      if (kc + 3 < nk) fetch(odd, kc + 3);
+    }
+    // squared norms of the router rows, once per row
+    if (blockIdx.x == 0) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float v = n2[u];
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        if (col == 0 && wok[u]) norm2[r0 + row + 32 * u] = v;
+      }
+    }
+    // accumulator rows 32 q .. (tokens), columns 64 h .. (experts)
+    if (ok) ok = mbar_wait_bounded(done_bar, 0u, abort, kDefaultWaitLimitNs);
+    ok = __all_sync(0xFFFFFFFFu, ok && !*abort) != 0;
+    tc_fence_after();
+    const int q = warp & 3, c_first = (warp >> 2) * 64;
+#pragma unroll
+    for (int c = 0; c < 64; c += 32) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t v[16];
+        tmem_ld_frag(tmem + ((uint32_t)(32 * q + 16 * h) << 16) + (uint32_t)(c_first + c), v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          // values 2i, 2i + 1: column block i / 2, row half i % 2
+          const int t = t0 + 32 * q + 16 * h + 8 * (i & 1) + (lane >> 2);
+          const int r = r0 + c_first + c + 8 * (i >> 1) + 2 * (lane & 3);
+          // a wait that gave up: no value, so every logit is evaluated
+          const float a = ok ? __uint_as_float(v[2 * i]) : __uint_as_float(0x7FC00000u);
+          const float b = ok ? __uint_as_float(v[2 * i + 1]) : __uint_as_float(0x7FC00000u);
+          if (t < d.B) {
+            float *dst = z + (size_t)t * m + r;
+            if ((m & 1) == 0 && r + 1 < m) {
+              *reinterpret_cast<float2 *>(dst) = make_float2(a, b);
+            } else {
+              if (r < m) dst[0] = a;
+              if (r + 1 < m) dst[1] = b;
+            }
+          }
+        }
+      }
+    }
+    tc_fence_before();
+  } else {
+    const uint32_t idesc = idesc_bf16_f32(kBoundTile, kBoundTile);
+    int issued = 0;
+    for (int kc = 0; kc < nk; ++kc) {
+      const int s = kc % kBoundStages;
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(full_bar(s), (uint32_t)(kc / kBoundStages) & 1u,
+                                                     abort, kDefaultWaitLimitNs))) {
+        *abort = 1;
+        __threadfence_block();
+        break;
+      }
+      tc_fence_after();
+      const uint32_t a = smem + (uint32_t)(s * 3 * kBoundOperand);
+      if (elect_one()) {
+#pragma unroll
+        for (int term = 1; term <= 2; ++term)
+#pragma unroll
+          for (int kk = 0; kk < kBoundK / 16; ++kk)
+            tc_mma_bf16(tmem, smem_desc_sw128(a + kk * 32),
+                        smem_desc_sw128(a + term * kBoundOperand + kk * 32), idesc,
+                        (kc > 0 || term > 1 || kk > 0) ? 1u : 0u);
+        tc_commit(empty_bar(s));
+      }
+      __syncwarp();
+      ++issued;
+    }
+    // the accumulator is complete (after a wait that gave up: nothing of this
+    // CTA's is in flight any more)
+    if (issued > 0) {
+      if (elect_one()) tc_commit(done_bar);
+      __syncwarp();
+      mbar_wait_timeout(done_bar, 0u, 10000000ull);
+    }
+  }
+  __syncthreads();
+  if (warp == 8) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kBoundTile);
+  }
+}
+
+// Canonical logits (see the head of this file) of N experts for one token, by
+// one warp; every lane gets them.
+template <int N>
+__device__ __forceinline__ void canonical_logits(const __nv_bfloat16 *__restrict__ x,
+                                                 const float *const (&w)[N], int H, int lane,
+                                                 float (&p)[N]) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) p[j] = 0.0f;
+#pragma unroll 2
+  for (int c = 0; c < H / 128; ++c) {
+    const int h = 128 * c + 4 * lane;
+    const uint2 xv = __ldg(reinterpret_cast<const uint2 *>(x + h));
+    const float xf[4] = {__uint_as_float(xv.x << 16), __uint_as_float(xv.x & 0xFFFF0000u),
+                         __uint_as_float(xv.y << 16), __uint_as_float(xv.y & 0xFFFF0000u)};
+    float4 wv[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) wv[j] = __ldg(reinterpret_cast<const float4 *>(w[j] + h));
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      p[j] = fmaf(xf[0], wv[j].x, p[j]);
+      p[j] = fmaf(xf[1], wv[j].y, p[j]);
+      p[j] = fmaf(xf[2], wv[j].z, p[j]);
+      p[j] = fmaf(xf[3], wv[j].w, p[j]);
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int j = 0; j < N; ++j) p[j] += __shfl_xor_sync(0xFFFFFFFFu, p[j], off);
+}
+// ... of experts r of list[0, N), into exact[r].
+template <int N>
+__device__ __forceinline__ void refine(const unsigned short *list, const int32_t *ids,
+                                       const __nv_bfloat16 *__restrict__ x,
+                                       const float *__restrict__ router_w, int H, int lane,
+                                       float *exact) {
+  const float *w[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) w[j] = router_w + (size_t)ids[list[j]] * H;
+  float p[N];
+  canonical_logits<N>(x, w, H, lane, p);
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (lane == j) exact[list[j]] = p[j];
+}
+
+// NC: 32 NC >= m'.
+template <int NC>
+__global__ void __launch_bounds__(kRouteThreads)
+    route_refine_kernel(const __nv_bfloat16 *__restrict__ hidden,
+                        const float *__restrict__ router_w,
+                        const int32_t *__restrict__ retained, Dims d, Ws ws,
+                        const float *__restrict__ z, const float *__restrict__ norm2, int parts) {
+  __shared__ int32_t ids[32 * NC];
+  __shared__ float exact[kRouteWarps][32 * NC];
+  __shared__ unsigned short list[kRouteWarps][32 * NC];
+  __shared__ uint32_t wmax;
+  if (threadIdx.x == 0) wmax = 0u;
+  pdl_wait_primary();
+  pdl_launch_dependents();
+  const int m = d.m_ret, H = d.H, k = d.k;
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = blockIdx.x * kRouteWarps + wi;
+  const __nv_bfloat16 *x = hidden + (size_t)min(t, d.B - 1) * H;
+  // this lane's approximate logits (the sum of their parts) and the token's
+  // squared norm: every load of the parts is issued before any is used
+  float part[kBoundParts][NC], zc[NC];
+#pragma unroll
+  for (int p = 0; p < kBoundParts; ++p)
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int r = lane + 32 * i;
+      part[p][i] = p < parts && r < m ? z[((size_t)p * d.B + min(t, d.B - 1)) * m + r] : 0.0f;
+    }
+  float x2 = 0.0f;
+#pragma unroll 8
+  for (int c = 0; c < H / 128; ++c) {
+    const uint2 xv = __ldg(reinterpret_cast<const uint2 *>(x + 128 * c + 4 * lane));
+    const float a = __uint_as_float(xv.x << 16), b = __uint_as_float(xv.x & 0xFFFF0000u);
+    const float e = __uint_as_float(xv.y << 16), f = __uint_as_float(xv.y & 0xFFFF0000u);
+    x2 = fmaf(a, a, fmaf(b, b, fmaf(e, e, fmaf(f, f, x2))));
+  }
+  for (int r = threadIdx.x; r < m; r += blockDim.x)
+    ids[r] = min(max(retained ? retained[r] : r, 0), d.E - 1);
+  if (blockIdx.x == gridDim.x - 1) report_retained(retained, d, ws);
+  __syncthreads();
+  // largest squared norm of the router rows, as bits: above every finite value
+  // where one is infinite or NaN
+  {
+    uint32_t v = 0u;
+    for (int r = threadIdx.x; r < m; r += blockDim.x) {
+      float s = 0.0f;
+#pragma unroll
+      for (int p = 0; p < kBoundParts; ++p) s += p < parts ? norm2[(size_t)p * m + r] : 0.0f;
+      v = max(v, __float_as_uint(s));
+    }
+    v = __reduce_max_sync(0xFFFFFFFFu, v);
+    if (lane == 0) atomicMax(&wmax, v);
+  }
+  __syncthreads();
+  if (t < d.B) {
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      zc[i] = part[0][i];
+#pragma unroll
+      for (int p = 1; p < kBoundParts; ++p) zc[i] += part[p][i];
+      bad |= !(fabsf(zc[i]) < __uint_as_float(0x7F800000u));
+      exact[wi][lane + 32 * i] = -__uint_as_float(0x7F800000u);  // below every candidate
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x2 += __shfl_xor_sync(0xFFFFFFFFu, x2, off);
+    // product of the norms (0.2 % up for the sums' rounding and underflow)
+    const float w2 = __uint_as_float(wmax);
+    const float prod = sqrtf(x2) * sqrtf(w2) * 1.002f;
+    bad |= !(x2 > 1e-24f && x2 < 1e36f && w2 > 1e-24f && w2 < 1e36f && prod < 1e36f);
+    // T: the k-th largest approximate logit, one per distinct expert
+    uint32_t left[NC];  // order bits of the logits not taken yet, 0 = none
+#pragma unroll
+    for (int i = 0; i < NC; ++i) left[i] = lane + 32 * i < m ? logit_order_bits(zc[i]) : 0u;
+    float T = 0.0f;
+    for (int j = 0; j < k; ++j) {
+      uint32_t best = 0u;
+      int bid = 0;
+      float bz = 0.0f;
+#pragma unroll
+      for (int i = 0; i < NC; ++i)
+        if (left[i] > best) {
+          best = left[i];
+          bid = ids[lane + 32 * i];
+          bz = zc[i];
+        }
+      const uint32_t win = __reduce_max_sync(0xFFFFFFFFu, best);
+      bad |= win == 0u;
+      const int src = __ffs(__ballot_sync(0xFFFFFFFFu, best == win)) - 1;
+      const int id = __shfl_sync(0xFFFFFFFFu, bid, src);
+      T = __shfl_sync(0xFFFFFFFFu, bz, src);
+#pragma unroll
+      for (int i = 0; i < NC; ++i)
+        if (lane + 32 * i < m && ids[lane + 32 * i] == id) left[i] = 0u;
+    }
+    const bool all = __any_sync(0xFFFFFFFFu, bad) != 0;
+    const float least = T - 2.02f * filter_bound(H) * prod;
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int r = lane + 32 * i;
+      const bool c = r < m && (all || zc[i] >= least);
+      const uint32_t mask = __ballot_sync(0xFFFFFFFFu, c);
+      if (c) list[wi][n + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)r;
+      n += __popc(mask);
+    }
+    __syncwarp();
+    int j = 0;
+    for (; j + 8 <= n; j += 8) refine<8>(list[wi] + j, ids, x, router_w, H, lane, exact[wi]);
+    for (; j + 2 <= n; j += 2) refine<2>(list[wi] + j, ids, x, router_w, H, lane, exact[wi]);
+    if (j < n) refine<1>(list[wi] + j, ids, x, router_w, H, lane, exact[wi]);
+    __syncwarp();
+    topk_token<NC>(exact[wi], ids, d, ws, t, lane);
+  }
+#ifdef SLIMWISE_TRACE
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const int tr_step = ws.ctrl[kCtrlTraceStep];
+    trace_stamp(ws, tr_step, kTrRouteEnd);
+    ws.ctrl[kCtrlTraceStep] = tr_step + 1;
+  }
+#endif
+}
+
+// Which calls take the filtered kernels (where the scratch rows hold `parts`
+// approximate logits).  The refining work grows with k, the full product with
+// m', and the two kernels' latency (about 20 us) has to be earned.  Whole
+// layers at H = 2048, k = 8, full product / filtered, us:
+//   m' = 32    B = 8192 594.6 / 610.9     m' = 64   B = 8192 630.9 / 636.5
+//   m' = 96    B = 5000 451.4 / 452.5
+//   m' = 128   B = 1536 247.4 / 250.0    2048 275.5 / 273.4   2560 304.1 / 297.9
+//              3000 328.8 / 320.0   4001 411.6 / 390.6   8192 718.1 / 681.5
+//   m' = 192   B = 4096 436.4 / 410.9
+//   m' = 256   B =  768 303.3 / 306.2    1024 317.7 / 315.0   1536 358.1 / 347.7
+//              2048 389.7 / 366.5   4096 517.5 / 464.6   8192 825.2 / 725.7
+inline bool filtered_fits(const Dims &d, int parts) {
+  return (size_t)parts * (d.B + 1) * d.m_ret * 4 <= (size_t)d.B * d.k * d.H * 2;
+}
+inline bool route_filtered(const Dims &d) {
+  const long long bm = (long long)d.B * d.m_ret;
+  return d.m_ret >= 128 && d.m_ret >= 16 * d.k && d.m_ret <= 256 && bm >= (1ll << 18) &&
+         bm * d.H >= (1ll << 29) && filtered_fits(d, 1);
+}
+
+cudaError_t launch_route_filtered(const __nv_bfloat16 *hidden, const float *router_w,
+                                  const int32_t *retained, Dims d, Ws ws, bool pdl, int sms,
+                                  cudaStream_t stream) {
+  // approximate logits, then the router rows' norms, where the call's expert
+  // outputs will be
+  float *z = reinterpret_cast<float *>(ws.y);
+  // K in 2 or 4 parts while they leave at most one CTA per SM (each writes its
+  // own approximate logits): 4001 tokens x 128 experts 410.9 us a layer with
+  // one part, 398.6 with two, 392.9 with four, 392.8 with eight
+  const int tiles = ((d.B + kBoundTile - 1) / kBoundTile) * ((d.m_ret + kBoundTile - 1) / kBoundTile);
+  int parts = 1;
+  while (parts < kBoundParts && 2 * parts * tiles <= sms && d.H / 128 % (2 * parts) == 0 &&
+         filtered_fits(d, 2 * parts))
+    parts *= 2;
+  float *norm2 = z + (size_t)parts * d.B * d.m_ret;
+  cudaError_t err = cudaFuncSetAttribute(
+      route_bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBoundSmem);
+  if (err != cudaSuccess) return err;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.gridDim = dim3((d.B + kBoundTile - 1) / kBoundTile, (d.m_ret + kBoundTile - 1) / kBoundTile, parts);
+  cfg.blockDim = dim3(kBoundThreads);
+  cfg.dynamicSmemBytes = kBoundSmem;
+  err = cudaLaunchKernelEx(&cfg, route_bound_kernel, hidden, router_w, retained, d, ws, z, norm2);
+  if (err != cudaSuccess) return err;
+  cfg.gridDim = dim3((d.B + kRouteWarps - 1) / kRouteWarps);
+  cfg.blockDim = dim3(kRouteThreads);
+  cfg.dynamicSmemBytes = 0;
+  auto refine = d.m_ret <= 128 ? route_refine_kernel<4> : route_refine_kernel<8>;
+  return cudaLaunchKernelEx(&cfg, refine, hidden, router_w, retained, d, ws, (const float *)z,
+                            (const float *)norm2, parts);
+}
+
 cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w,
                               const int32_t *retained, Dims d, Ws ws, bool pdl,
                               cudaStream_t stream) {
   int dev = 0, optin = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  if (route_tiled(d)) {
+  const bool filtered = route_filtered(d);
+  if (filtered || route_tiled(d)) {
     int sms = 0;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    return launch_route_tiled(hidden, router_w, retained, d, ws, pdl, sms, stream);
+    auto launch = filtered ? launch_route_filtered : launch_route_tiled;
+    return launch(hidden, router_w, retained, d, ws, pdl, sms, stream);
   }
   err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (err != cudaSuccess) return err;

@@ -101,6 +101,43 @@ def test_tiled_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
                            r["topk_gate"][t0:t0 + step].view(torch.int32))
 
 
+# Routing that bounds the logits on the tensor cores and evaluates those that
+# can be selected: at the smallest sizes of its range, with ragged tiles of
+# tokens and experts, an odd pool (unpaired stores), K in 4 parts and in one,
+# ids in any order, and where no bound holds (values that are not finite, norms
+# that leave the range, tied and repeated experts)
+@pytest.mark.parametrize("H,E,k,B,m_prime", [(2048, 128, 8, 2048, 128), (2048, 256, 8, 1025, 256),
+                                             (640, 200, 8, 5001, 177), (256, 256, 16, 8193, 256),
+                                             (2048, 160, 1, 2050, 129)])
+def test_filtered_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
+    shape = synth.LayerShape(hidden=H, num_experts=E, inter=64, top_k=k)
+    x, wr = synth.hidden_states(B, shape, 3), synth.router_weight(shape, 4)
+    wr[E // 2] = wr[E // 3]  # equal logits: ties to the lowest id
+    wr[E // 4] = wr[E // 5] * (1 + 1e-6)  # closer than any bound of the filter
+    ret = synth.retained_set(E, m_prime, 5, shuffle=True)
+    xd, wd, rd = x.to(DEV), wr.to(DEV), ret.to(DEV)
+    r = sw.slimwise_moe_route(xd, wd, rd, k, E)
+    idx, gates = oracle.route(oracle.router_logits(synth.bf16_bits(x), wr.numpy()), ret.numpy(), k)
+    assert np.array_equal(r["topk_idx"].cpu().numpy(), idx)
+    np.testing.assert_allclose(r["topk_gate"].cpu().numpy(), gates, rtol=4e-6, atol=1e-7)
+    # bit for bit what the cluster kernel gives (small batches)
+    xd[5], xd[B - 1, 7], xd[30, 9] = 0.0, float("inf"), float("nan")
+    xd[31], xd[32] = xd[31] * 1e36, xd[32] * 1e-30
+    rep = rd.clone()
+    rep[1::2] = rep[0::2][:len(rep[1::2])]  # every id twice
+    big = wd.clone()
+    big[E // 6, 3] = float("inf")
+    rows = np.r_[0:64, B // 2:B // 2 + 64, B - 65:B]
+    for w, ids in [(wd, rd), (wd, rep), (big, rd), (torch.zeros_like(wd), rd), (wd * 1e-30, rd),
+                   (wd[:1] + 1e-5 * wd, rd)]:
+        r = sw.slimwise_moe_route(xd, w, ids, k, E)
+        s = [sw.slimwise_moe_route(xd[rows[i:i + 28]].contiguous(), w, ids, k, E)
+             for i in range(0, len(rows), 28)]
+        assert torch.equal(torch.cat([v["topk_idx"] for v in s]), r["topk_idx"][rows])
+        assert torch.equal(torch.cat([v["topk_gate"] for v in s]).view(torch.int32),
+                           r["topk_gate"][rows].view(torch.int32))
+
+
 @pytest.mark.parametrize("B,E,k", [(1, 16, 1), (5, 1024, 32), (300, 96, 8)])
 def test_routing_outputs_may_be_left_out(B, E, k):
     # any output may be NULL; one written alone equals the same one among all
