@@ -810,14 +810,14 @@ cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_
 //                        loaded), fp32 accumulation.  Writes the approximate
 //                        logits and the router rows' squared norms to scratch.
 //   route_refine_kernel  one warp per token: the k-th largest approximate
-//                        logit T of distinct experts, the canonical logit of
-//                        every expert whose approximate one reaches T - 2 b,
+//                        logit T (equal ones counted once, which can only lower
+//                        it), the canonical logit of every expert whose approximate one reaches T - 2 b,
 //                        and the top-k of those.
 // b bounds |approximate - canonical| (filter_bound): k experts have canonical
 // logits of at least T - b, an expert left out has less, so the selections,
 // the gates and the order are the canonical ones bit for bit.  Where no bound
 // holds (a value that is not finite, norms that over- or underflow, fewer than
-// k distinct experts) every logit of the token is evaluated.
+// k different logits, a repeated id) every logit of the token is evaluated.
 // The bounding kernel (12 us at 4001 tokens x 128 experts) waits for its loads;
 // the refining one reads k router rows per token from L2, which bounds it at
 // large batches (8192 tokens x 256 experts: 0.55 GB), and is a chain of a few
@@ -1096,34 +1096,39 @@ __device__ __forceinline__ void canonical_logits(const __nv_bfloat16 *__restrict
 #pragma unroll
     for (int j = 0; j < N; ++j) p[j] += __shfl_xor_sync(0xFFFFFFFFu, p[j], off);
 }
-// ... of experts r of list[0, N), into exact[r].
+// ... of the experts cand[0, N), into exact[0, N).
 template <int N>
-__device__ __forceinline__ void refine(const unsigned short *list, const int32_t *ids,
-                                       const __nv_bfloat16 *__restrict__ x,
+__device__ __forceinline__ void refine(const int32_t *cand, const __nv_bfloat16 *__restrict__ x,
                                        const float *__restrict__ router_w, int H, int lane,
                                        float *exact) {
   const float *w[N];
 #pragma unroll
-  for (int j = 0; j < N; ++j) w[j] = router_w + (size_t)ids[list[j]] * H;
+  for (int j = 0; j < N; ++j) w[j] = router_w + (size_t)cand[j] * H;
   float p[N];
   canonical_logits<N>(x, w, H, lane, p);
 #pragma unroll
   for (int j = 0; j < N; ++j)
-    if (lane == j) exact[list[j]] = p[j];
+    if (lane == j) exact[j] = p[j];
 }
 
-// NC: 32 NC >= m'.
+// NC: 32 NC >= m'.  Registers for 4 CTAs on an SM, so that 4001 tokens x 128
+// experts are one wave (78 of them: 390.5 -> 395.0 us a layer), or for 3 with the
+// larger pool (2048 tokens: 363.2 us, 372.2 with 4).  The top-k runs over the
+// candidates alone, one per lane where they are at most 32, and T comes from
+// values, not from (value, id) pairs: 8192 tokens x 256 experts 725 -> 715 us.
 template <int NC>
-__global__ void __launch_bounds__(kRouteThreads)
+__global__ void __launch_bounds__(kRouteThreads, NC == 4 ? 4 : 3)
     route_refine_kernel(const __nv_bfloat16 *__restrict__ hidden,
                         const float *__restrict__ router_w,
                         const int32_t *__restrict__ retained, Dims d, Ws ws,
                         const float *__restrict__ z, const float *__restrict__ norm2, int parts) {
   __shared__ int32_t ids[32 * NC];
   __shared__ float exact[kRouteWarps][32 * NC];
-  __shared__ unsigned short list[kRouteWarps][32 * NC];
-  __shared__ uint32_t wmax;
-  if (threadIdx.x == 0) wmax = 0u;
+  __shared__ int32_t cand[kRouteWarps][32 * NC];
+  __shared__ uint32_t wmax, seen[kMaxExperts / 32];
+  __shared__ int repeated;  // an id is listed twice
+  if (threadIdx.x == 0) wmax = 0u, repeated = 0;
+  if (threadIdx.x < kMaxExperts / 32) seen[threadIdx.x] = 0u;
   pdl_wait_primary();
   pdl_launch_dependents();
   const int m = d.m_ret, H = d.H, k = d.k;
@@ -1161,20 +1166,21 @@ __global__ void __launch_bounds__(kRouteThreads)
 #pragma unroll
       for (int p = 0; p < kBoundParts; ++p) s += p < parts ? norm2[(size_t)p * m + r] : 0.0f;
       v = max(v, __float_as_uint(s));
+      const uint32_t bit = 1u << (ids[r] & 31);
+      if (atomicOr(&seen[ids[r] >> 5], bit) & bit) repeated = 1;
     }
     v = __reduce_max_sync(0xFFFFFFFFu, v);
     if (lane == 0) atomicMax(&wmax, v);
   }
   __syncthreads();
   if (t < d.B) {
-    bool bad = false;
+    bool bad = repeated != 0;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
       zc[i] = part[0][i];
 #pragma unroll
       for (int p = 1; p < kBoundParts; ++p) zc[i] += part[p][i];
       bad |= !(fabsf(zc[i]) < __uint_as_float(0x7F800000u));
-      exact[wi][lane + 32 * i] = -__uint_as_float(0x7F800000u);  // below every candidate
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) x2 += __shfl_xor_sync(0xFFFFFFFFu, x2, off);
@@ -1182,49 +1188,40 @@ __global__ void __launch_bounds__(kRouteThreads)
     const float w2 = __uint_as_float(wmax);
     const float prod = sqrtf(x2) * sqrtf(w2) * 1.002f;
     bad |= !(x2 > 1e-24f && x2 < 1e36f && w2 > 1e-24f && w2 < 1e36f && prod < 1e36f);
-    // T: the k-th largest approximate logit, one per distinct expert
-    uint32_t left[NC];  // order bits of the logits not taken yet, 0 = none
+    // T: the k-th largest distinct value, so at most the k-th largest logit
+    uint32_t left[NC], win = 0u;  // order bits of the values not taken yet, 0 = none
 #pragma unroll
     for (int i = 0; i < NC; ++i) left[i] = lane + 32 * i < m ? logit_order_bits(zc[i]) : 0u;
-    float T = 0.0f;
     for (int j = 0; j < k; ++j) {
-      uint32_t best = 0u;
-      int bid = 0;
-      float bz = 0.0f;
+      uint32_t best = left[0];
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        if (left[i] > best) {
-          best = left[i];
-          bid = ids[lane + 32 * i];
-          bz = zc[i];
-        }
-      const uint32_t win = __reduce_max_sync(0xFFFFFFFFu, best);
-      bad |= win == 0u;
-      const int src = __ffs(__ballot_sync(0xFFFFFFFFu, best == win)) - 1;
-      const int id = __shfl_sync(0xFFFFFFFFu, bid, src);
-      T = __shfl_sync(0xFFFFFFFFu, bz, src);
+      for (int i = 1; i < NC; ++i) best = max(best, left[i]);
+      win = __reduce_max_sync(0xFFFFFFFFu, best);
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        if (lane + 32 * i < m && ids[lane + 32 * i] == id) left[i] = 0u;
+      for (int i = 0; i < NC; ++i) left[i] = left[i] == win ? 0u : left[i];
     }
+    bad |= win == 0u;
     const bool all = __any_sync(0xFFFFFFFFu, bad) != 0;
-    const float least = T - 2.02f * filter_bound(H) * prod;
+    const float least = logit_from_order_bits(win) - 2.02f * filter_bound(H) * prod;
     int n = 0;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
       const int r = lane + 32 * i;
       const bool c = r < m && (all || zc[i] >= least);
       const uint32_t mask = __ballot_sync(0xFFFFFFFFu, c);
-      if (c) list[wi][n + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)r;
+      if (c) cand[wi][n + __popc(mask & ((1u << lane) - 1u))] = ids[r];
       n += __popc(mask);
     }
     __syncwarp();
     int j = 0;
-    for (; j + 8 <= n; j += 8) refine<8>(list[wi] + j, ids, x, router_w, H, lane, exact[wi]);
-    for (; j + 2 <= n; j += 2) refine<2>(list[wi] + j, ids, x, router_w, H, lane, exact[wi]);
-    if (j < n) refine<1>(list[wi] + j, ids, x, router_w, H, lane, exact[wi]);
+    for (; j + 8 <= n; j += 8) refine<8>(cand[wi] + j, x, router_w, H, lane, exact[wi] + j);
+    for (; j + 2 <= n; j += 2) refine<2>(cand[wi] + j, x, router_w, H, lane, exact[wi] + j);
+    if (j < n) refine<1>(cand[wi] + j, x, router_w, H, lane, exact[wi] + j);
     __syncwarp();
-    topk_token<NC>(exact[wi], ids, d, ws, t, lane);
+    Dims dn = d;
+    dn.m_ret = n;
+    if (n <= 32) topk_token<1>(exact[wi], cand[wi], dn, ws, t, lane);
+    else topk_token<NC>(exact[wi], cand[wi], dn, ws, t, lane);
   }
 #ifdef SLIMWISE_TRACE
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1244,8 +1241,8 @@ __global__ void __launch_bounds__(kRouteThreads)
 //   m' = 128   B = 1536 247.4 / 250.0    2048 275.5 / 273.4   2560 304.1 / 297.9
 //              3000 328.8 / 320.0   4001 411.6 / 390.6   8192 718.1 / 681.5
 //   m' = 192   B = 4096 436.4 / 410.9
-//   m' = 256   B =  768 303.3 / 306.2    1024 317.7 / 315.0   1536 358.1 / 347.7
-//              2048 389.7 / 366.5   4096 517.5 / 464.6   8192 825.2 / 725.7
+//   m' = 256   B =  768 303.3 / 306.2    1024 317.7 / 312.6   1536 358.1 / 347.7
+//              2048 389.7 / 363.2   4096 517.5 / 464.6   8192 825.2 / 715.2
 inline bool filtered_fits(const Dims &d, int parts) {
   return (size_t)parts * (d.B + 1) * d.m_ret * 4 <= (size_t)d.B * d.k * d.H * 2;
 }
