@@ -578,8 +578,9 @@ def main_gpu(args, ws, rank, local):
         "step_ms_p10_p50_p90": [pt["step_ms_p10"], pt["step_ms_p50"], pt["step_ms_p90"]],
         "step_spread": "percentiles of the mean step over blocks of 10 consecutive layer calls",
         "graph": graph,
-        # route, expert FFN and combine per step, and above 96 tokens group
-        "gpu_launches": (3 if B <= 96 and FFN_ITEMS <= 0 else 4) * args.steps,
+        # route, expert FFN and combine per step; above 96 tokens group; above
+        # 256 tokens the selecting kernel of routing
+        "gpu_launches": ((3 if B <= 96 and FFN_ITEMS <= 0 else 4) + (B > 256)) * args.steps,
         "clocks": dict(clk.summary(), soak_s=CLOCK_SOAK_S),
     }
     if FFN_ITEMS:

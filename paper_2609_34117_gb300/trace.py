@@ -6,7 +6,9 @@ words at the head of the workspace, one step per layer call:
 
     route_start, route_end    routing grid, first CTA: after its dependency
                               wait, and when it finishes
-    group_start, group_end    grouping grid, first CTA, likewise
+    group_start, group_end    grouping grid, first CTA, likewise (in a batch
+                              grouped inside the FFN, up to 96 tokens: the FFN
+                              grid's first CTA around its own grouping)
     ffn_start                 expert-FFN grid, first CTA after its wait
     ffn_first_data            first stage of weights and tokens in that CTA
     ffn_end                   the FFN grid's last CTA to finish
