@@ -126,14 +126,19 @@ int slimwise_moe_decode_full(const void *hidden, const float *router_w,
  *   grid_ctas            >0: persistent expert-FFN grid size (default: the
  *                        device's SM count).
  *   wait_limit_ns        >0: limit, in ns, of every bounded wait of the
- *                        expert-FFN kernel (default 1 s).  A wait that runs
- *                        out sets SLIMWISE_DEVERR_PIPELINE_TIMEOUT or
+ *                        expert-FFN kernel and of the kernel that bounds a
+ *                        prompt chunk's router logits (default 1 s).  A wait
+ *                        that runs out sets SLIMWISE_DEVERR_PIPELINE_TIMEOUT or
  *                        SLIMWISE_DEVERR_DEPENDENCY_TIMEOUT; its CTA then
  *                        drains its copies and MMAs, frees its tensor memory
- *                        and exits, and the output is incomplete.
+ *                        and exits, and the output is incomplete (after a
+ *                        bounding kernel's wait it is complete: every logit
+ *                        is then evaluated).
  *   test_starve_first_down  tests only: 1 makes the first routed down item
  *                        wait for one more gate/up tile than exists, so that
- *                        wait runs out after wait_limit_ns (the timeout path).
+ *                        wait runs out after wait_limit_ns (the timeout path);
+ *                        2 does the same to the waits of the bounding kernel's
+ *                        first CTA (nothing where the call does not run it).
  *   ffn_items            form of the expert-FFN work items: 0 or -1 the
  *                        default, 128-row items (256-row ones at token chunks
  *                        of 64-80 rows); 1 CTA-pair items (two 128-row weight

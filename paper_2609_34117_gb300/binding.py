@@ -295,7 +295,7 @@ def slimwise_moe_compact_layer(w_gate_up, w_down, router_w, retained_idx, stream
 def _opts(ffn_events, disable_pdl, grid_ctas, wait_limit_ns=0, test_starve_first_down=False,
           ffn_items=0):
     opts = DecodeOpts(None, None, int(bool(disable_pdl)), int(grid_ctas), int(wait_limit_ns),
-                      int(bool(test_starve_first_down)), int(ffn_items))
+                      int(test_starve_first_down), int(ffn_items))
     if ffn_events is not None:
         opts.ffn_begin = ctypes.c_void_p(ffn_events[0].cuda_event)
         opts.ffn_end = ctypes.c_void_p(ffn_events[1].cuda_event)
@@ -309,10 +309,11 @@ def slimwise_moe_decode_ex(hidden, router_w, retained_idx, w_gate_up, w_down, to
     """slimwise_moe_decode with launch options; retained_idx None = full pool.
 
     ffn_events: optional (begin, end) torch.cuda.Event pair recorded around the
-    expert-FFN kernel on the launch stream.  wait_limit_ns: limit of the FFN
-    kernel's bounded waits (0: 1 s).  test_starve_first_down: tests only, makes
-    the first down item's dependency wait run out.  ffn_items: form of the FFN
-    work items (0 or -1 the default, 1 CTA-pair items where the layer allows).
+    expert-FFN kernel on the launch stream.  wait_limit_ns: limit of the
+    kernels' bounded waits (0: 1 s).  test_starve_first_down: tests only, makes
+    the first down item's dependency wait run out (2: the waits of the first
+    CTA that bounds router logits).  ffn_items: form of the FFN work items (0
+    or -1 the default, 1 CTA-pair items where the layer allows).
     """
     s, out, workspace = _prep(hidden, router_w, w_gate_up, w_down, top_k, out, workspace)
     if retained_idx is not None:

@@ -250,10 +250,16 @@ constexpr int kWideMinPool = 64;
 // tried (B = 64-512, m' = 32-128: 15-40 %), so a layer uses them only when
 // the caller asks (slimwise_decode_opts.ffn_items = 1).
 
+// Default limit of every bounded wait.
+constexpr uint64_t kDefaultWaitLimitNs = 1000000000ull;
+
 // Kernel launch declarations (defined in their own translation units).
+// timeout_ns: limit of the bounding kernel's waits; starve_bound (tests only):
+// its first CTA's waits run out.
 cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w,
                               const int32_t *retained, Dims d, Ws ws, bool pdl,
-                              cudaStream_t stream);
+                              cudaStream_t stream, uint64_t timeout_ns = kDefaultWaitLimitNs,
+                              int starve_bound = 0);
 // w_shared_gate: fp32 [H] gate row of the shared expert, or NULL (d.Is == 0).
 cudaError_t launch_group_gather(const __nv_bfloat16 *hidden, const float *w_shared_gate,
                                 Dims d, Ws ws, bool pdl, bool gather, cudaStream_t stream);
@@ -287,15 +293,14 @@ struct FfnMaps {
   CUtensorMap act_s[kTokBoxSizes];  // [B rows, Is cols] bf16, token order
 };
 
-// timeout_ns: limit of every bounded wait; starve_first_down (tests only):
-// the first routed down item waits for a gate/up tile that never exists.
-constexpr uint64_t kDefaultWaitLimitNs = 1000000000ull;
 // The gate-weighted combine of every (token, 128-column tile), after the
 // expert FFN.
 cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStream_t stream);
 // retained: the call's retained ids (NULL: the full pool or a compacted one),
 // read only to guess which weight tiles to warm in L2.
 // hidden, w_shared_gate: read only when the call groups locally (d.local).
+// timeout_ns: limit of every bounded wait; starve_first_down (tests only):
+// the first routed down item waits for a gate/up tile that never exists.
 cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
                               const float *w_shared_gate, Dims d, Ws ws,
                               const int32_t *retained, int grid, bool pdl,

@@ -182,14 +182,16 @@ __device__ __forceinline__ void take_winner(uint32_t whi, uint32_t wlo, int j, i
 }
 
 // The grid's last CTA reports bad and repeated retained ids and resets the
-// error word (and, for a call that groups locally, the counters).
+// error word (and, for a call that groups locally, the counters).  `earlier`:
+// this thread's error bits of the kernels before this one.
 __device__ __forceinline__ void report_retained(const int32_t *__restrict__ retained, const Dims &d,
-                                                const Ws &ws) {
+                                                const Ws &ws, int earlier = 0) {
   __shared__ uint32_t seen[kMaxExperts / 32];
   __shared__ int bad;
   for (int i = threadIdx.x; i < kMaxExperts / 32; i += blockDim.x) seen[i] = 0;
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
+  if (earlier) atomicOr(&bad, earlier);
   for (int r = threadIdx.x; r < d.m_ret; r += blockDim.x) {
     int e = retained ? retained[r] : r;
     if (e < 0 || e >= d.E) {
@@ -818,6 +820,9 @@ cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_
 // the gates and the order are the canonical ones bit for bit.  Where no bound
 // holds (a value that is not finite, norms that over- or underflow, fewer than
 // k different logits, a repeated id) every logit of the token is evaluated.
+// A wait of the bounding kernel that gives up leaves no value (NaN) of its
+// tokens' logits and, where it sums them, of its experts' norms, so that no
+// token takes a bound from half a norm; the refining kernel reports it.
 // The bounding kernel (20 us at 8192 tokens x 128 experts, 33 at 256) waits for
 // its loads, the tensor pipe 17-22 % busy; the refining one (43 and 51 us) reads
 // k router rows per token from L2 (0.41 and 0.56 GB into the SMs), a few round
@@ -860,7 +865,8 @@ __global__ void __launch_bounds__(kBoundThreads, 1)
     route_bound_kernel(const __nv_bfloat16 *__restrict__ hidden,
                        const float *__restrict__ router_w,
                        const int32_t *__restrict__ retained, Dims d, Ws ws,
-                       float *__restrict__ z, float *__restrict__ norm2) {
+                       float *__restrict__ z, float *__restrict__ norm2,
+                       int32_t *__restrict__ gave_up, uint64_t timeout_ns, int starve) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[2 * kBoundStages + 1];
   __shared__ uint32_t tmem_slot;
@@ -941,7 +947,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1)
     auto put = [&](const Block &b, int kc) {
       const int s = kc % kBoundStages;
       const bool got = mbar_wait_bounded(
-          empty_bar(s), ((uint32_t)(kc / kBoundStages) & 1u) ^ 1u, abort, kDefaultWaitLimitNs);
+          empty_bar(s), ((uint32_t)(kc / kBoundStages) & 1u) ^ 1u, abort, timeout_ns);
       if (!__all_sync(0xFFFFFFFFu, got)) {
         *abort = 1;
         return false;
@@ -983,19 +989,21 @@ __global__ void __launch_bounds__(kBoundThreads, 1)
       if (!ok) break;
       if (kc + 3 < nk) fetch(odd, kc + 3);
     }
-    // squared norms of the router rows, once per row
+    // squared norms of the router rows, once per row (none of rows that this
+    // warp has not seen to the end)
     if (blockIdx.x == 0) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         float v = n2[u];
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-        if (col == 0 && wok[u]) norm2[r0 + row + 32 * u] = v;
+        if (col == 0 && wok[u]) norm2[r0 + row + 32 * u] = ok ? v : __uint_as_float(0x7FC00000u);
       }
     }
     // accumulator rows 32 q .. (tokens), columns 64 h .. (experts)
-    if (ok) ok = mbar_wait_bounded(done_bar, 0u, abort, kDefaultWaitLimitNs);
+    if (ok) ok = mbar_wait_bounded(done_bar, 0u, abort, timeout_ns);
     ok = __all_sync(0xFFFFFFFFu, ok && !*abort) != 0;
+    if (!ok) *abort = 1;
     tc_fence_after();
     const int q = warp & 3, c_first = (warp >> 2) * 64;
 #pragma unroll
@@ -1029,10 +1037,13 @@ __global__ void __launch_bounds__(kBoundThreads, 1)
   } else {
     const uint32_t idesc = idesc_bf16_f32(kBoundTile, kBoundTile);
     int issued = 0;
-    for (int kc = 0; kc < nk; ++kc) {
+    // tests only: the first CTA multiplies nothing, so the waits of its loading
+    // warps run out
+    const bool starved = starve && (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
+    for (int kc = 0; kc < nk && !starved; ++kc) {
       const int s = kc % kBoundStages;
       if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(full_bar(s), (uint32_t)(kc / kBoundStages) & 1u,
-                                                     abort, kDefaultWaitLimitNs))) {
+                                                     abort, timeout_ns))) {
         *abort = 1;
         __threadfence_block();
         break;
@@ -1061,6 +1072,8 @@ __global__ void __launch_bounds__(kBoundThreads, 1)
     }
   }
   __syncthreads();
+  if (tid == 0)
+    gave_up[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = *abort ? 1 : 0;
   if (warp == 8) {
     tc_fence_after();
     tmem_dealloc(tmem, kBoundTile);
@@ -1122,7 +1135,8 @@ __global__ void __launch_bounds__(kRouteThreads, NC == 4 ? 4 : 3)
     route_refine_kernel(const __nv_bfloat16 *__restrict__ hidden,
                         const float *__restrict__ router_w,
                         const int32_t *__restrict__ retained, Dims d, Ws ws,
-                        const float *__restrict__ z, const float *__restrict__ norm2, int parts) {
+                        const float *__restrict__ z, const float *__restrict__ norm2, int parts,
+                        const int32_t *__restrict__ gave_up, int bound_ctas) {
   __shared__ int32_t ids[32 * NC];
   __shared__ float exact[kRouteWarps][32 * NC];
   __shared__ int32_t cand[kRouteWarps][32 * NC];
@@ -1156,7 +1170,12 @@ __global__ void __launch_bounds__(kRouteThreads, NC == 4 ? 4 : 3)
   }
   for (int r = threadIdx.x; r < m; r += blockDim.x)
     ids[r] = min(max(retained ? retained[r] : r, 0), d.E - 1);
-  if (blockIdx.x == gridDim.x - 1) report_retained(retained, d, ws);
+  if (blockIdx.x == gridDim.x - 1) {
+    int timeout = 0;  // any bounding CTA's wait
+    for (int i = threadIdx.x; i < bound_ctas; i += blockDim.x)
+      if (gave_up[i]) timeout = SLIMWISE_DEVERR_PIPELINE_TIMEOUT;
+    report_retained(retained, d, ws, timeout);
+  }
   __syncthreads();
   // largest squared norm of the router rows, as bits: above every finite value
   // where one is infinite or NaN
@@ -1255,7 +1274,7 @@ inline bool route_filtered(const Dims &d) {
 
 cudaError_t launch_route_filtered(const __nv_bfloat16 *hidden, const float *router_w,
                                   const int32_t *retained, Dims d, Ws ws, bool pdl, int sms,
-                                  cudaStream_t stream) {
+                                  cudaStream_t stream, uint64_t timeout_ns, int starve) {
   // approximate logits, then the router rows' norms, where the call's expert
   // outputs will be
   float *z = reinterpret_cast<float *>(ws.y);
@@ -1268,6 +1287,9 @@ cudaError_t launch_route_filtered(const __nv_bfloat16 *hidden, const float *rout
          filtered_fits(d, 2 * parts))
     parts *= 2;
   float *norm2 = z + (size_t)parts * d.B * d.m_ret;
+  // one word per bounding CTA (at most B / 16 + 8) where the call's activations
+  // will be (at least 32 words a token)
+  int32_t *gave_up = reinterpret_cast<int32_t *>(ws.act);
   cudaError_t err = cudaFuncSetAttribute(
       route_bound_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBoundSmem);
   if (err != cudaSuccess) return err;
@@ -1281,19 +1303,20 @@ cudaError_t launch_route_filtered(const __nv_bfloat16 *hidden, const float *rout
   cfg.gridDim = dim3((d.B + kBoundTile - 1) / kBoundTile, (d.m_ret + kBoundTile - 1) / kBoundTile, parts);
   cfg.blockDim = dim3(kBoundThreads);
   cfg.dynamicSmemBytes = kBoundSmem;
-  err = cudaLaunchKernelEx(&cfg, route_bound_kernel, hidden, router_w, retained, d, ws, z, norm2);
+  err = cudaLaunchKernelEx(&cfg, route_bound_kernel, hidden, router_w, retained, d, ws, z, norm2,
+                           gave_up, timeout_ns, starve);
   if (err != cudaSuccess) return err;
   cfg.gridDim = dim3((d.B + kRouteWarps - 1) / kRouteWarps);
   cfg.blockDim = dim3(kRouteThreads);
   cfg.dynamicSmemBytes = 0;
   auto refine = d.m_ret <= 128 ? route_refine_kernel<4> : route_refine_kernel<8>;
   return cudaLaunchKernelEx(&cfg, refine, hidden, router_w, retained, d, ws, (const float *)z,
-                            (const float *)norm2, parts);
+                            (const float *)norm2, parts, (const int32_t *)gave_up, tiles * parts);
 }
 
 cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w,
                               const int32_t *retained, Dims d, Ws ws, bool pdl,
-                              cudaStream_t stream) {
+                              cudaStream_t stream, uint64_t timeout_ns, int starve_bound) {
   int dev = 0, optin = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
@@ -1302,8 +1325,9 @@ cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w
     int sms = 0;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    auto launch = filtered ? launch_route_filtered : launch_route_tiled;
-    return launch(hidden, router_w, retained, d, ws, pdl, sms, stream);
+    return filtered ? launch_route_filtered(hidden, router_w, retained, d, ws, pdl, sms, stream,
+                                            timeout_ns, starve_bound)
+                    : launch_route_tiled(hidden, router_w, retained, d, ws, pdl, sms, stream);
   }
   err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (err != cudaSuccess) return err;

@@ -298,8 +298,12 @@ int decode_impl(const void *hidden, const float *router_w, const int32_t *retain
   const uint64_t slots = (uint64_t)d.B * d.k;
   if (!ffn_maps_for(&maps, hidden, w_gate_up, w_down, w, d, slots, se)) return SLIMWISE_ERR_CUDA;
 
+  const uint64_t wait_limit = (opts && opts->wait_limit_ns > 0)
+                                  ? (uint64_t)opts->wait_limit_ns
+                                  : kDefaultWaitLimitNs;
+  const int test_starve = opts ? opts->test_starve_first_down : 0;
   if (launch_route_topk(static_cast<const __nv_bfloat16 *>(hidden), router_w, retained,
-                        d, w, pdl, st) != cudaSuccess)
+                        d, w, pdl, st, wait_limit, test_starve == 2) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
   if (!d.local && launch_group_gather(static_cast<const __nv_bfloat16 *>(hidden), se.gate, d, w,
                                       pdl, true, st) != cudaSuccess)
@@ -307,10 +311,7 @@ int decode_impl(const void *hidden, const float *router_w, const int32_t *retain
   const bool timed = opts && opts->ffn_begin && opts->ffn_end;
   if (timed && cudaEventRecord(static_cast<cudaEvent_t>(opts->ffn_begin), st) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;
-  const uint64_t wait_limit = (opts && opts->wait_limit_ns > 0)
-                                  ? (uint64_t)opts->wait_limit_ns
-                                  : kDefaultWaitLimitNs;
-  const int starve = (opts && opts->test_starve_first_down) ? 1 : 0;
+  const int starve = test_starve != 0 && test_starve != 2;
   if (launch_expert_ffn(maps, static_cast<const __nv_bfloat16 *>(hidden), se.gate, d, w, retained,
                         grid, pdl && !timed, st, wait_limit, starve) != cudaSuccess)
     return SLIMWISE_ERR_CUDA;

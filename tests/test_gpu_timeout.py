@@ -8,6 +8,11 @@ that gave up drains its copies and MMAs, frees its tensor memory and exits,
 and the kernel completes well before the default 1 s limit.  The next normal
 call on the same workspace must read a clear error word and match the oracle
 (the GPU stays usable).
+
+The kernel that bounds the router logits of large batches waits too; there the
+option's value 2 makes the waits of one CTA run out.  The selections must not
+change (every logit is evaluated then) and the call must record
+SLIMWISE_DEVERR_PIPELINE_TIMEOUT.
 """
 import time
 
@@ -72,3 +77,37 @@ def test_dependency_wait_runs_out_and_next_call_is_clean(tiny, B, k):
                                      wait_limit_ns=WAIT_LIMIT_NS)
     assert sw.slimwise_moe_device_status(ws) == 0
     assert torch.equal(out2, out)
+
+
+# (2048, ...): the starved CTA's loading warps give up in the middle of their
+# share of K, so its experts' squared norms would cover half of it; (256, ...):
+# the whole of K fits its ring, and the wait for the accumulator gives up
+@pytest.mark.parametrize("H,E,k,B", [(2048, 128, 8, 2048), (256, 256, 16, 8193)])
+def test_bounding_wait_runs_out_without_changing_the_selections(H, E, k, B):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    shape = synth.LayerShape(hidden=H, num_experts=E, inter=64, top_k=k)
+    w_gu, w_d = synth.expert_weights(shape, 1, device=DEV)
+    g = torch.Generator().manual_seed(7)
+    # groups of 16 experts closer than the approximate logits resolve, with
+    # nearly all of their norm in the elements that the starved CTA never sees
+    wr = (0.02 * torch.randn((E // 16, H), generator=g)).repeat_interleave(16, dim=0)
+    wr *= 1 + 1e-6 * torch.randn((E, H), generator=g)
+    if H > 512:
+        wr[:, :256] *= 1e-6
+        wr[:, 512:] *= 1e-6
+    x = synth.hidden_states(B, shape, 3)
+    xd, wrd = x.to(DEV), wr.to(DEV)
+    ws = sw.alloc_workspace(B, H, E, 64, k, DEV)
+    want = sw.slimwise_moe_decode_ex(xd, wrd, None, w_gu, w_d, k, workspace=ws)
+    assert sw.slimwise_moe_device_status(ws) == 0
+    t0 = time.perf_counter()
+    got = sw.slimwise_moe_decode_ex(xd, wrd, None, w_gu, w_d, k, workspace=ws,
+                                    wait_limit_ns=WAIT_LIMIT_NS, test_starve_first_down=2)
+    flags = sw.slimwise_moe_device_status(ws)
+    assert time.perf_counter() - t0 < 0.5
+    assert flags == sw.binding.DEVERR_PIPELINE_TIMEOUT, flags
+    assert torch.equal(got, want)
+    # the next call on the workspace reads a clear error word
+    got = sw.slimwise_moe_decode_ex(xd, wrd, None, w_gu, w_d, k, workspace=ws)
+    assert sw.slimwise_moe_device_status(ws) == 0 and torch.equal(got, want)
