@@ -63,6 +63,16 @@ __host__ __device__ inline int entry_tokens(int n, int chunk) {
   const int parts = (n + chunk - 1) / chunk;
   return parts > 1 ? round16((n + parts - 1) / parts) : chunk;
 }
+// Entries of an expert with n selections, ceil(n / chunk): the rounded product
+// with inv = 1 / chunk is at most one off (2^25 selections are the most a call
+// can have, all of one expert where a token lists it twice), and then corrected.
+__host__ __device__ inline int entry_count(int n, int chunk, float inv) {
+  const int x = n + chunk - 1;
+  int q = (int)(((float)x + 0.5f) * inv);
+  q -= q * chunk > x ? 1 : 0;
+  q += (q + 1) * chunk <= x ? 1 : 0;
+  return q;
+}
 // Index m of the token box (kTokBox * (m + 1) rows) that covers n16 16-row groups.
 __host__ __device__ inline int token_box_for(int n16) { return n16 - 1; }
 constexpr int kMinTokChunk = 16;     // smallest token_chunk_for(): bounds the entry count

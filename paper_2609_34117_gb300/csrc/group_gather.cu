@@ -49,9 +49,8 @@ constexpr int kGroupTiledMin = 768;
 __device__ __forceinline__ void scan_pool(const int *cnt, int E, int tok_chunk, int *offs,
                                           int *flags, int *entries) {
   const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  // exact for up to 2^20 tokens: the quotient's fraction is at least 1 / 256
   const float inv = 1.0f / (float)tok_chunk;
-  auto entries_of = [&](int n) { return (int)(((float)(n + tok_chunk - 1) + 0.5f) * inv); };
+  auto entries_of = [&](int n) { return entry_count(n, tok_chunk, inv); };
   for (int c = threadIdx.x >> 5; 32 * c < E; c += nwarps) {
     int n0 = 0, f0 = 0, e0 = 0;
     for (int e = lane; e < 32 * c; e += 32) {
