@@ -526,6 +526,10 @@ size_t route_smem_bytes(const Dims &d) {
          (size_t)((TB + kClusterCtas - 1) / kClusterCtas) * d.m_ret * 4 + (size_t)d.m_ret * 4;
 }
 
+// What a routing CTA leaves of the opt-in limit for its static shared memory
+// (report_retained's, 132 bytes).
+constexpr size_t kRouteStaticSmem = 1024;
+
 template <int TB, int NC>
 cudaError_t launch_route_tb(const __nv_bfloat16 *hidden, const float *router_w,
                             const int32_t *retained, Dims d, Ws ws, bool pdl,
@@ -1337,7 +1341,7 @@ cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w
     const size_t need = t == 16 ? route_smem_bytes<16>(d) : t == 8 ? route_smem_bytes<8>(d)
                       : t == 4 ? route_smem_bytes<4>(d) : t == 2 ? route_smem_bytes<2>(d)
                       : route_smem_bytes<1>(d);
-    return need <= (size_t)optin;
+    return need + kRouteStaticSmem <= (size_t)optin;
   };
   while (tb > 1 && !fits(tb)) tb >>= 1;
   switch (tb) {

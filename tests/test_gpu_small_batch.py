@@ -47,3 +47,17 @@ def test_layer_small_batches(B, E, k, shared):
     if not shared:
         y = sw.slimwise_moe_decode_full(args[0], args[1], *args[3:], out=args[0])
         assert torch.equal(y, out)
+
+
+# hidden rows that leave a routing CTA no room for its static shared memory at
+# the usual tokens per cluster: fewer tokens, not a refused launch
+@pytest.mark.parametrize("B", [40, 70])
+def test_routing_of_rows_that_fill_shared_memory(B):
+    H, E, k = 28928, 128, 2
+    shape = synth.LayerShape(hidden=H, num_experts=E, inter=64, top_k=k)
+    x, wr = synth.hidden_states(B, shape, 1), synth.router_weight(shape, 2)
+    r = sw.slimwise_moe_route(x.to(DEV), wr.to(DEV), None, k, E)
+    idx, gates = oracle.route(oracle.router_logits(synth.bf16_bits(x), wr.numpy()),
+                              np.arange(E, dtype=np.int32), k)
+    assert np.array_equal(r["topk_idx"].cpu().numpy(), idx)
+    np.testing.assert_allclose(r["topk_gate"].cpu().numpy(), gates, rtol=4e-6, atol=1e-7)
