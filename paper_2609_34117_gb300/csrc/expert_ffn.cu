@@ -1283,7 +1283,9 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
                 : d.wide     ? expert_ffn_kernel<false, true, false, false, 0>
                 : ahead      ? expert_ffn_kernel<false, false, false, true, 0>
                              : expert_ffn_kernel<false, false, false, false, 0>;
-  err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // one value for every call: the attribute is the kernel's, not the launch's,
+  // and another thread may be launching it with another size
+  err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   if (err != cudaSuccess) return err;
   int tmem_cols = 32;
   while (tmem_cols < 2 * ffn_acc_cols(d)) tmem_cols <<= 1;

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kGroupThreads)
 }
 
 // blockIdx.x = tile, blockIdx.y = part: tokens [y part, (y + 1) part) of every
-// 128-token block of the tile.  Dynamic shared memory: see place_smem_bytes.
+// 128-token block of the tile.  Dynamic shared memory: see place_smem.
 __global__ void __launch_bounds__(kGroupThreads)
     group_place_kernel(const __nv_bfloat16 *__restrict__ hidden, const float *__restrict__ w_sg,
                        Dims d, Ws ws, const int32_t *__restrict__ tile_cnt, int part,
@@ -450,13 +450,17 @@ __global__ void __launch_bounds__(kGroupThreads)
 #endif
 }
 
+constexpr int kMaxGroupPart = 16;
 // Tokens of a block per CTA of group_place_kernel: enough CTAs for the GPU at
 // the smallest batches, fewer recounts of the tile at the largest.
-inline int group_part_tokens(int B) { return B <= 1024 ? 4 : B <= 4096 ? 8 : 16; }
+inline int group_part_tokens(int B) { return B <= 1024 ? 4 : B <= 4096 ? 8 : kMaxGroupPart; }
 
-size_t place_smem_bytes(const Dims &d, int part) {
-  return (size_t)(5 * d.E + 3 + d.E * kTileWords + part * d.k) * 4;
+constexpr size_t place_smem(int E, int k, int part) {
+  return (size_t)(5 * E + 3 + E * kTileWords + part * k) * 4;
 }
+// never more than a kernel gets without asking (an attribute of the kernel,
+// which calls of other threads would set to other sizes)
+static_assert(place_smem(kMaxExperts, kMaxTopK, kMaxGroupPart) <= 48 * 1024, "shared memory");
 
 cudaError_t launch_group_tiled(const __nv_bfloat16 *hidden, const float *w_shared_gate, Dims d,
                                Ws ws, bool pdl, bool gather, cudaStream_t stream) {
@@ -464,10 +468,6 @@ cudaError_t launch_group_tiled(const __nv_bfloat16 *hidden, const float *w_share
   // E / 32 bytes a token at most against k H bf16
   int32_t *tile_cnt = reinterpret_cast<int32_t *>(ws.y);
   const int tiles = group_tile_count(d.B), part = group_part_tokens(d.B);
-  const size_t smem = place_smem_bytes(d, part);
-  cudaError_t err = cudaFuncSetAttribute(group_place_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -477,10 +477,10 @@ cudaError_t launch_group_tiled(const __nv_bfloat16 *hidden, const float *w_share
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   cfg.gridDim = dim3(tiles);
-  err = cudaLaunchKernelEx(&cfg, group_count_kernel, d, ws, tile_cnt);
+  cudaError_t err = cudaLaunchKernelEx(&cfg, group_count_kernel, d, ws, tile_cnt);
   if (err != cudaSuccess) return err;
   cfg.gridDim = dim3(tiles, kGroupTile / part);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = place_smem(d.E, d.k, part);
   return cudaLaunchKernelEx(&cfg, group_place_kernel, hidden, w_shared_gate, d, ws,
                             (const int32_t *)tile_cnt, part, gather ? 1 : 0);
 }

@@ -526,17 +526,19 @@ size_t route_smem_bytes(const Dims &d) {
          (size_t)((TB + kClusterCtas - 1) / kClusterCtas) * d.m_ret * 4 + (size_t)d.m_ret * 4;
 }
 
-// What a routing CTA leaves of the opt-in limit for its static shared memory
-// (report_retained's, 132 bytes).
+// What a routing CTA may take, of the opt-in limit: the rest is for its static
+// shared memory (report_retained's, 132 bytes).
 constexpr size_t kRouteStaticSmem = 1024;
 
 template <int TB, int NC>
 cudaError_t launch_route_tb(const __nv_bfloat16 *hidden, const float *router_w,
-                            const int32_t *retained, Dims d, Ws ws, bool pdl,
+                            const int32_t *retained, Dims d, Ws ws, bool pdl, size_t max_smem,
                             cudaStream_t stream) {
   const size_t smem = route_smem_bytes<TB>(d);
+  // one value for every call: the attribute is the kernel's, not the launch's,
+  // and another thread may be launching it with another size
   cudaError_t err = cudaFuncSetAttribute(
-      route_topk_kernel<TB, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      route_topk_kernel<TB, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
   if (err != cudaSuccess) return err;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(((d.B + TB - 1) / TB) * kClusterCtas);
@@ -557,11 +559,12 @@ cudaError_t launch_route_tb(const __nv_bfloat16 *hidden, const float *router_w,
 
 template <int TB>
 cudaError_t launch_route_nc(const __nv_bfloat16 *hidden, const float *router_w,
-                            const int32_t *retained, Dims d, Ws ws, bool pdl,
+                            const int32_t *retained, Dims d, Ws ws, bool pdl, size_t max_smem,
                             cudaStream_t stream) {
-  if (d.m_ret <= 128) return launch_route_tb<TB, 4>(hidden, router_w, retained, d, ws, pdl, stream);
-  if (d.m_ret <= 256) return launch_route_tb<TB, 8>(hidden, router_w, retained, d, ws, pdl, stream);
-  return launch_route_tb<TB, 0>(hidden, router_w, retained, d, ws, pdl, stream);
+  auto launch = d.m_ret <= 128   ? launch_route_tb<TB, 4>
+                : d.m_ret <= 256 ? launch_route_tb<TB, 8>
+                                 : launch_route_tb<TB, 0>;
+  return launch(hidden, router_w, retained, d, ws, pdl, max_smem, stream);
 }
 
 // --------------------------------------------------------------------------
@@ -1335,22 +1338,22 @@ cudaError_t launch_route_topk(const __nv_bfloat16 *hidden, const float *router_w
   }
   err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (err != cudaSuccess) return err;
+  const size_t max_smem = (size_t)optin - kRouteStaticSmem;
   // wide hidden rows: fewer tokens per cluster until they fit in shared memory
   int tb = route_tokens_per_cluster(d.B, d.m_ret);
   auto fits = [&](int t) {
     const size_t need = t == 16 ? route_smem_bytes<16>(d) : t == 8 ? route_smem_bytes<8>(d)
                       : t == 4 ? route_smem_bytes<4>(d) : t == 2 ? route_smem_bytes<2>(d)
                       : route_smem_bytes<1>(d);
-    return need + kRouteStaticSmem <= (size_t)optin;
+    return need <= max_smem;
   };
   while (tb > 1 && !fits(tb)) tb >>= 1;
-  switch (tb) {
-    case 1: return launch_route_nc<1>(hidden, router_w, retained, d, ws, pdl, stream);
-    case 2: return launch_route_nc<2>(hidden, router_w, retained, d, ws, pdl, stream);
-    case 4: return launch_route_nc<4>(hidden, router_w, retained, d, ws, pdl, stream);
-    case 8: return launch_route_nc<8>(hidden, router_w, retained, d, ws, pdl, stream);
-    default: return launch_route_nc<16>(hidden, router_w, retained, d, ws, pdl, stream);
-  }
+  auto launch = tb == 1   ? launch_route_nc<1>
+                : tb == 2 ? launch_route_nc<2>
+                : tb == 4 ? launch_route_nc<4>
+                : tb == 8 ? launch_route_nc<8>
+                          : launch_route_nc<16>;
+  return launch(hidden, router_w, retained, d, ws, pdl, max_smem, stream);
 }
 
 }  // namespace slimwise
