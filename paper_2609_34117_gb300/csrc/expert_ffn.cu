@@ -620,7 +620,8 @@ __global__ void __maxnreg__(128)
   // Above 64 tokens the combine kernel that follows may become resident now
   // (it waits for this grid to finish): measured 2-4 us faster per step at
   // B = 128-512, 0.5 us slower at B = 64, where the trigger stays at the end
-  // of the work.
+  // of the work (launch_expert_ffn: and where a combine that groups locally
+  // finds no room yet).
   if (early_dependents) pdl_launch_dependents();
 #ifdef SLIMWISE_TRACE
   const int tr_step = ws.ctrl[kCtrlTraceStep] - 1;
@@ -1175,6 +1176,11 @@ __global__ void __launch_bounds__(kCombineThreads)
   }
 }
 
+// Dynamic shared memory of a combine CTA: the local grouping's masks and bases.
+size_t combine_smem_bytes(const Dims &d) {
+  return d.local ? (size_t)d.E * (local_words(d) * 4 + 2) : 0;
+}
+
 cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStream_t stream) {
   const int pairs = d.B * (d.H / kCombineTile);
   const int wpc = kCombineThreads / 32;
@@ -1182,7 +1188,7 @@ cudaError_t launch_combine(Dims d, Ws ws, __nv_bfloat16 *out, bool pdl, cudaStre
   cfg.gridDim = dim3((pairs + wpc - 1) / wpc);
   cfg.blockDim = dim3(kCombineThreads);
   const int words = local_words(d);
-  cfg.dynamicSmemBytes = d.local ? (size_t)d.E * (words * 4 + 2) : 0;
+  cfg.dynamicSmemBytes = combine_smem_bytes(d);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1324,7 +1330,23 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
   cfg.attrs = attr;
   cfg.numAttrs = na;
   const int static_first = grid <= resident ? 1 : 0;
-  const int early_dependents = d.B > 64 ? 1 : 0;
+  // The combine is signalled early above 64 tokens, but a locally grouping one
+  // only where its CTAs find room beside these: signalled without room (65-80
+  // tokens) it was later than after the last item.  Early / after, us: H = 512,
+  // 1024 experts 45.1 / 35.1 (m' = 256), H = 2048, 1024 experts 100.1 / 91.8,
+  // Qwen-class m' = 128 172.9 / 171.7, m' = 32 54.8 / 54.2.  Where there is
+  // room (81-96 tokens) early is the better for short rows (H = 512, 1024
+  // experts 32.6 / 35.8), within 0.4 us with up to 256 experts, and the worse
+  // with 1024 experts at H = 2048 (101.7 / 95.6).
+  int early_dependents = d.B > 64 ? 1 : 0;
+  if (early_dependents && d.local) {
+    int sm_smem = 0, reserved = 0;  // an SM's, and what each CTA takes besides its own
+    err = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (err != cudaSuccess) return err;
+    err = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (err != cudaSuccess) return err;
+    if (smem + combine_smem_bytes(d) + 2 * (size_t)reserved > (size_t)sm_smem) early_dependents = 0;
+  }
   return cudaLaunchKernelEx(&cfg, kernel, maps, hidden, w_shared_gate, d, ws, retained, stages,
                             tmem_cols, static_first, early_dependents, timeout_ns, starve_first_down);
 }
