@@ -524,6 +524,23 @@ def workload_config(name, wl, shape, ws):
             "parallelism": f"replicas{ws}", "l2": l2}
 
 
+def layer_launches(shape, B, m_prime, shared=0, ffn_items=0):
+    """Kernels that the library launches for one layer call: routing (one, or
+    two where it is tiled or filtered), grouping (none up to 96 tokens, two from
+    768 on), the expert FFN and the combine.  The rules are route_filtered and
+    route_tiled (route_topk.cu), make_dims (slimwise_api.cu) and kGroupTiledMin
+    (group_gather.cu)."""
+    H, k, m = shape.hidden, shape.top_k, m_prime
+    scratch = B * k * H * 2
+    filtered = (128 <= m <= 256 and m >= 16 * k and B * m >= 1 << 18 and B * m * H >= 1 << 29 and
+                (B + 1) * m * 4 <= scratch)
+    tiled = (B * m * 4 <= scratch and
+             (B > 256 or m > 256 or B * m >= (16384 if m > 128 else 24576)))
+    pair = ffn_items > 0 and not shared and shape.inter % 128 == 0 and H % 256 == 0
+    group = 0 if B <= 96 and not pair else 1 if B < 768 else 2
+    return (2 if filtered or tiled else 1) + group + 2
+
+
 def main_gpu(args, ws, rank, local):
     import paper_2609_34117_gb300 as sw
     from paper_2609_34117_gb300 import build as swbuild
@@ -578,9 +595,8 @@ def main_gpu(args, ws, rank, local):
         "step_ms_p10_p50_p90": [pt["step_ms_p10"], pt["step_ms_p50"], pt["step_ms_p90"]],
         "step_spread": "percentiles of the mean step over blocks of 10 consecutive layer calls",
         "graph": graph,
-        # route, expert FFN and combine per step; above 96 tokens group; above
-        # 256 tokens the selecting kernel of routing
-        "gpu_launches": ((3 if B <= 96 and FFN_ITEMS <= 0 else 4) + (B > 256)) * args.steps,
+        "gpu_launches": args.steps * layer_launches(shape, B, min(m_prime, shape.num_experts),
+                                                    wl.get("shared", 0), FFN_ITEMS),
         "clocks": dict(clk.summary(), soak_s=CLOCK_SOAK_S),
     }
     if FFN_ITEMS:
