@@ -822,11 +822,12 @@ cudaError_t launch_route_tiled(const __nv_bfloat16 *hidden, const float *router_
 //                        logit T (equal ones counted once, which can only lower
 //                        it), the canonical logit of every expert whose
 //                        approximate one reaches T - 2 b, and the top-k of those.
-// b bounds |approximate - canonical| (filter_bound): k experts have canonical
-// logits of at least T - b, an expert left out has less, so the selections,
-// the gates and the order are the canonical ones bit for bit.  Where no bound
-// holds (a value that is not finite, norms that over- or underflow, fewer than
-// k different logits, a repeated id) every logit of the token is evaluated.
+// b bounds |approximate - canonical| (filter_bound, which says what it assumes
+// of the tensor core): k experts have canonical logits of at least T - b, an
+// expert left out has less, so the selections, the gates and the order are the
+// canonical ones bit for bit.  Where no bound holds (a value that is not finite,
+// norms that over- or underflow, fewer than k different logits, a repeated id)
+// every logit of the token is evaluated.
 // A wait of the bounding kernel that gives up leaves no value (NaN) of its
 // tokens' logits and, where it sums them, of its experts' norms, so that no
 // token takes a bound from half a norm; the refining kernel reports it.
@@ -850,10 +851,13 @@ constexpr int kBoundSmem = kBoundStages * 3 * kBoundOperand + 1024;
 //                 2^-18 of it);
 //   (H/8) 2^-21   the tensor core's sum: one step per 16 elements of each term,
 //                 allowed 2^-21 of the sum of magnitudes (four units of fp32
-//                 truncation) each;
+//                 truncation) each -- an assumption, since how the unit
+//                 rounds its sums is not documented; everything that the
+//                 filter claims rests on it;
 //   (H/32+6) 2^-23  the canonical sum's own rounding, at least twice over.
-// Largest |approximate - exact| seen, of this bound: 0.4 % with normal rows, 3 %
-// with elements over e^+-6, 6 % with rows of one sign (H = 8192).
+// Largest |approximate - exact| seen, of this bound: 0.5 % with normal rows and
+// with elements over e^+-6, 4.5 to 6.7 % with rows of one sign (H = 2048 to
+// 32768; the tests hold it to 25 %).
 __device__ __forceinline__ float filter_bound(int H) {
   return 0x1p-17f + (float)(H / 8) * 0x1p-21f + (float)(H / 32 + 6) * 0x1p-23f;
 }

@@ -138,6 +138,65 @@ def test_filtered_routing_equals_oracle_and_small_batches(H, E, k, B, m_prime):
                            r["topk_gate"][rows].view(torch.int32))
 
 
+def _rows(kind, shape, g):
+    """normal, of one sign (sums without cancellation), elements over e^+-6"""
+    r = torch.randn(shape, generator=g, device=DEV)
+    if kind == "sign":
+        r = r.abs()
+    elif kind == "wide":
+        r = r.sign() * torch.exp(12 * torch.rand(shape, generator=g, device=DEV) - 6)
+    return r
+
+
+def _filter_bound(H):
+    return 2.0**-17 + H / 8 * 2.0**-21 + (H / 32 + 6) * 2.0**-23
+
+
+# The filter's bound allows the tensor core's sum a rounding that its
+# documentation does not give; what it really has is seen here: the approximate
+# logits (left in the workspace's last region by a routing-only call) against
+# 64 bits, K in one part.  At most a quarter of the bound.
+@pytest.mark.parametrize("kind", ["normal", "sign", "wide"])
+@pytest.mark.parametrize("H,k", [(2048, 8), (8192, 8), (32768, 2)])
+def test_tensor_core_logits_stay_well_inside_their_bound(H, k, kind):
+    B, E = 5120, 256
+    assert torch.cuda.get_device_properties(0).multi_processor_count < 2 * 2 * B // 128
+    g = torch.Generator(device=DEV).manual_seed(H)
+    x = _rows(kind, (B, H), g).to(torch.bfloat16)
+    wr = 0.02 * _rows(kind, (E, H), g)
+    ws = sw.alloc_workspace(B, H, E, 64, k, DEV)
+    sw.slimwise_moe_route(x, wr, None, k, E, 64, workspace=ws)
+    y0 = ws.numel() - (B * k * H * 2 + 1023) // 1024 * 1024
+    z = ws[y0:y0 + B * E * 4].view(torch.float32).view(B, E)[64:].double()  # grouping wrote the first
+    x, wr = x[64:].double(), wr.double()
+    norms = x.norm(dim=1)[:, None] * wr.norm(dim=1)[None, :]
+    ratio = ((z - x @ wr.T).abs() / (norms * _filter_bound(H))).max().item()
+    assert 0 < ratio <= 0.25, ratio
+
+
+# every token's selections are those of small batches bit for bit, for rows of
+# each kind and long sums: the bound is then up to several gaps between the
+# logits wide.  Half of the experts are one row spread over three bounds.
+@pytest.mark.parametrize("copies", [False, True])
+@pytest.mark.parametrize("kind", ["normal", "sign", "wide"])
+@pytest.mark.parametrize("H,B,E", [(4096, 1030, 256), (8192, 2050, 128), (8192, 5120, 256)])
+def test_filtered_routing_of_long_rows(H, B, E, kind, copies):
+    k = 8
+    g = torch.Generator(device=DEV).manual_seed(B)
+    x = _rows(kind, (B, H), g).to(torch.bfloat16)
+    wr = 0.02 * _rows(kind, (E, H), g)
+    if copies:
+        spread = 3 * _filter_bound(H) * torch.rand((E // 2, 1), generator=g, device=DEV)
+        noise = 1e-5 * torch.randn((E // 2, H), generator=g, device=DEV)
+        wr[::2] = wr[:1] * (1 + spread) * (1 + noise)
+    r = sw.slimwise_moe_route(x, wr, None, k, E)
+    for t0 in range(0, B, 28):
+        s = sw.slimwise_moe_route(x[t0:t0 + 28].contiguous(), wr, None, k, E)
+        assert torch.equal(s["topk_idx"], r["topk_idx"][t0:t0 + 28])
+        assert torch.equal(s["topk_gate"].view(torch.int32),
+                           r["topk_gate"][t0:t0 + 28].view(torch.int32))
+
+
 @pytest.mark.parametrize("B,E,k", [(1, 16, 1), (5, 1024, 32), (300, 96, 8)])
 def test_routing_outputs_may_be_left_out(B, E, k):
     # any output may be NULL; one written alone equals the same one among all
