@@ -280,7 +280,9 @@ enum {
  * highest score, ties to the lowest id, written ascending to retained_idx
  * (device int32 [n_retained]) -- ready for slimwise_moe_decode or for building
  * the compact checkpoint.  stats: device fp64 [num_experts, 4].  One kernel
- * launch on `stream`; num_experts <= 1024.
+ * launch on `stream`; num_experts <= 1024.  A NaN score ranks neither above nor
+ * below any other: its expert is kept, and of more than n_retained kept experts
+ * the lowest ids are written.
  */
 int slimwise_moe_select_retained(const double *stats, int32_t num_experts,
                                  int32_t n_retained, int32_t criterion,

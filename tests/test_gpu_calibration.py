@@ -53,3 +53,17 @@ def test_selection_of_special_scores(m):
     st[4, 1], st[9, 1] = np.inf, -np.inf
     ids = sw.slimwise_moe_select_retained(torch.from_numpy(st).to(DEV), m, "mass").cpu().numpy()
     assert np.array_equal(ids, oracle.select_retained(st, m, "mass"))
+
+
+@pytest.mark.parametrize("m", [1, 7, 32])
+def test_selection_with_nan_scores(m):
+    # a NaN score is neither above nor below another: its expert is kept beside
+    # the m highest of the others, and the lowest m ids of those are written
+    st = np.zeros((32, 4))
+    st[:, 0], st[:, 1] = 1.0, (np.arange(32) * 7) % 32
+    nan = np.array([2, 19, 31])
+    st[nan, 1] = np.nan
+    ids = sw.slimwise_moe_select_retained(torch.from_numpy(st).to(DEV), m, "mass").cpu().numpy()
+    rest = np.setdiff1d(np.arange(32), nan)
+    best = rest[np.argsort(-st[rest, 1], kind="stable")[:m]]
+    assert np.array_equal(ids, np.sort(np.concatenate([best, nan]))[:m])
