@@ -219,7 +219,8 @@ struct Dims {
   int local;      // 1: no grouping kernel; the FFN and combine CTAs group the batch themselves
 };
 // Batches of at most kLocalTokens tokens are grouped inside the FFN and the
-// combine (expert_ffn.cu), from one bit mask of tokens per expert.
+// combine (expert_ffn.cu, which has the figures), from one bit mask of tokens
+// per expert, whatever the pool.
 constexpr int kLocalTokens = 96;
 // 32-token words of an expert's mask: 2 up to 64 tokens, else 4.
 __host__ __device__ inline int local_words(const Dims &d) {

@@ -281,7 +281,7 @@ __device__ __forceinline__ Item decode_item(int item, const ItemPlan &ip, const 
 
 // out[t, h] = sum_j g[t,j] y[pos(t,j), h] in j order (then the shared
 // expert's term) for the 128 h of one tile, by one warp: lane l covers
-// h = 4l..4l+3 with one 16-byte load per selection (a y tile row is 512
+// h = 4l..4l+3 with one 8-byte load per selection (a y tile row is 256
 // contiguous bytes), up to 8 loads in flight per lane; lanes j < k hold
 // selection j's grouped position and gate.
 template <bool kShared>
@@ -440,7 +440,7 @@ __device__ __forceinline__ void raise_abort(volatile int *abort, Ws &ws, int bit
 }
 
 // At most 128 registers a thread (320 threads: 40 K of the SM's 64 K), so
-// that a CTA of the dependent combine kernel (256 threads, 72 registers)
+// that a CTA of the dependent combine kernel (256 threads, 40 registers)
 // can become resident beside this one.
 //
 // kPair: the grid is made of 2-CTA clusters.  A routed work item covers two
@@ -474,7 +474,10 @@ __device__ __forceinline__ void raise_abort(volatile int *abort, Ws &ws, int bit
 // 31.8 / 27.8, full pool B = 64 176.9 / 172.4, Qwen3.6-shaped layer with the
 // shared expert B = 32 120.8 / 114.4; 64 to 128 tokens, m' = 64: 64 99.4 /
 // 95.8, 96 100.2 / 98.1, 112 100.2 / 99.7, 128 100.1 / 101.4 (larger token
-// boxes take the ring's place and L2 reads; the line is drawn at 96).
+// boxes take the ring's place and L2 reads; the line is drawn at 96).  The scan
+// of the pool in every CTA does not move it: pools of 512 and 1024 experts at
+// H = 512-8192 took 0.72-0.99 of the time with the grouping kernel at 1-96
+// tokens.
 template <bool kShared, bool kWide, bool kPair, bool kAhead, int kLocalWords>
 __global__ void __maxnreg__(128)
     expert_ffn_kernel(const __grid_constant__ FfnMaps maps,
@@ -1263,8 +1266,10 @@ cudaError_t launch_expert_ffn(const FfnMaps &maps, const __nv_bfloat16 *hidden,
   // of 16 in [16, 256]
   if (d.tok_chunk < kTokBox || d.tok_chunk > kMaxTokTile || d.tok_chunk % kTokBox != 0)
     return cudaErrorInvalidValue;
-  // the dependent combine kernel needs no shared memory: every byte the
-  // block may opt into goes to pipeline stages
+  // every byte the block may opt into goes to pipeline stages, whether or not
+  // that leaves room for a CTA of the dependent combine kernel (whose shared
+  // memory is the local grouping's): a stage less for its sake cost 0.4-1.4 us
+  // at 65-80 tokens (Qwen-class, m' = 64 and 128)
   const int stages = ffn_stages_for(d, (size_t)optin);
   const size_t smem =
       ffn_smem_plan(d.tok_chunk, stages, d.wide, d.pair, d.E, local_words(d)).total + 1024;

@@ -27,11 +27,13 @@ namespace slimwise {
 // Layers of at most 96 tokens do without this kernel (expert_ffn.cu), except
 // for statistics, pair items and routing-only calls.
 //
-// Tokens per CTA: one up to 64 tokens, two above.  Fewer tokens per CTA
-// spread the grouped-row copy over more SMs (one against two: up to 1.1 us a
-// step faster at B = 8-64), but every CTA recounts the whole batch's
-// selections, and above 64 tokens the extra CTAs cost more (B = 256: 0.9 us,
-// B = 512: 2 us slower); four per CTA was slower at every size.
+// Tokens per CTA: one up to 64 tokens (only the calls above come here with so
+// few), two above.  Fewer tokens per CTA spread the grouped-row copy over more
+// SMs (one against two at 4-64 tokens: 0.1-0.2 us of a routing-only call,
+// 0.2-0.7 us of a calibration batch or a layer of pair items), but every CTA
+// recounts the whole batch's selections, and above 64 tokens the extra CTAs
+// cost more (B = 256: 0.9 us, B = 512: 2 us a step); four per CTA was slower at
+// every size.
 inline int group_tokens_per_cta(int B) { return B <= 64 ? 1 : 2; }
 constexpr int kGroupThreads = 512;
 // Batches from here on take the tiled kernels below (whole layers, one kernel
@@ -509,7 +511,8 @@ cudaError_t launch_group_gather(const __nv_bfloat16 *hidden, const float *w_shar
 
 // The results a routing-only call hands out, copied by one launch: eight
 // device-to-device copies of a few KB took longer than the routing itself
-// (B = 300, m' = 96: 70.5 us a call, now 47, most of it host time).
+// (B = 300, m' = 96: 70.5 us a call, 47 with one launch, and 37-40 since the
+// binding's calls take raw handles; most of it is host time).
 __global__ void __launch_bounds__(256) export_kernel(ExportList x) {
   pdl_wait_primary();
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gstride = gridDim.x * blockDim.x;

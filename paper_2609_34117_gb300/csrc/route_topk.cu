@@ -526,8 +526,8 @@ size_t route_smem_bytes(const Dims &d) {
          (size_t)((TB + kClusterCtas - 1) / kClusterCtas) * d.m_ret * 4 + (size_t)d.m_ret * 4;
 }
 
-// What a routing CTA may take, of the opt-in limit: the rest is for its static
-// shared memory (report_retained's, 132 bytes).
+// What a routing CTA leaves of the opt-in limit for its static shared memory
+// (report_retained's, 144 bytes).
 constexpr size_t kRouteStaticSmem = 1024;
 
 template <int TB, int NC>
@@ -1274,6 +1274,10 @@ __global__ void __launch_bounds__(kRouteThreads, NC == 4 ? 4 : 3)
 //   m' = 192   B = 4096 436.4 / 410.9
 //   m' = 256   B =  768 303.3 / 306.2    1024 317.7 / 312.6   1536 358.1 / 347.7
 //              2048 389.7 / 363.2   4096 517.5 / 464.6   8192 825.2 / 715.2
+// Routing and grouping alone, at the smallest batch of the rule, half as many
+// again, twice that batch and 8192, H = 512-8192, m' = 128-256, k = 1-16: 0.28
+// to 0.99 of the full product's time, but for H = 8192 at the smallest batch
+// with m' = 16 k (113.2 / 116.8, 116.4 / 121.2).
 inline bool filtered_fits(const Dims &d, int parts) {
   return (size_t)parts * (d.B + 1) * d.m_ret * 4 <= (size_t)d.B * d.k * d.H * 2;
 }
